@@ -182,7 +182,10 @@ typedef struct {
     uint32_t head_streams;       /* 0 (default) or 1: in a plan of explicit pairs that is not
                                     filtered, the parts of items split by sets read head
                                     streams written by a pass before the simulator;
-                                    0xFFFFFFFF: every part gathers its heads itself */
+                                    0xFFFFFFFF: every part gathers its heads itself.
+                                    2 or 0xFFFFFFFF: every item runs in the simulator's
+                                    units, uniform chains among them (see
+                                    pchase_sim_plan_create) */
 } pchase_tune;
 
 typedef struct pchase_sim_plan pchase_sim_plan;
@@ -209,7 +212,15 @@ typedef struct pchase_sim_plan pchase_sim_plan;
  * (at most 16 GB in all; pchase_sim_plan_workspace_bytes counts it) and
  * reusing it from unit to unit.  Analytic chains (idx == NULL) whose visited
  * lines are every lstep-th line key a whole unit's state by line / lstep, so
- * their line tables cover the chain's lines, not the array's.  Errors: EINVAL
+ * their line tables cover the chain's lines, not the array's.
+ * Items whose stride divides their array (n_elems a multiple of stride, and
+ * the stride at most a line or a multiple of one) over equal sets are uniform
+ * chains: pchase_sim_run, and pchase_match_run without a bound, replay them
+ * outside the units once their trace has proved to be (t * stride) mod n_elems
+ * at every access: analytic chains are, index arrays are compared on every
+ * run, and one that differs anywhere goes to the units.  The results are the
+ * same.  Filtered plans, profiled runs and bounded matches use the units
+ * alone.  Errors: EINVAL
  * for a bad geometry, pair or trace; ERANGE for a geometry of more than 2^24
  * lines.
  */

@@ -137,11 +137,24 @@ constexpr uint64_t kPoolMaxWarps = 608;
 constexpr uint32_t kPoolWarpsPerCta = 4;
 constexpr uint64_t kPoolMaxBytes = 16ull << 30;
 
+// Shared memory of the played sets' tasks, one launch per class: 32 small sets
+// (5 KB) or the tables of one larger set (6 B per way, 4 B per line); a fixed
+// size per launch, so the classes keep a set of thousands of ways from taking
+// the occupancy of the small ones.
+constexpr int kUniformClasses = 4;
+constexpr uint32_t kUniformCaps[kUniformClasses] = {8192, 24576, 73728, 196608};
+// ns of a small set's miss (with its group's victims hashed ahead, or hashing
+// each itself) and of a window of a larger set; a task takes sets up to
+// kUniformTaskNs of work.
+constexpr double kUniformMissNs = 30.0, kUniformHashMissNs = 50.0, kUniformWindowNs = 230.0;
+constexpr double kUniformTaskNs = 30.0e3;
+
 // The tuning knobs as the planner reads them, and whether the plan's split
 // parts read head streams (plans of explicit pairs that are not a lower level
 // of a hierarchy; the matcher and filtered runs gather instead).
 struct PlanTune : pchase_tune {
     bool streams = false;
+    bool uniform = true;  // uniform chains outside the units (uniform.cu)
 };
 
 // What the planner assumes about an item's access stream, from its trace's
@@ -550,15 +563,31 @@ struct pchase_sim_plan {
     uint32_t n_slots = 0, n_census = 0;
     size_t off_jobs = 0, off_segjob = 0, off_itemslot = 0, off_cnt = 0, off_parts = 0,
            off_ents = 0, off_tgt = 0;
+    // uniform chains (uniform.cu): items that may be done there, whether every
+    // item may be, and for certain (analytic chains, nothing left for the
+    // units), the tasks of the played sets by shared-memory class, and per trace a unit
+    // that reads its index array (or ~0: nothing to check)
+    bool uniform = false, uniform_every = false, uniform_all = false;
+    uint64_t n_uniform = 0, n_explicit = 0;
+    std::vector<UniformTask> utasks;
+    uint32_t uclass[kUniformClasses] = {};
+    std::vector<uint32_t> trace_unit;
+    size_t off_bad = 0, off_utasks = 0, off_tunit = 0;
     double gwork_main[kUnitGroups] = {};  // estimated work of each unit group in the
                                           // slot-mix launch
     bool affinity = false;
-    cudaStream_t side = nullptr, side2 = nullptr;
+    cudaStream_t side = nullptr, side2 = nullptr, uside = nullptr, uside2 = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr, fork2 = nullptr, join2 = nullptr;
+    cudaEvent_t ufork = nullptr, ujoin = nullptr, ujoin2 = nullptr;
 
     ~pchase_sim_plan() {
         if (side) cudaStreamDestroy(side);
         if (side2) cudaStreamDestroy(side2);
+        if (uside) cudaStreamDestroy(uside);
+        if (uside2) cudaStreamDestroy(uside2);
+        if (ufork) cudaEventDestroy(ufork);
+        if (ujoin) cudaEventDestroy(ujoin);
+        if (ujoin2) cudaEventDestroy(ujoin2);
         if (fork) cudaEventDestroy(fork);
         if (join) cudaEventDestroy(join);
         if (fork2) cudaEventDestroy(fork2);
@@ -567,6 +596,126 @@ struct pchase_sim_plan {
 };
 
 namespace {
+
+// ---------------------------------------------------------- uniform chains
+// The host's view of an item's chain (uniform.cu's Chain).
+struct HostChain {
+    uint32_t per, nl, st, Tp, n_max, over;  // over: overflowing classes (mapping 0)
+    bool ok = false;                        // stride divides the array, lines regular
+
+    HostChain(const SimItem &it, uint32_t T) {
+        const uint32_t s = it.stride, lb = it.lsh & 255u;
+        if (it.n_elems > (1u << 31) || (it.lsh >> 16) & 1u) return;
+        if (s && it.n_elems % s) return;
+        per = s ? it.n_elems / s : 1u;
+        const bool strided = s > (1u << lb);
+        if (strided && s % (1u << lb)) return;
+        if (((it.lsh >> 8) & 255u) && strided) return;
+        nl = strided ? per : (((per - 1u) * s) >> lb) + 1u;
+        st = strided ? s >> lb : 1u;
+        Tp = T / (uint32_t)gcd64(st, T);
+        n_max = (nl - 1u) / Tp + 1u;
+        const uint64_t room = (uint64_t)it.ways * Tp;
+        over = nl > room ? (uint32_t)std::min<uint64_t>(Tp, nl - room) : 0u;
+        ok = true;
+    }
+};
+
+// shared memory of one larger set's tables (play_window's arena)
+uint64_t uniform_window_bytes(uint32_t n, uint32_t ways) {
+    return align16(6ull * ways + 4ull * n + kUniformRingBytes);
+}
+
+// The lsh bits of an item that may be done as a uniform chain (0: it may not).
+uint32_t uniform_bits(const pchase_geom &G, const SimItem &it) {
+    const HostChain c(it, G.sets);
+    if (!c.ok || it.len == 0) return 0;
+    const uint32_t both = (1u << kUniformBit) | (1u << kUniformMatchBit);
+    if (G.policy < PCHASE_RANDOM || G.ways == 1) return both;
+    if (map_shift(G)) {
+        // sets of 2^m consecutive lines: nothing is played here, so no set
+        // may overflow
+        const uint32_t m = map_shift(G), blk = 1u << m;
+        const uint64_t most = (((uint64_t)(c.nl >> m) + G.sets - 1) / G.sets) * blk +
+                              (c.nl & (blk - 1u));
+        return most <= G.ways ? both : 0u;
+    }
+    if (!c.over) return both;
+    if (it.len > kUniformPlayLen || c.n_max > 65534u ||
+        (c.n_max > 32 && uniform_window_bytes(c.n_max, G.ways) > kUniformCaps[kUniformClasses - 1]))
+        return 0;
+    return it.len <= kUniformMatchLen ? both : 1u << kUniformBit;
+}
+
+// Tasks of the played sets, and the traces to check.
+void plan_uniform(pchase_sim_plan *p) {
+    struct Costed {
+        UniformTask t;
+        int cls;
+        double cost;
+    };
+    std::vector<Costed> all;
+    p->trace_unit.assign(p->n_trace, 0xFFFFFFFFu);
+    p->uniform_all = p->uniform_every = true;
+    for (size_t k = 0; k < p->items.size(); ++k) {
+        const SimItem &it = p->items[k];
+        if (!it.lead) continue;
+        if (!((it.lsh >> kUniformBit) & 1u)) {
+            p->uniform_all = p->uniform_every = false;
+            continue;
+        }
+        p->n_uniform += 1;
+        if (it.idx) {
+            p->uniform_all = false;
+            if (p->trace_unit[it.obs] == 0xFFFFFFFFu) {
+                p->trace_unit[it.obs] = (uint32_t)k;
+                p->n_explicit += 1;
+            }
+        }
+        if (it.policy < PCHASE_RANDOM || it.ways == 1) continue;
+        const HostChain c(it, p->geoms[it.cand].sets);
+        if (!c.over || ((it.lsh >> 8) & 255u) || it.len <= c.per) continue;
+        // misses of one set: the share of its accesses that a random victim
+        // leaves missing is near 1 - (a / n)^2
+        const double passes = (double)(it.len - c.per) / c.per + 1.0;
+        const double n = c.n_max, r = it.ways / n, misses = passes * n * (1.0 - r * r);
+        uint32_t lanes = 0;
+        double set_ns = passes * std::max(1.0, n / 32.0) * kUniformWindowNs;
+        if (c.n_max <= 32) {
+            lanes = 32;
+            while (lanes > 1 && 32u / lanes < c.over) lanes /= 2;
+            const double ns = misses * (lanes > 1 ? kUniformMissNs : kUniformHashMissNs);
+            // few sets of a few dozen lines that mostly miss: a window of them
+            // at a time beats miss by miss (1.5: windows take a warp per set)
+            if (c.over <= 8 && ns > 1.5 * set_ns) lanes = 0;
+            else set_ns = ns;
+        }
+        const uint32_t step = lanes ? 32u / lanes : 1u;
+        const uint32_t steps = (uint32_t)std::max(1.0, std::min(1e6, kUniformTaskNs / set_ns));
+        const uint32_t bytes = lanes ? kUniformSmallBytes : (uint32_t)uniform_window_bytes(c.n_max, it.ways);
+        int cls = 0;
+        while (kUniformCaps[cls] < bytes) ++cls;
+        for (uint64_t first = 0; first < c.over; first += (uint64_t)step * steps) {
+            const uint32_t count = (uint32_t)std::min<uint64_t>((uint64_t)step * steps, c.over - first);
+            all.push_back({{(uint32_t)k, (uint32_t)first, count, lanes}, cls,
+                           set_ns * ((count + step - 1) / step)});
+        }
+    }
+    if (!p->n_uniform) {
+        p->uniform_all = p->uniform_every = false;
+        p->trace_unit.clear();
+        return;
+    }
+    p->uniform = true;
+    std::stable_sort(all.begin(), all.end(), [](const Costed &x, const Costed &y) {
+        return x.cls != y.cls ? x.cls < y.cls : x.cost > y.cost;
+    });
+    p->utasks.reserve(all.size());
+    for (const Costed &c : all) {
+        p->utasks.push_back(c.t);
+        p->uclass[c.cls] += 1;
+    }
+}
 
 // Unit-group homes of the slot-mix launch: `sites` SMs (CTA b sits on site
 // b mod sites) shared among the groups with work in proportion to their
@@ -625,6 +774,8 @@ int plan_runtime(pchase_sim_plan *p) {
         if (dev != p->device) return fail(PCHASE_EINVAL, "plan used on another device");
         return PCHASE_OK;
     }
+    PCHASE_CUDA(prepare_sim(kMaxArena), "cudaFuncSetAttribute");
+    PCHASE_CUDA(prepare_uniform(kUniformCaps[kUniformClasses - 1]), "cudaFuncSetAttribute");
     p->sms = sm_count();
     if (p->sms <= 0) return fail(PCHASE_ECUDA, "no CUDA device");
     // A CTA of either launch fills an SM's shared memory, so a main launch
@@ -659,6 +810,20 @@ int plan_runtime(pchase_sim_plan *p) {
         PCHASE_CUDA(cudaEventCreateWithFlags(&p->fork2, cudaEventDisableTiming), "cudaEventCreate");
         PCHASE_CUDA(cudaEventCreateWithFlags(&p->join2, cudaEventDisableTiming), "cudaEventCreate");
     }
+    // played sets run beside the simulator's units, the large ones beside the
+    // small ones (where every item may be a uniform chain the units mostly have
+    // nothing to do, and one stream less is needed)
+    const bool large = p->utasks.size() > p->uclass[0];
+    if (!p->utasks.empty() && (large || !p->uniform_every))
+        PCHASE_CUDA(cudaEventCreateWithFlags(&p->ufork, cudaEventDisableTiming), "cudaEventCreate");
+    if (p->uclass[0] && !p->uniform_every) {
+        PCHASE_CUDA(cudaStreamCreateWithFlags(&p->uside, cudaStreamNonBlocking), "cudaStreamCreate");
+        PCHASE_CUDA(cudaEventCreateWithFlags(&p->ujoin, cudaEventDisableTiming), "cudaEventCreate");
+    }
+    if (large) {
+        PCHASE_CUDA(cudaStreamCreateWithFlags(&p->uside2, cudaStreamNonBlocking), "cudaStreamCreate");
+        PCHASE_CUDA(cudaEventCreateWithFlags(&p->ujoin2, cudaEventDisableTiming), "cudaEventCreate");
+    }
     p->device = dev;
     return PCHASE_OK;
 }
@@ -667,14 +832,52 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
     int rc = plan_runtime(p);
     if (rc) return rc;
     uint8_t *w = static_cast<uint8_t *>(ws);
-    PCHASE_CUDA(cudaMemsetAsync(w, 0, kQueueHeader, st), "cudaMemsetAsync(queues)");
     SimOut o = out;
+    // uniform chains, unless the run filters accesses, records a timeline of
+    // the units, or may stop its candidates early
+    const bool uni = p->uniform && !o.filter && !o.timeline && (!o.dist || o.stop_above == ~0ull);
+    PCHASE_CUDA(cudaMemsetAsync(w, 0, kQueueHeader + (uni ? 4ull * p->n_trace : 0), st),
+                "cudaMemsetAsync(queues)");
     if (!o.status) o.status = reinterpret_cast<uint32_t *>(w + kStatusOffset);
     o.gstate = w + p->off_gstate;
     const SimItem *items = reinterpret_cast<const SimItem *>(w + p->off_items);
     uint32_t *queues = reinterpret_cast<uint32_t *>(w);
-    PCHASE_CUDA(launch_sim_zero(items, p->n_units, p->sms, o, st), "output clear");
-    if (!p->jobs.empty() && !o.dist && !o.filter) {
+    const bool units = !(uni && p->uniform_all && !o.dist);  // the units have work, or may have
+    if (uni) {
+        uint32_t *const bad = reinterpret_cast<uint32_t *>(w + p->off_bad);
+        o.uniform_bad = bad;
+        o.uniform_live = reinterpret_cast<uint32_t *>(w + kLiveOffset);
+        PCHASE_CUDA(launch_uniform_prep(items, reinterpret_cast<const uint32_t *>(w + p->off_tunit),
+                                        p->n_trace, p->n_explicit, p->n_items, o.miss_counts, bad,
+                                        p->sms, st),
+                    "uniform check");
+        PCHASE_CUDA(launch_uniform_out(items, p->n_units, p->sms, o,
+                                       reinterpret_cast<uint32_t *>(w + kLiveOffset), st),
+                    "uniform words");
+        const UniformTask *const tasks = reinterpret_cast<const UniformTask *>(w + p->off_utasks);
+        if (p->ufork) PCHASE_CUDA(cudaEventRecord(p->ufork, st), "cudaEventRecord");
+        if (p->uside2) {
+            PCHASE_CUDA(cudaStreamWaitEvent(p->uside2, p->ufork, 0), "cudaStreamWaitEvent");
+            uint32_t first = (uint32_t)p->utasks.size();
+            for (int c = kUniformClasses - 1; c > 0; --c) {
+                first -= p->uclass[c];
+                PCHASE_CUDA(launch_uniform_play(items, tasks + first, p->uclass[c], kUniformCaps[c], o,
+                                                p->uside2),
+                            "uniform sets");
+            }
+            PCHASE_CUDA(cudaEventRecord(p->ujoin2, p->uside2), "cudaEventRecord");
+        }
+        if (p->uclass[0]) {
+            cudaStream_t us = p->uside ? p->uside : st;
+            if (p->uside) PCHASE_CUDA(cudaStreamWaitEvent(us, p->ufork, 0), "cudaStreamWaitEvent");
+            PCHASE_CUDA(launch_uniform_play(items, tasks, p->uclass[0], kUniformCaps[0], o, us),
+                        "uniform sets");
+            if (p->uside) PCHASE_CUDA(cudaEventRecord(p->ujoin, us), "cudaEventRecord");
+        }
+    } else {
+        PCHASE_CUDA(launch_sim_zero(items, p->n_units, p->sms, o, st), "output clear");
+    }
+    if (units && !p->jobs.empty() && !o.dist && !o.filter) {
         // the split parts' head streams, before any launch that reads them
         o.item_slot = reinterpret_cast<const uint32_t *>(w + p->off_itemslot);
         o.parts = reinterpret_cast<const PartInfo *>(w + p->off_parts);
@@ -691,10 +894,11 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
                                    reinterpret_cast<uint32_t *>(w + p->off_cnt),
                                    reinterpret_cast<PartInfo *>(w + p->off_parts),
                                    reinterpret_cast<uint2 *>(w + p->off_ents),
-                                   reinterpret_cast<uint32_t *>(w + p->off_tgt), o.status, st),
+                                   reinterpret_cast<uint32_t *>(w + p->off_tgt), o.status,
+                                   o.uniform_bad, st),
                     "head streams");
     }
-    if (p->gpool.nwarps) {
+    if (units && p->gpool.nwarps) {
         // units with global set state first (the longest of a hierarchy's
         // large levels), on a side stream of their own joined back below
         PCHASE_CUDA(cudaEventRecord(p->fork2, st), "cudaEventRecord");
@@ -702,17 +906,21 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
         PCHASE_CUDA(launch_sim(items, p->gpool, queues, p->ggrid, o, p->side2), "pool launch");
         PCHASE_CUDA(cudaEventRecord(p->join2, p->side2), "cudaEventRecord");
     }
-    if (p->jumbo.nwarps) {
-        // jumbo items first, on a side stream joined back before returning
+    // jumbo items first, on a side stream joined back before returning
+    const bool jside = units && p->jumbo.nwarps;
+    if (jside) {
         PCHASE_CUDA(cudaEventRecord(p->fork, st), "cudaEventRecord");
         PCHASE_CUDA(cudaStreamWaitEvent(p->side, p->fork, 0), "cudaStreamWaitEvent");
         PCHASE_CUDA(launch_sim(items, p->jumbo, queues, p->jgrid, o, p->side), "jumbo launch");
         PCHASE_CUDA(cudaEventRecord(p->join, p->side), "cudaEventRecord");
     }
-    if (p->layout.nwarps)
+    if (units && p->layout.nwarps)
         PCHASE_CUDA(launch_sim(items, p->layout, queues, p->grid, o, st), "simulator launch");
-    if (p->jumbo.nwarps) PCHASE_CUDA(cudaStreamWaitEvent(st, p->join, 0), "cudaStreamWaitEvent");
-    if (p->gpool.nwarps) PCHASE_CUDA(cudaStreamWaitEvent(st, p->join2, 0), "cudaStreamWaitEvent");
+    if (jside) PCHASE_CUDA(cudaStreamWaitEvent(st, p->join, 0), "cudaStreamWaitEvent");
+    if (units && p->gpool.nwarps)
+        PCHASE_CUDA(cudaStreamWaitEvent(st, p->join2, 0), "cudaStreamWaitEvent");
+    if (uni && p->uside) PCHASE_CUDA(cudaStreamWaitEvent(st, p->ujoin, 0), "cudaStreamWaitEvent");
+    if (uni && p->uside2) PCHASE_CUDA(cudaStreamWaitEvent(st, p->ujoin2, 0), "cudaStreamWaitEvent");
     return PCHASE_OK;
 }
 
@@ -781,7 +989,9 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
         if (tune->big_slots) tn.big_slots = std::min<uint32_t>(tune->big_slots, 4);
         tn.kind_affinity = tune->kind_affinity == 0xFFFFFFFFu ? 0u : 1u;
         tn.head_streams = tune->head_streams == 0xFFFFFFFFu ? 0u : 1u;
+        tn.uniform = tune->head_streams <= 1u;
     }
+    if (tn.filtered) tn.uniform = false;
     tn.streams = pairs != nullptr && !tn.filtered && tn.head_streams;
     for (uint32_t i = 0; i < n_geom; ++i) {
         int rc = check_geom(geoms[i], i);
@@ -877,6 +1087,7 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
         it.gs2 = (uint8_t)gdm.s2;
         it.lead = 1;
         it.kcnt = 1;
+        if (tn.uniform) it.lsh |= uniform_bits(G, it);
         ItemShape &sh = shape[i];
         item_shape(G, Tr, sh);
         UnitShape u;
@@ -1177,6 +1388,12 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
     for (uint64_t k = 0; k < n_units; ++k) p->items.push_back(items[order[k]]);
     // the pool's units after every size class, costliest first
     for (const SimItem &it : gitems) p->items.push_back(it);
+    try {
+        if (tn.uniform) plan_uniform(p);
+    } catch (...) {
+        delete p;
+        return fail(PCHASE_ENOMEM, "uniform task allocation");
+    }
     // head streams: one job per caller item whose parts read them, its K
     // streams side by side in an entry area as long as its trace
     try {
@@ -1402,6 +1619,8 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
     // workspace: [queues + status: kQueueHeader][items][geoms][seg offsets][obs word
     // offsets][pool]
     size_t off = kQueueHeader;
+    p->off_bad = off;  // right behind the header: cleared with it
+    if (p->uniform) off = align256(off + (size_t)n_trace * sizeof(uint32_t));
     p->off_items = off;
     off = align256(off + p->n_units * sizeof(SimItem));  // size classes and pool
     p->off_geoms = off;
@@ -1428,6 +1647,10 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
     off = align256(off + p->n_ents * sizeof(uint2));
     p->off_tgt = off;
     off = align256(off + p->n_tgt * sizeof(uint32_t));
+    p->off_utasks = off;
+    off = align256(off + p->utasks.size() * sizeof(UniformTask));
+    p->off_tunit = off;
+    off = align256(off + p->trace_unit.size() * sizeof(uint32_t));
     p->ws_bytes = off;
     *plan_out = p;
     return PCHASE_OK;
@@ -1440,6 +1663,7 @@ size_t pchase_sim_plan_upload_bytes(const pchase_sim_plan *plan) {
     return plan->items.size() * sizeof(SimItem) + plan->geoms.size() * sizeof(pchase_geom) +
            plan->seg_offsets.size() * sizeof(uint64_t) +
            plan->obs_word_offsets.size() * sizeof(uint64_t) + 2 * sizeof(uint64_t) +
+           plan->utasks.size() * sizeof(UniformTask) + plan->trace_unit.size() * sizeof(uint32_t) +
            (plan->jobs.empty() ? 0
                                : plan->jobs.size() * sizeof(StreamJob) +
                                      plan->seg_job.size() * sizeof(uint32_t) +
@@ -1455,9 +1679,18 @@ uint64_t pchase_sim_plan_bitmap_words(const pchase_sim_plan *plan) {
 }
 uint32_t pchase_sim_plan_launches(const pchase_sim_plan *plan) {
     if (!plan) return 0;
-    // output clear + head streams (offsets; count and write when there are
-    // segments) + main slot-mix launch + side launch of jumbo units + pool
-    return (plan->n_units ? 1u : 0u) + (plan->jobs.empty() ? 0u : 1u) +
+    // output clear (with uniform chains: their check, the words, and a launch
+    // per shared-memory class of played sets) + head streams (offsets; count
+    // and write when there are segments) + main slot-mix launch + side launch
+    // of jumbo units + pool; a plan of analytic uniform chains alone launches
+    // nothing for its units
+    uint32_t n = plan->n_units ? 1u : 0u;
+    if (plan->uniform) {
+        n += 1u;
+        for (uint32_t c : plan->uclass) n += c ? 1u : 0u;
+        if (plan->uniform_all) return n;
+    }
+    return n + (plan->jobs.empty() ? 0u : 1u) +
            (plan->seg_job.empty() ? 0u : 2u) + (plan->layout.nwarps ? 1u : 0u) +
            (plan->jumbo.nwarps ? 1u : 0u) + (plan->gpool.nwarps ? 1u : 0u);
 }
@@ -1556,6 +1789,12 @@ size_t pchase_sim_plan_describe(const pchase_sim_plan *plan, char *buf, size_t b
         }
         snprintf(tmp, sizeof tmp, " affinity=%d", plan->affinity ? 1 : 0);
         d += tmp;
+        if (plan->uniform) {
+            // items that may be done as uniform chains, tasks of played sets
+            snprintf(tmp, sizeof tmp, " uniform=%llu,%zu", (unsigned long long)plan->n_uniform,
+                     plan->utasks.size());
+            d += tmp;
+        }
         if (!plan->jobs.empty()) {
             // head streams: split items, their parts, entries (8 bytes each);
             // census: LRU items cut in time whose sets' lines are counted
@@ -1608,6 +1847,16 @@ int pchase_sim_plan_upload(const pchase_sim_plan *plan, void *workspace, size_t 
     const uint64_t pool[2] = {0, plan->total_len};
     PCHASE_CUDA(cudaMemcpyAsync(w + plan->off_pool, pool, sizeof pool, cudaMemcpyHostToDevice, st),
                 "upload pooled offsets");
+    if (!plan->utasks.empty())
+        PCHASE_CUDA(cudaMemcpyAsync(w + plan->off_utasks, plan->utasks.data(),
+                                    plan->utasks.size() * sizeof(UniformTask),
+                                    cudaMemcpyHostToDevice, st),
+                    "upload uniform tasks");
+    if (!plan->trace_unit.empty())
+        PCHASE_CUDA(cudaMemcpyAsync(w + plan->off_tunit, plan->trace_unit.data(),
+                                    plan->trace_unit.size() * sizeof(uint32_t),
+                                    cudaMemcpyHostToDevice, st),
+                    "upload uniform traces");
     if (!plan->jobs.empty()) {
         PCHASE_CUDA(cudaMemcpyAsync(w + plan->off_jobs, plan->jobs.data(),
                                     plan->jobs.size() * sizeof(StreamJob), cudaMemcpyHostToDevice, st),

@@ -102,6 +102,7 @@ struct SimItem {
                           // bit 16: unequal sets (gsets/gmagic: M = T*a + extra, kmagic: a,
                           // ways: a + extra, the ways of set 0); bit 17: way scans with the
                           // set state in global memory at 16 * kres bytes (whole units);
+                          // bits 19, 20: kUniformBit, kUniformMatchBit (every unit of the item);
                           // bit 18: compact lines (whole units of analytic chains whose
                           // visited lines are the multiples of gsets: the unit keys its
                           // state by line / gsets, gmagic/gs1/gs2 its DivMagic, and takes
@@ -163,6 +164,7 @@ constexpr int kUnitGroups = 9;
 constexpr uint32_t kQueueStride = 32;  // queue counter of (group g, class c): g * 32 + c
 constexpr size_t kQueueHeader = 2048;  // workspace head: the queue counters, then the status word
 constexpr size_t kStatusOffset = 1536;
+constexpr size_t kLiveOffset = 1600;  // SimOut::uniform_live
 __host__ __device__ __forceinline__ uint32_t unit_group(uint32_t mode, uint32_t policy) {
     return mode * 3u + (policy < 2u ? policy : 2u);
 }
@@ -222,6 +224,29 @@ struct SimOut {
     // per set: min(a, the set's distinct lines over the whole trace), the
     // lines a time part's read-back needs before the set is complete
     const uint32_t *targets;
+    // items done as uniform chains (uniform.cu): a word per trace, 0 where the
+    // trace is the chain its descriptor states (NULL: no such run), and the
+    // word that is 0 when every item of the run was done there
+    const uint32_t *uniform_bad;
+    const uint32_t *uniform_live;
+};
+
+// Uniform chains (uniform.cu).  An item with kUniformBit is replayed there
+// when its trace proves uniform, in matcher runs only if it has
+// kUniformMatchBit too; its units then return at once.  A task plays the
+// overflowing sets of classes [first, first + count) of a RANDOM or WEIGHTED
+// item: `lanes` lanes to a set, 32 / lanes sets at a time, or (lanes 0) the
+// whole warp one set after the other.
+constexpr uint32_t kUniformBit = 19, kUniformMatchBit = 20;
+constexpr uint32_t kUniformMatchLen = 1u << 15;  // accesses a played item may have in the matcher
+constexpr uint32_t kUniformPlayLen = 1u << 26;   // and in any run (times stay below 2^32)
+constexpr uint32_t kUniformSmallBytes = 1024 + 32 * 32 * 4;  // shared memory of 32 small sets
+constexpr uint32_t kUniformRingBytes = 256 * 6;  // rings of hashed evictions of one larger set
+struct UniformTask {
+    uint32_t unit;
+    uint32_t first;
+    uint32_t count;
+    uint32_t lanes;
 };
 
 // Head streams (streams.cu).  Every item split by sets into K parts is one
@@ -265,10 +290,23 @@ cudaError_t launch_sim(const SimItem *items, const SlotLayout &layout, uint32_t 
 cudaError_t launch_sim_zero(const SimItem *items, uint64_t n_units, int sms, const SimOut &out,
                             cudaStream_t st);
 int sim_max_ctas_per_sm(const SlotLayout &layout);
+// Shared memory the simulator's (the played sets') launches may ask for, on the
+// current device: once per plan, with the same constants from every plan.
+cudaError_t prepare_sim(uint32_t smem_bytes);
+cudaError_t prepare_uniform(uint32_t smem_bytes);
+// Uniform chains: traces checked and counts cleared, the words of every item,
+// the tasks of one shared-memory class.
+cudaError_t launch_uniform_prep(const SimItem *items, const uint32_t *trace_unit, uint32_t n_trace,
+                                uint64_t n_explicit, uint64_t n_items, uint64_t *counts,
+                                uint32_t *bad, int sms, cudaStream_t st);
+cudaError_t launch_uniform_out(const SimItem *items, uint64_t n_units, int sms, const SimOut &out,
+                               uint32_t *live, cudaStream_t st);
+cudaError_t launch_uniform_play(const SimItem *items, const UniformTask *tasks, uint32_t n_tasks,
+                                uint32_t smem_bytes, const SimOut &out, cudaStream_t st);
 // The head streams of a plan's split items (three launches on `st`).
 cudaError_t launch_streams(const SimItem *items, const StreamJob *jobs, uint32_t n_jobs,
                            const uint32_t *seg_job, uint32_t n_seg, uint32_t *cnt,
                            PartInfo *parts, uint2 *ents, uint32_t *targets, uint32_t *status,
-                           cudaStream_t st);
+                           const uint32_t *uniform_bad, cudaStream_t st);
 
 }  // namespace pchase

@@ -1671,6 +1671,10 @@ __device__ __forceinline__ void run_unit(const SimItem &it, uint32_t arena, cons
     const bool gmem = POOL;  // the planner puts every global-state unit in the pool
     uint8_t *const gst = gmem ? out.gstate + 16ull * it.kres : nullptr;
     const uint32_t kind = gmem ? (uint32_t)kGlobalScanLru + pol : (uint32_t)it.mode * 3u + pol;
+    // done as a uniform chain
+    if (out.uniform_bad && ((it.lsh >> kUniformBit) & 1u) &&
+        (!out.dist || ((it.lsh >> kUniformMatchBit) & 1u)) && out.uniform_bad[it.obs] == 0u)
+        return;
     // matcher: a candidate whose other units already exceed the bound is out
     if (out.dist && over_bound(out, it.cand, 0, lane)) return;
     clear_state<POOL>(kind, st, gst, it, lane);
@@ -1717,6 +1721,7 @@ __global__ void __launch_bounds__(512) sim_kernel(const SimItem *__restrict__ it
                                                   uint32_t *queues, SimOut out) {
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
+    if (out.uniform_live && *out.uniform_live == 0u) return;  // every item is done
     const uint32_t arena = L.warp_off[warp];
     const uint32_t top = L.warp_class[warp];
     // class this lane watches (pad + lane <= top), in every group
@@ -1858,9 +1863,6 @@ cudaError_t launch_sim(const SimItem *items, const SlotLayout &layout, uint32_t 
     // layout with spec set, the per-mode unit loops
     const auto k = layout.pool16 ? sim_kernel<true, false>
                                  : layout.spec ? sim_kernel<false, true> : sim_kernel<false, false>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)layout.smem_bytes);
-    if (e != cudaSuccess) return e;
     k<<<grid, layout.nwarps * 32, layout.smem_bytes, st>>>(items, layout, queues, out);
     return cudaGetLastError();
 }
@@ -1873,11 +1875,16 @@ cudaError_t launch_sim_zero(const SimItem *items, uint64_t n_units, int sms, con
     return cudaGetLastError();
 }
 
+cudaError_t prepare_sim(uint32_t smem_bytes) {
+    cudaError_t e = cudaSuccess;
+    for (const auto k : {sim_kernel<true, false>, sim_kernel<false, true>, sim_kernel<false, false>})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    return e;
+}
+
 int sim_max_ctas_per_sm(const SlotLayout &layout) {
     const auto k = layout.spec ? sim_kernel<false, true> : sim_kernel<false, false>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)layout.smem_bytes) != cudaSuccess)
-        return 0;
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, layout.nwarps * 32,
                                                       layout.smem_bytes) != cudaSuccess)

@@ -154,10 +154,15 @@ __device__ __forceinline__ void census_segment(const SimItem &it, const StreamJo
         if (sbm[k]) atomicOr(gbm + k, sbm[k]);
 }
 
+// an item done as a uniform chain needs no streams
+__device__ __forceinline__ bool done_uniform(const SimItem &it, const uint32_t *bad) {
+    return bad && ((it.lsh >> kUniformBit) & 1u) && bad[it.obs] == 0u;
+}
+
 __global__ void __launch_bounds__(kStreamWarps * 32)
     head_count_kernel(const SimItem *__restrict__ items, const StreamJob *__restrict__ jobs,
                       const uint32_t *__restrict__ seg_job, uint32_t n_seg, uint32_t *cnt,
-                      uint32_t *status) {
+                      uint32_t *status, const uint32_t *uniform_bad) {
     __shared__ uint32_t counts[kStreamWarps][32];
     __shared__ uint32_t census[kStreamWarps][kCensusMaxLines / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -165,6 +170,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32)
     if (g >= n_seg) return;
     const StreamJob J = jobs[seg_job[g]];
     const SimItem it = items[J.unit];
+    if (done_uniform(it, uniform_bad)) return;
     if (J.kind == kJobCensus) {
         census_segment(it, J, g - J.seg_first, lane, census[w], cnt + J.cnt_off);
         return;
@@ -184,12 +190,14 @@ __global__ void __launch_bounds__(kStreamWarps * 32)
 // part's stream and takes its total; the parts' streams follow one another.
 __global__ void __launch_bounds__(256)
     head_offsets_kernel(const SimItem *__restrict__ items, const StreamJob *__restrict__ jobs,
-                        uint32_t n_jobs, uint32_t *cnt, PartInfo *parts, uint32_t *targets) {
+                        uint32_t n_jobs, uint32_t *cnt, PartInfo *parts, uint32_t *targets,
+                        const uint32_t *uniform_bad) {
     __shared__ uint32_t per_set[8][kCensusMaxSets];
     const int lane = threadIdx.x & 31;
     const uint32_t j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (j >= n_jobs) return;
     const StreamJob J = jobs[j];
+    if (done_uniform(items[J.unit], uniform_bad)) return;
     if (J.kind == kJobCensus) {
         // each set's distinct lines, at most a of them
         const SimItem it = items[J.unit];
@@ -243,7 +251,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32)
     head_write_kernel(const SimItem *__restrict__ items, const StreamJob *__restrict__ jobs,
                       const uint32_t *__restrict__ seg_job, uint32_t n_seg,
                       const uint32_t *__restrict__ cnt, const PartInfo *__restrict__ parts,
-                      uint2 *ents, uint32_t *status) {
+                      uint2 *ents, uint32_t *status, const uint32_t *uniform_bad) {
     __shared__ uint64_t cursor[kStreamWarps][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t g = blockIdx.x * kStreamWarps + (uint32_t)w;
@@ -251,6 +259,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32)
     const StreamJob J = jobs[seg_job[g]];
     if (J.kind == kJobCensus) return;
     const SimItem it = items[J.unit];
+    if (done_uniform(it, uniform_bad)) return;
     uint64_t *const cur = cursor[w];
     if ((uint32_t)lane < J.K)
         cur[lane] = parts[J.slot_first + lane].start +
@@ -271,17 +280,18 @@ __global__ void __launch_bounds__(kStreamWarps * 32)
 cudaError_t launch_streams(const SimItem *items, const StreamJob *jobs, uint32_t n_jobs,
                            const uint32_t *seg_job, uint32_t n_seg, uint32_t *cnt,
                            PartInfo *parts, uint2 *ents, uint32_t *targets, uint32_t *status,
-                           cudaStream_t st) {
+                           const uint32_t *uniform_bad, cudaStream_t st) {
     if (!n_jobs) return cudaSuccess;
     // (items with empty traces still get their parts' {start, 0})
     const unsigned blocks = (n_seg + kStreamWarps - 1) / kStreamWarps;
     if (n_seg)
         head_count_kernel<<<blocks, kStreamWarps * 32, 0, st>>>(items, jobs, seg_job, n_seg, cnt,
-                                                                status);
-    head_offsets_kernel<<<(n_jobs + 7) / 8, 256, 0, st>>>(items, jobs, n_jobs, cnt, parts, targets);
+                                                                status, uniform_bad);
+    head_offsets_kernel<<<(n_jobs + 7) / 8, 256, 0, st>>>(items, jobs, n_jobs, cnt, parts, targets,
+                                                          uniform_bad);
     if (n_seg)
         head_write_kernel<<<blocks, kStreamWarps * 32, 0, st>>>(items, jobs, seg_job, n_seg, cnt,
-                                                                parts, ents, status);
+                                                                parts, ents, status, uniform_bad);
     return cudaGetLastError();
 }
 
