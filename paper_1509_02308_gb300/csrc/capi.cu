@@ -526,6 +526,8 @@ int pchase::set_last_error(int code, const char *msg) { return fail(code, msg); 
 struct pchase_sim_plan {
     std::vector<SimItem> items;
     SlotLayout layout{};
+    SlotLayout ulayout{};  // layout with the homes of a run whose analytic uniform
+                           // chains are not the units' work
     SlotLayout jumbo{};   // items too large for the main slot mix (nwarps 0: none)
     SlotLayout gpool{};   // units with global set state, one pool region per warp
     uint32_t pool_warps = 0;    // warps (and state regions) of the pool launch
@@ -573,6 +575,7 @@ struct pchase_sim_plan {
     uint32_t uclass[kUniformClasses] = {};
     std::vector<uint32_t> trace_unit;
     size_t off_bad = 0, off_utasks = 0, off_tunit = 0;
+    double gwork_live[kUnitGroups] = {};  // (ulayout's)
     double gwork_main[kUnitGroups] = {};  // estimated work of each unit group in the
                                           // slot-mix launch
     bool affinity = false;
@@ -791,8 +794,10 @@ int plan_runtime(pchase_sim_plan *p) {
         if (per <= 0) return fail(PCHASE_ECUDA, "simulator kernel cannot be resident");
         p->grid = (int)std::max<uint64_t>(
             1, std::min<uint64_t>((uint64_t)per * (p->sms - jsms), p->n_units - p->n_jumbo));
-        set_homes(p->layout, p->gwork_main, p->affinity,
-                  (uint32_t)std::max(1, std::min(p->grid, p->sms - jsms)));
+        const uint32_t sites = (uint32_t)std::max(1, std::min(p->grid, p->sms - jsms));
+        p->ulayout = p->layout;
+        set_homes(p->layout, p->gwork_main, p->affinity, sites);
+        set_homes(p->ulayout, p->gwork_live, p->affinity, sites);
     }
     if (p->jumbo.nwarps) {
         const int per = sim_max_ctas_per_sm(p->jumbo);
@@ -915,7 +920,8 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
         PCHASE_CUDA(cudaEventRecord(p->join, p->side), "cudaEventRecord");
     }
     if (units && p->layout.nwarps)
-        PCHASE_CUDA(launch_sim(items, p->layout, queues, p->grid, o, st), "simulator launch");
+        PCHASE_CUDA(launch_sim(items, uni ? p->ulayout : p->layout, queues, p->grid, o, st),
+                    "simulator launch");
     if (jside) PCHASE_CUDA(cudaStreamWaitEvent(st, p->join, 0), "cudaStreamWaitEvent");
     if (units && p->gpool.nwarps)
         PCHASE_CUDA(cudaStreamWaitEvent(st, p->join2, 0), "cudaStreamWaitEvent");
@@ -1462,8 +1468,9 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
     SlotLayout &L = p->layout;
     memset(&L, 0, sizeof L);
     std::vector<double> work(ncap, 0.0);
-    std::vector<double> gwork[kUnitGroups];
+    std::vector<double> gwork[kUnitGroups], glive[kUnitGroups];
     for (auto &v : gwork) v.assign(ncap, 0.0);
+    for (auto &v : glive) v.assign(ncap, 0.0);
     uint32_t nclass = 0;
     {
         // classes present, in increasing cap order, renumbered 0..nclass-1
@@ -1490,6 +1497,8 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
                         ++count;
                         work[q] += cost[order[k]];
                         gwork[g][q] += cost[order[k]];
+                        const SimItem &it = items[order[k]];
+                        if (it.idx || !((it.lsh >> kUniformBit) & 1u)) glive[g][q] += cost[order[k]];
                     }
                 L.cls_first[g][q] = (uint32_t)(count ? first : 0);
                 L.cls_count[g][q] = (uint32_t)count;
@@ -1573,7 +1582,10 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
         // 2000th of the longest unit's estimate below that
         L.stagger_ns = (uint32_t)std::min(4000.0, p->est_max_unit / 2000.0);
         for (int g = 0; g < kUnitGroups; ++g)
-            for (int q = 0; q <= main_top; ++q) p->gwork_main[g] += gwork[g][q];
+            for (int q = 0; q <= main_top; ++q) {
+                p->gwork_main[g] += gwork[g][q];
+                p->gwork_live[g] += glive[g][q];
+            }
         p->affinity = tn.kind_affinity != 0;
         // jumbo layout: one warp, the largest jumbo arena; serves jumbo classes
         SlotLayout &J = p->jumbo;

@@ -83,6 +83,43 @@ struct Chain {
         rnd = it.policy >= PCHASE_RANDOM && a > 1;
         sm = ss1 = ss2 = 0;
     }
+    // miss bits of accesses [t0, t0 + 32) (the played sets' only in the first
+    // pass); held: no set misses after the first pass, all: every one does
+    __device__ __forceinline__ uint32_t word(uint32_t t0, bool held, bool all) const {
+        if (nl == 1u) return t0 == 0u ? 1u : 0u;
+        uint32_t bits = 0, k = t0 % per;
+        if (strided) {
+            // every access is a head; x: its line's class
+            uint32_t x = k % Tp;
+#pragma unroll 8
+            for (uint32_t i = 0; i < 32; ++i) {
+                const bool miss = t0 + i < per || (!held && (all || x < thr));
+                bits |= (miss ? 1u : 0u) << i;
+                x = x + 1u == Tp ? 0u : x + 1u;
+                if (++k == per) k = x = 0;
+            }
+            return bits;
+        }
+        // heads from the first one at or after t0
+        uint32_t base = t0 - k, kk = k ? (((k - 1u) * s) >> lb) + 1u : 0u;
+        if (kk == nl) {
+            kk = 0;
+            base += per;
+        }
+        uint32_t x = m || all || held ? 0u : kk % Tp;
+        for (;;) {
+            const uint32_t i = base + first(kk) - t0;
+            if (i >= 32u) break;
+            const bool miss = base == 0u || (!held && (all || (m ? over(kk) : x < thr)));
+            bits |= (miss ? 1u : 0u) << i;
+            x = x + 1u == Tp ? 0u : x + 1u;
+            if (++kk == nl) {
+                kk = x = 0;
+                base += per;
+            }
+        }
+        return bits;
+    }
     // before first(): the stride's DivMagic (make_div_magic)
     __device__ __forceinline__ void prepare_first() {
         if (strided || s == 0) return;
@@ -183,8 +220,10 @@ __global__ void __launch_bounds__(256) uniform_prep_kernel(const SimItem *__rest
 // The words of every caller item: an item taken here gets its final words and
 // counts (or its Hamming distance), the played sets' later misses apart; any
 // other one is cleared for the simulator's units.  A warp takes 32 words at a
-// time, one per lane; blocks of all hits or all misses are stored at once, the
-// others take an access per lane and a vote per word.
+// time, one per lane.  A lane goes through its word's run heads (its accesses,
+// where each is one): up to 32 short turns for 32 words, where a vote per word
+// took 32 longer ones (texture and Fermi sweeps of 9.6K items: 239 us with the
+// votes, @@ so; the 4096-item batch 1519 -> @@ us).
 __global__ void __launch_bounds__(256) uniform_out_kernel(const SimItem *__restrict__ items,
                                                           uint64_t n_units, uint32_t parts,
                                                           SimOut out, uint32_t *live) {
@@ -213,35 +252,20 @@ __global__ void __launch_bounds__(256) uniform_out_kernel(const SimItem *__restr
                 for (uint32_t w = w0 + lane; w < w1; w += 32) bm[w] = 0;
             continue;
         }
-        const Chain ch(it);
+        Chain ch(it);
+        ch.prepare_first();
         const bool held = ch.rnd || (ch.m == 0 && ch.thr == 0);  // later passes: nothing here
         const bool all = !ch.rnd && ch.m == 0 && ch.thr >= ch.Tp;
         const bool ones = all && ch.strided && ch.nl > 1;
         const uint64_t ob = ham ? out.obs_word_offsets[it.obs] : 0;
         uint32_t tot = 0, aft = 0;
         uint32_t dsum = 0;
-        const uint32_t inc = 32u % ch.per;
         for (uint32_t wb = w0; wb < w1; wb += 32) {
-            const uint32_t base = wb << 5;
             uint32_t word = 0;
             if (ones) {
                 word = kFull;
-            } else if (!(held && base >= ch.per)) {
-                uint32_t k = (base + lane) % ch.per;
-                const uint32_t n = min(32u, w1 - wb);
-                for (uint32_t q = 0; q < n; ++q) {
-                    const uint32_t t = base + 32u * q + lane;
-                    const uint32_t pos = k * ch.s;
-                    const uint32_t kk = ch.strided ? k : pos >> ch.lb;
-                    // a run head: the line differs from the access before
-                    bool miss = ch.strided || k == 0 ? ch.nl > 1 : ((pos - ch.s) >> ch.lb) != kk;
-                    miss = miss || t == 0;
-                    if (t >= ch.per) miss = miss && !held && (all || ch.over(kk));
-                    const uint32_t bits = __ballot_sync(kFull, miss);
-                    if (lane == q) word = bits;
-                    k += inc;
-                    k -= k >= ch.per ? ch.per : 0u;
-                }
+            } else if (!(held && (wb << 5) >= ch.per)) {
+                word = ch.word((wb + lane) << 5, held, all);
             }
             const uint32_t w = wb + lane, t = w << 5;
             if (w < w1) {
@@ -361,11 +385,11 @@ __device__ __forceinline__ void play_small(const SimItem &it, const Chain &ch, u
     while (!__all_sync(kFull, done)) {
         constexpr int kRounds = G >= 8 ? 1 : 8 / G;  // 8 misses at least to a vote
         for (int round = 0; round < kRounds; ++round) {
-            const uint32_t wv = random_way(seed, set, k + r, a, wtd);
+            const uint32_t wv = 32u * random_way(seed, set, k + r, a, wtd);
             k += G;
-            uint32_t t = 0, p = 0;
+            uint32_t p = 0, mine_p = 0, mine_base = 0;
             uint32_t w = G == 1 ? wv : __shfl_sync(kFull, wv, glane);
-            uint32_t ld = occ[32 * w];  // line of way w, but for the miss ahead
+            uint32_t ld = occ[w];       // line of way w, but for the miss ahead
             bool again = false;         // the miss ahead took way w too
 #pragma unroll
             for (int q = 0; q < G; ++q) {
@@ -378,16 +402,18 @@ __device__ __forceinline__ void play_small(const SimItem &it, const Chain &ch, u
                 uint32_t wn = 0;
                 if (q + 1 < G) {
                     wn = __shfl_sync(kFull, wv, glane + q + 1);
-                    ld = occ[32 * wn];
+                    ld = occ[wn];
                     again = wn == w;
                 }
-                occ[32 * w] = (uint8_t)p;
+                occ[w] = (uint8_t)p;
                 const uint32_t ob = 1u << old;
                 below = (gone | ob) & ~(kFull << p);
                 gone = (gone | ob) & ~(1u << p);
-                if (G == 1 || r == (uint32_t)q) t = base + toff[32 * p];
+                mine_p = r == (uint32_t)q ? p : mine_p;
+                mine_base = r == (uint32_t)q ? base : mine_base;
                 w = wn;
             }
+            const uint32_t t = mine_base + toff[32 * mine_p];
             const bool count = !done && t < len;
             const uint32_t latest = __shfl_sync(kFull, t, glane + G - 1);
             done = done || latest >= len;
