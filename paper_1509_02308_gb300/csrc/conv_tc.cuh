@@ -81,4 +81,12 @@ cudaError_t tc_gemm(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int
 cudaError_t transpose_bf16(const __nv_bfloat16 *in, int R, int C, int ldi, __nv_bfloat16 *out,
                            int ldo, int Cpad, cudaStream_t st);
 
+// The exhaustive least-squares matcher (lsq.cu) of the first min(n, *n_dev)
+// traces y [n][512] (n_dev NULL: all) against rates [n_geoms][512]: best
+// candidate and its residual (resid_out may be NULL) per trace; work: lsq_work_bytes(n).
+size_t lsq_work_bytes(uint32_t n);
+cudaError_t lsq_run(const float *rates, uint32_t n_geoms, const float *y, uint32_t n,
+                    const uint32_t *n_dev, uint32_t *best_out, float *resid_out, void *work, int sms,
+                    cudaStream_t st);
+
 }  // namespace pchase

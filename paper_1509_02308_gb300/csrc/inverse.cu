@@ -275,141 +275,6 @@ __global__ void f2b_kernel(const float *x, size_t n, __nv_bfloat16 *y) {
         y[i] = __float2bfloat16(x[i]);
 }
 
-// ---- exhaustive least-squares matcher (FP32)
-// Per trace: keep the points at or below its 507th smallest value (drops the
-// 5 largest of 512, the spike allowance); mask m_p.  For candidate g with
-// miss rates r_gp the best affine fit y ~ alpha + beta r_g over kept points
-// leaves residual Var_y - Cov^2 / Var_r (Var_y when Var_r is 0 or the slope is
-// not positive).  The smallest residual wins; equal residuals go to the lower
-// candidate index.
-constexpr int kKeep = kPoints - 5;
-
-__global__ void lsq_prep_kernel(const float *y, uint32_t n, const uint32_t *n_dev, float *ym,
-                                float *mask, float *stats) {
-    __shared__ float v[kPoints];
-    const uint32_t i = blockIdx.x;
-    if (n_dev && *n_dev < n) n = *n_dev;
-    if (i >= n) return;
-    for (int p = threadIdx.x; p < kPoints; p += blockDim.x) v[p] = y[(size_t)i * kPoints + p];
-    __syncthreads();
-    // bitonic sort of a copy in shared memory (ascending)
-    __shared__ float sv[kPoints];
-    for (int p = threadIdx.x; p < kPoints; p += blockDim.x) sv[p] = v[p];
-    __syncthreads();
-    for (int k = 2; k <= kPoints; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int p = threadIdx.x; p < kPoints; p += blockDim.x) {
-                const int q = p ^ j;
-                if (q > p) {
-                    const bool up = (p & k) == 0;
-                    const float a = sv[p], b = sv[q];
-                    if ((a > b) == up) { sv[p] = b; sv[q] = a; }
-                }
-            }
-            __syncthreads();
-        }
-    const float thr = sv[kKeep - 1];
-    __shared__ float acc[3];
-    if (threadIdx.x < 3) acc[threadIdx.x] = 0.0f;
-    __syncthreads();
-    float c = 0.0f, sy = 0.0f, syy = 0.0f;
-    for (int p = threadIdx.x; p < kPoints; p += blockDim.x) {
-        const float m = v[p] <= thr ? 1.0f : 0.0f;
-        mask[(size_t)i * kPoints + p] = m;
-        ym[(size_t)i * kPoints + p] = m * v[p];
-        c += m;
-        sy += m * v[p];
-        syy += m * v[p] * v[p];
-    }
-    atomicAdd(&acc[0], c);
-    atomicAdd(&acc[1], sy);
-    atomicAdd(&acc[2], syy);
-    __syncthreads();
-    if (threadIdx.x < 3) stats[(size_t)i * 3 + threadIdx.x] = acc[threadIdx.x];
-}
-
-// 64 traces x 64 candidates per block, 256 threads with 4 x 4 outputs each
-__global__ void __launch_bounds__(256) lsq_kernel(const float *ym, const float *mask,
-                                                  const float *stats, uint32_t n,
-                                                  const uint32_t *n_dev, const float *rates,
-                                                  uint32_t G, unsigned long long *best) {
-    __shared__ float sY[32][65], sM[32][65], sR[32][65];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const uint32_t i0 = blockIdx.y * 64, g0 = blockIdx.x * 64;
-    if (n_dev && *n_dev < n) n = *n_dev;
-    if (i0 >= n) return;  // rows beyond the device-side count: nothing to do
-    float dyr[4][4], dr[4][4], drr[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) dyr[a][b] = dr[a][b] = drr[a][b] = 0.0f;
-    for (int k0 = 0; k0 < kPoints; k0 += 32) {
-        for (int e = threadIdx.x; e < 32 * 64; e += 256) {
-            const int kk = e & 31, r = e >> 5;
-            const uint32_t ti = i0 + r, gi = g0 + r;
-            sY[kk][r] = ti < n ? ym[(size_t)ti * kPoints + k0 + kk] : 0.0f;
-            sM[kk][r] = ti < n ? mask[(size_t)ti * kPoints + k0 + kk] : 0.0f;
-            sR[kk][r] = gi < G ? rates[(size_t)gi * kPoints + k0 + kk] : 0.0f;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int kk = 0; kk < 32; ++kk) {
-            float yv[4], mv[4], rv[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                yv[a] = sY[kk][ty * 4 + a];
-                mv[a] = sM[kk][ty * 4 + a];
-                rv[a] = sR[kk][tx * 4 + a];
-            }
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    dyr[a][b] = fmaf(yv[a], rv[b], dyr[a][b]);
-                    dr[a][b] = fmaf(mv[a], rv[b], dr[a][b]);
-                    drr[a][b] = fmaf(mv[a], rv[b] * rv[b], drr[a][b]);
-                }
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const uint32_t ti = i0 + ty * 4 + a;
-        if (ti >= n) continue;
-        const float cnt = stats[ti * 3], sy = stats[ti * 3 + 1], syy = stats[ti * 3 + 2];
-        const float var_y = syy - sy * sy / cnt;
-        unsigned long long b_best = ~0ull;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const uint32_t gi = g0 + tx * 4 + b;
-            if (gi >= G) continue;
-            const float cov = dyr[a][b] - sy * dr[a][b] / cnt;
-            const float var_r = drr[a][b] - dr[a][b] * dr[a][b] / cnt;
-            float res = var_y;
-            if (var_r > 1e-12f && cov > 0.0f) res = var_y - cov * cov / var_r;
-            res = fmaxf(res, 0.0f);
-            const unsigned long long key = ((unsigned long long)__float_as_uint(res) << 32) | gi;
-            b_best = key < b_best ? key : b_best;
-        }
-        if (b_best != ~0ull) atomicMin(best + ti, b_best);
-    }
-}
-
-__global__ void fill_u64_kernel(unsigned long long *p, size_t n, unsigned long long v) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x)
-        p[i] = v;
-}
-
-__global__ void lsq_unpack_kernel(const unsigned long long *best, uint32_t n, const uint32_t *n_dev,
-                                  uint32_t *idx, float *res) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n_dev && *n_dev < n) n = *n_dev;
-    if (i >= n) return;
-    idx[i] = (uint32_t)(best[i] & 0xFFFFFFFFull);
-    if (res) res[i] = __uint_as_float((uint32_t)(best[i] >> 32));
-}
-
 // learned predictions -> candidate index through a label table; low
 // confidence or an unknown label combination marks the trace for fallback
 __global__ void route_kernel(const uint32_t *pred, const float *conf, uint32_t n,
@@ -822,45 +687,17 @@ int pchase_inverse_infer(const pchase_inverse *h, const void *params, void *work
     return PCHASE_OK;
 }
 
-static int lsq_run(const float *rates, uint32_t n_geoms, const float *y, uint32_t n,
-                   const uint32_t *n_dev, uint32_t *best_out, float *resid_out, void *work,
-                   cudaStream_t st);
-
-size_t pchase_lsq_work_bytes(uint32_t n) {
-    return a256((size_t)n * kPoints * 4) * 2 + a256((size_t)n * 12) + a256((size_t)n * 8);
-}
+size_t pchase_lsq_work_bytes(uint32_t n) { return lsq_work_bytes(n); }
 
 int pchase_lsq_match(const float *rates, uint32_t n_geoms, const float *y, uint32_t n,
                      uint32_t *best_out, float *resid_out, void *work, pchase_stream_t stream) {
     if (!rates || !y || !best_out || !work || n_geoms == 0)
         return inv_fail(PCHASE_EINVAL, "NULL argument or no geometries");
     if (n == 0) return PCHASE_OK;
-    return lsq_run(rates, n_geoms, y, n, nullptr, best_out, resid_out, work,
-                   reinterpret_cast<cudaStream_t>(stream));
-}
-
-}  // extern "C"
-
-// The least-squares matcher over the first min(n, *n_dev) rows (n_dev NULL:
-// all n); grids cover n rows and blocks past the device-side count return.
-static int lsq_run(const float *rates, uint32_t n_geoms, const float *y, uint32_t n,
-                   const uint32_t *n_dev, uint32_t *best_out, float *resid_out, void *work,
-                   cudaStream_t st) {
-    float *ym = at<float>(work, 0);
-    float *mask = at<float>(work, a256((size_t)n * kPoints * 4));
-    float *stats = at<float>(work, 2 * a256((size_t)n * kPoints * 4));
-    unsigned long long *best = at<unsigned long long>(
-        work, 2 * a256((size_t)n * kPoints * 4) + a256((size_t)n * 12));
-    lsq_prep_kernel<<<n, 256, 0, st>>>(y, n, n_dev, ym, mask, stats);
-    fill_u64_kernel<<<grid_for(n), 256, 0, st>>>(best, n, ~0ull);
-    dim3 grid((n_geoms + 63) / 64, (n + 63) / 64);
-    lsq_kernel<<<grid, 256, 0, st>>>(ym, mask, stats, n, n_dev, rates, n_geoms, best);
-    lsq_unpack_kernel<<<(n + 255) / 256, 256, 0, st>>>(best, n, n_dev, best_out, resid_out);
-    INV_CUDA(cudaGetLastError());
+    INV_CUDA(lsq_run(rates, n_geoms, y, n, nullptr, best_out, resid_out, work, device_sms(),
+                     reinterpret_cast<cudaStream_t>(stream)));
     return PCHASE_OK;
 }
-
-extern "C" {
 
 int pchase_inverse_classify(const pchase_inverse *h, const void *params, void *work,
                             const float *x, uint32_t n, const uint32_t *label_to_cand,
@@ -881,8 +718,8 @@ int pchase_inverse_classify(const pchase_inverse *h, const void *params, void *w
     // the fallback runs over a compacted copy whose size is known only on the
     // device: the matcher's grids cover n rows and its blocks stop at the count
     gather_rows_kernel<<<n, 128, 0, st>>>(x, fallback_list, n_fallback, fb_rows);
-    rc = lsq_run(rates, n_geoms, fb_rows, n, n_fallback, fb_idx, nullptr, lsq_work, st);
-    if (rc) return rc;
+    INV_CUDA(lsq_run(rates, n_geoms, fb_rows, n, n_fallback, fb_idx, nullptr, lsq_work, device_sms(),
+                     st));
     scatter_fallback_kernel<<<(n + 255) / 256, 256, 0, st>>>(fallback_list, n_fallback, fb_idx,
                                                              cand_out);
     INV_CUDA(cudaGetLastError());
