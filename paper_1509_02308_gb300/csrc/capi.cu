@@ -21,6 +21,9 @@ size_t classify_bucket_bytes(uint32_t n_obs, uint64_t max_len);
 cudaError_t classify_thresholds(const float *lat, const uint64_t *offsets, uint32_t n_obs,
                                 uint64_t max_len, void *meta_mem, void *bucket_mem,
                                 float *thresh_out, cudaStream_t st, int sms);
+cudaError_t classify_all(const float *lat, const uint64_t *offsets, uint32_t n_obs, uint64_t max_len,
+                         void *meta_mem, void *bucket_mem, float *thresh_out, uint32_t *bits,
+                         const uint64_t *word_offsets, cudaStream_t st, int sms);
 cudaError_t classify_bits(const float *lat, const uint64_t *seg_offsets, int per_seg,
                           uint32_t n_seg, uint64_t max_seg_len, const void *meta_mem,
                           uint32_t *bits, const uint64_t *word_offsets, cudaStream_t st, int sms);
@@ -1971,11 +1974,9 @@ int pchase_classify(const float *lat, const uint64_t *offsets, uint32_t n_obs, u
     void *meta = w;
     void *bk = w + classify_meta_bytes(n_obs);
     const int sms = sm_count();
-    PCHASE_CUDA(classify_thresholds(lat, offsets, n_obs, max_len, meta, bk, thresh_out, st, sms),
-                "classify thresholds");
-    PCHASE_CUDA(classify_bits(lat, offsets, 1, n_obs, max_len,
-                              meta, bits_out, bit_word_offsets, st, sms),
-                "classify bits");
+    PCHASE_CUDA(classify_all(lat, offsets, n_obs, max_len, meta, bk, thresh_out, bits_out,
+                             bit_word_offsets, st, sms),
+                "classify");
     return PCHASE_OK;
 }
 

@@ -6,7 +6,10 @@
 // largest, take the largest gap between consecutive distinct kept values (the
 // lowest on ties) and cut at (lo + hi) * 0.5f.
 //
-// GPU form, without a sort:
+// GPU form, without a sort.  Observations of up to 8 x 48K latencies take one
+// launch (classify_cluster_kernel): a cluster of up to eight CTAs holds the
+// observation in shared memory from end to end.  Longer ones take the same
+// steps as launches over global memory:
 //   1. radix select (four 8-bit digit passes over order-preserving keys) finds
 //      the cut value v[keep-1] exactly, and the minimum;
 //   2. maximum gap by pigeonhole (Gonzalez's linear-time maximum-gap method):
@@ -19,6 +22,8 @@
 #include <mutex>
 
 #include <algorithm>
+
+#include <cooperative_groups.h>
 
 #include "pchase_internal.cuh"
 
@@ -40,6 +45,278 @@ struct ObsMeta {
     uint32_t nb;   // buckets (0: no gap possible)
     float thr;
 };
+
+// ---- one launch per call: a cluster of CTAs per observation
+// Each CTA keeps a slice of the observation's keys in shared memory.  The cut
+// value is found by three histogram passes (11, 11 and 10 bits; a bin's count
+// goes up by one per latency, which the hardware adds up within a warp), rank 0
+// adding the CTAs' bins through distributed shared memory.  The maximum gap:
+// kGapBuckets equal buckets first (min and max key of each); when the largest
+// gap between neighbouring buckets is wider than a bucket no gap inside one
+// can reach it, and it is the answer (two latency plateaus: always).  If not,
+// or where the bucket arithmetic is not regular, the 2 * keep buckets of the
+// pigeonhole method follow, kGapBuckets of them at a time.  Bound by the
+// passes over shared memory and a dozen cluster barriers: 64 observations of
+// 16K-64K latencies take @@ us against 288 us as four launches, one CTA per
+// observation; one of 177K latencies, as the matcher pools, @@ against 458 us.
+constexpr uint32_t kGapBuckets = 4096;
+constexpr uint32_t kClusterThreads = 1024;
+constexpr uint32_t kClusterMaxKeys = 49152;  // of one CTA (192 KB, beside 33 KB of buckets)
+constexpr uint32_t kClusterMax = 8;
+
+struct ClusterShared {
+    uint4 bucket4[kGapBuckets / 2];  // uint2 {min key, max key} per bucket; the histogram's bins before
+    unsigned long long best;
+    uint32_t warp_v[32];
+    uint32_t prefix, k, min_key, carry, found;
+    float gap, lo, hi, thr;
+};
+constexpr size_t kClusterSmemBase = (sizeof(ClusterShared) + 15) & ~size_t(15);
+
+// Exclusive prefix of v over the CTA's threads under op (identity id).
+template <typename Op>
+__device__ __forceinline__ uint32_t block_exclusive(uint32_t v, uint32_t id, uint32_t *warp_v, Op op) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc = op(inc, x);
+    }
+    if (lane == 31) warp_v[w] = inc;
+    __syncthreads();
+    uint32_t before = id;
+    for (int q = 0; q < w; ++q) before = op(before, warp_v[q]);
+    const uint32_t up = __shfl_up_sync(kFull, inc, 1);
+    __syncthreads();
+    return lane ? op(before, up) : before;
+}
+
+__global__ void __launch_bounds__(kClusterThreads)
+    classify_cluster_kernel(const float *__restrict__ lat, const uint64_t *__restrict__ offsets,
+                            uint64_t max_len, ObsMeta *meta, float *thresh_out, uint32_t *bits,
+                            const uint64_t *__restrict__ word_offsets) {
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) uint8_t c_smem[];
+    ClusterShared &S = *reinterpret_cast<ClusterShared *>(c_smem);
+    uint32_t *const keys = reinterpret_cast<uint32_t *>(c_smem + kClusterSmemBase);
+    uint32_t *const hist = reinterpret_cast<uint32_t *>(S.bucket4);
+    uint2 *const bucket = reinterpret_cast<uint2 *>(S.bucket4);
+    cg::cluster_group cluster = cg::this_cluster();
+    const uint32_t C = cluster.num_blocks(), rank = cluster.block_rank();
+    ClusterShared *const S0 = cluster.map_shared_rank(&S, 0);
+    const uint32_t o = blockIdx.x / C, tid = threadIdx.x;
+    const uint64_t b0 = offsets[o], n64 = offsets[o + 1] - b0;
+    if (n64 == 0 || n64 > max_len) {
+        // empty, or longer than the caller's max_len: refused (NaN cut, bits 0)
+        const float thr = n64 ? __int_as_float(0x7FC00000) : 0.0f;
+        if (rank == 0 && tid == 0) {
+            meta[o] = ObsMeta{0, 0, 0, thr};
+            if (thresh_out) thresh_out[o] = thr;
+        }
+        if (bits && n64) {
+            const uint64_t words = (n64 + 31) / 32;
+            for (uint64_t w = (uint64_t)rank * kClusterThreads + tid; w < words; w += (uint64_t)C * kClusterThreads)
+                bits[word_offsets[o] + w] = 0;
+        }
+        return;
+    }
+    const uint32_t n = (uint32_t)n64, keep = n - n / 200;
+    const uint32_t per = ((n + C - 1) / C + 31u) & ~31u;
+    const uint32_t first = min(n, rank * per), cnt = min(n, first + per) - first;
+    const float *const x = lat + b0 + first;
+    if (tid == 0) {
+        S.min_key = 0xFFFFFFFFu;
+        S.prefix = 0;
+        S.k = keep;
+        S.carry = 0;
+        S.gap = 0.0f;
+        S.found = 0;
+    }
+    __syncthreads();
+    uint32_t mn = 0xFFFFFFFFu;
+    for (uint32_t i = tid; i < cnt; i += kClusterThreads) {
+        const uint32_t k = fkey(x[i]);
+        keys[i] = k;
+        mn = min(mn, k);
+    }
+    mn = __reduce_min_sync(kFull, mn);
+    if ((tid & 31) == 0) atomicMin(&S.min_key, mn);
+    // ---- the cut value: keep-th smallest key
+    uint32_t prefix = 0, mask = 0;
+    for (int pass = 0; pass < 3; ++pass) {
+        const uint32_t shift = pass == 0 ? 21u : pass == 1 ? 10u : 0u;
+        const uint32_t bins = pass == 2 ? 1024u : 2048u;
+        for (uint32_t i = tid; i < bins; i += kClusterThreads) hist[i] = 0;
+        __syncthreads();
+        for (uint32_t i = tid; i < cnt; i += kClusterThreads) {
+            const uint32_t k = keys[i];
+            if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & (bins - 1u)], 1u);
+        }
+        cluster.sync();
+        if (rank == 0) {
+            // two bins a thread (one in the last pass), all CTAs' counts
+            uint32_t c0 = 0, c1 = 0;
+            if (2 * tid < bins)
+                for (uint32_t c = 0; c < C; ++c) {
+                    const uint2 v = *reinterpret_cast<const uint2 *>(
+                        cluster.map_shared_rank(hist, c) + 2 * tid);
+                    c0 += v.x;
+                    c1 += v.y;
+                }
+            const uint32_t before =
+                block_exclusive(c0 + c1, 0u, S.warp_v, [](uint32_t a, uint32_t b) { return a + b; });
+            const uint32_t k = S.k;
+            __syncthreads();
+            if (before < k && k <= before + c0) {
+                S.prefix = prefix | ((2 * tid) << shift);
+                S.k = k - before;
+            } else if (before + c0 < k && k <= before + c0 + c1) {
+                S.prefix = prefix | ((2 * tid + 1) << shift);
+                S.k = k - before - c0;
+            }
+            if (pass == 0 && tid < C) atomicMin(&S.min_key, cluster.map_shared_rank(&S, tid)->min_key);
+        }
+        cluster.sync();
+        prefix = S0->prefix;
+        mask |= (bins - 1u) << shift;
+    }
+    const uint32_t cut = prefix, mnk = S0->min_key;
+    const float vlo = fval(mnk), vhi = fval(cut);
+    float thr = vhi;  // no gap: every latency a hit
+    if (cut != mnk) {
+        // one round of buckets [w0, w0 + kGapBuckets) of `nb` over [vlo, vhi];
+        // rank 0 adds the largest gap so far
+        auto round = [&](uint32_t w0, uint32_t nb, float scale) {
+            for (uint32_t i = tid; i < kGapBuckets; i += kClusterThreads) bucket[i] = make_uint2(0xFFFFFFFFu, 0u);
+            __syncthreads();
+            for (uint32_t i = tid; i < cnt; i += kClusterThreads) {
+                const uint32_t k = keys[i];
+                if (k > cut) continue;
+                uint32_t bi = (uint32_t)((fval(k) - vlo) * scale);
+                if (bi >= nb) bi = nb - 1;
+                bi -= w0;
+                if (bi >= kGapBuckets) continue;
+                // (a look first: most latencies move neither end)
+                if (k < bucket[bi].x) atomicMin(&bucket[bi].x, k);
+                if (k > bucket[bi].y) atomicMax(&bucket[bi].y, k);
+            }
+            cluster.sync();
+            if (rank == 0) {
+                uint2 m[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) m[e] = make_uint2(0xFFFFFFFFu, 0u);
+                for (uint32_t c = 0; c < C; ++c) {
+                    const uint4 *const r = cluster.map_shared_rank(S.bucket4, c) + 2 * tid;
+                    const uint4 a = r[0], b = r[1];
+                    m[0] = make_uint2(min(m[0].x, a.x), max(m[0].y, a.y));
+                    m[1] = make_uint2(min(m[1].x, a.z), max(m[1].y, a.w));
+                    m[2] = make_uint2(min(m[2].x, b.x), max(m[2].y, b.y));
+                    m[3] = make_uint2(min(m[3].x, b.z), max(m[3].y, b.w));
+                }
+                const uint32_t top = max(max(m[0].y, m[1].y), max(m[2].y, m[3].y));
+                const auto larger = [](uint32_t a, uint32_t b) { return max(a, b); };
+                uint32_t prev = max(block_exclusive(top, 0u, S.warp_v, larger), S.carry);
+                if (tid == 0) S.best = 0;
+                const uint32_t last = max(prev, top);  // (the last thread's: the carry)
+                float g = 0.0f, lo = 0.0f, hi = 0.0f;
+                uint32_t at = 0;
+#pragma unroll
+                for (uint32_t e = 0; e < 4; ++e) {
+                    if (m[e].x == 0xFFFFFFFFu) continue;
+                    if (prev) {
+                        const float a = fval(prev), c = fval(m[e].x), d = c - a;
+                        if (d > g) {
+                            g = d;
+                            lo = a;
+                            hi = c;
+                            at = 4 * tid + e;
+                        }
+                    }
+                    prev = m[e].y;
+                }
+                __syncthreads();
+                // the largest gap, the lowest one on ties
+                const unsigned long long key =
+                    g > 0.0f ? ((unsigned long long)__float_as_uint(g) << 32) | (0xFFFFFFFFu - at) : 0ull;
+                if (key) atomicMax(&S.best, key);
+                __syncthreads();
+                if (key && key == S.best && g > S.gap) {
+                    S.gap = g;
+                    S.lo = lo;
+                    S.hi = hi;
+                    S.found = 1;
+                }
+                if (tid == kClusterThreads - 1) S.carry = last;
+                __syncthreads();
+            }
+            cluster.sync();
+        };
+        const float range = vhi - vlo, width = range * (1.0f / kGapBuckets), coarse = (float)kGapBuckets / range;
+        bool done = false;
+        if (isfinite(range) && range > 1e-30f && isfinite(coarse)) {
+            round(0, kGapBuckets, coarse);
+            done = S0->gap > 1.01f * width;
+            cluster.sync();
+            if (!done && rank == 0 && tid == 0) {
+                S.carry = 0;
+                S.gap = 0.0f;
+                S.found = 0;
+            }
+            cluster.sync();
+        }
+        if (!done) {
+            const uint32_t nb = 2 * keep;
+            const float scale = (float)nb / (vhi - vlo);
+            for (uint32_t w0 = 0; w0 < nb; w0 += kGapBuckets) round(w0, nb, scale);
+        }
+        if (S0->found) thr = (S0->lo + S0->hi) * 0.5f;
+    }
+    if (rank == 0 && tid == 0) {
+        meta[o] = ObsMeta{cut, mnk, cut == mnk ? 0u : 2u * keep, thr};
+        if (thresh_out) thresh_out[o] = thr;
+    }
+    if (bits) {
+        uint32_t *const out = bits + word_offsets[o] + (first >> 5);
+        const uint32_t padded = (cnt + 31u) & ~31u;
+        for (uint32_t i = tid; i < padded; i += kClusterThreads) {
+            const uint32_t v = __ballot_sync(kFull, i < cnt && fval(keys[i]) > thr);
+            if ((tid & 31) == 0) out[i >> 5] = v;
+        }
+    }
+    cluster.sync();  // rank 0's shared memory outlives the others' reads
+}
+
+// CTAs of an observation's cluster (0: too long for one), and its launch.
+uint32_t cluster_ctas(uint64_t max_len) {
+    uint32_t c = 1;
+    while (c < kClusterMax && max_len > 8192ull * c) c *= 2;
+    return max_len <= (uint64_t)c * (kClusterMaxKeys - 32) ? c : 0;
+}
+
+cudaError_t launch_cluster(const float *lat, const uint64_t *offsets, uint32_t n_obs, uint64_t max_len,
+                           ObsMeta *meta, float *thresh_out, uint32_t *bits,
+                           const uint64_t *word_offsets, cudaStream_t st) {
+    const uint32_t C = cluster_ctas(max_len);
+    const size_t per = ((max_len + C - 1) / C + 31) & ~size_t(31);
+    const size_t smem = kClusterSmemBase + 4 * per;
+    cudaError_t e = cudaFuncSetAttribute(classify_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kClusterSmemBase + 4 * kClusterMaxKeys));
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(n_obs * C);
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, classify_cluster_kernel, lat, offsets, max_len, meta, thresh_out, bits,
+                              word_offsets);
+}
 
 // One CTA per observation: cut value by radix select, minimum, bucket init.
 __global__ void __launch_bounds__(1024) select_cut_kernel(const float *lat,
@@ -77,19 +354,12 @@ __global__ void __launch_bounds__(1024) select_cut_kernel(const float *lat,
         __syncthreads();
         const uint32_t prefix = s_prefix, mask = s_mask;
         uint32_t mn = 0xFFFFFFFFu;
-        // latencies crowd into a few digits, so lanes with the same digit add
-        // their count with one atomic (warp-aggregated)
-        for (uint64_t i0 = 0; i0 < n; i0 += blockDim.x) {
-            const uint64_t i = i0 + threadIdx.x;
-            uint32_t d = 0xFFFFFFFFu;
-            if (i < n) {
-                const uint32_t k = fkey(x[i]);
-                if (pass == 0) mn = min(mn, k);
-                if ((k & mask) == prefix) d = (k >> shift) & 255u;
-            }
-            const uint32_t peers = __match_any_sync(kFull, d);
-            if (d != 0xFFFFFFFFu && (peers & ((1u << (threadIdx.x & 31)) - 1u)) == 0)
-                atomicAdd(&hist[d], (uint32_t)__popc(peers));
+        // (counts go up by one: lanes with the same digit are added up by the
+        // shared-memory increment itself)
+        for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) {
+            const uint32_t k = fkey(x[i]);
+            if (pass == 0) mn = min(mn, k);
+            if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & 255u], 1u);
         }
         if (pass == 0) {
             mn = __reduce_min_sync(kFull, mn);
@@ -211,11 +481,21 @@ __global__ void bits_kernel(const float *lat, const uint64_t *seg_offsets, int p
     const int lane = threadIdx.x & 31;
     const uint64_t warp = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t w = warp; w < words; w += nwarps) {
-        const uint64_t i = w * 32 + lane;
-        const bool miss = i < n && lat[b0 + i] > thr;
-        const uint32_t v = __ballot_sync(kFull, miss);
-        if (lane == 0) bits[wo + w] = v;
+    for (uint64_t w = 4 * warp; w < words; w += 4 * nwarps) {
+        // four words' latencies in flight
+        bool miss[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint64_t i = (w + q) * 32 + lane;
+            miss[q] = i < n && lat[b0 + i] > thr;
+        }
+        uint32_t v = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t x = __ballot_sync(kFull, miss[q]);
+            if (lane == q) v = x;
+        }
+        if (lane < 4 && w + lane < words) bits[wo + w + lane] = v;
     }
 }
 
@@ -278,6 +558,8 @@ cudaError_t classify_thresholds(const float *lat, const uint64_t *offsets, uint3
                                 float *thresh_out, cudaStream_t st, int sms) {
     ObsMeta *meta = static_cast<ObsMeta *>(meta_mem);
     uint2 *bk = static_cast<uint2 *>(bucket_mem);
+    if (cluster_ctas(max_len))
+        return launch_cluster(lat, offsets, n_obs, max_len, meta, thresh_out, nullptr, nullptr, st);
     select_cut_kernel<<<n_obs, 1024, 0, st>>>(lat, offsets, max_len, meta, bk);
     uint32_t gx = (uint32_t)((max_len + 255) / 256);
     const uint32_t cap = (uint32_t)(sms > 0 ? sms : 1) * 8;
@@ -292,7 +574,7 @@ cudaError_t classify_bits(const float *lat, const uint64_t *seg_offsets, int per
                           uint32_t n_seg, uint64_t max_seg_len, const void *meta_mem,
                           uint32_t *bits, const uint64_t *word_offsets, cudaStream_t st,
                           int sms) {
-    uint32_t gx = (uint32_t)((max_seg_len + 255) / 256);
+    uint32_t gx = (uint32_t)((max_seg_len + 1023) / 1024);
     const uint32_t cap = (uint32_t)(sms > 0 ? sms : 1) * 8;
     if (gx > cap) gx = cap;
     if (gx < 1) gx = 1;
@@ -300,6 +582,19 @@ cudaError_t classify_bits(const float *lat, const uint64_t *seg_offsets, int per
                                                   static_cast<const ObsMeta *>(meta_mem), bits,
                                                   word_offsets);
     return cudaGetLastError();
+}
+
+// Thresholds and each observation's own bits.
+cudaError_t classify_all(const float *lat, const uint64_t *offsets, uint32_t n_obs, uint64_t max_len,
+                         void *meta_mem, void *bucket_mem, float *thresh_out, uint32_t *bits,
+                         const uint64_t *word_offsets, cudaStream_t st, int sms) {
+    if (cluster_ctas(max_len))
+        return launch_cluster(lat, offsets, n_obs, max_len, static_cast<ObsMeta *>(meta_mem), thresh_out, bits,
+                              word_offsets, st);
+    cudaError_t e = classify_thresholds(lat, offsets, n_obs, max_len, meta_mem, bucket_mem, thresh_out, st, sms);
+    if (e == cudaSuccess)
+        e = classify_bits(lat, offsets, 1, n_obs, max_len, meta_mem, bits, word_offsets, st, sms);
+    return e;
 }
 
 cudaError_t canonical_pick(const pchase_geom *geoms, const uint64_t *dist, uint32_t n,
@@ -403,9 +698,8 @@ extern "C" int pchase_classify_noalloc(const float *lat, const uint64_t *offsets
     uint8_t *w = static_cast<uint8_t *>(scratch);
     // the kernels write every metadata entry and initialise every bucket they
     // read, so nothing left by an earlier call is consumed
-    e = classify_thresholds(lat, offsets, n_obs, max_len, w, w + meta, thresh_out, st, sms);
-    if (e == cudaSuccess)
-        e = classify_bits(lat, offsets, 1, n_obs, max_len, w, bits_out, bit_word_offsets, st, sms);
+    e = classify_all(lat, offsets, n_obs, max_len, w, w + meta, thresh_out, bits_out, bit_word_offsets, st,
+                     sms);
     if (e != cudaSuccess) return set_last_error(PCHASE_ECUDA, cudaGetErrorString(e));
     return PCHASE_OK;
 }
