@@ -18,6 +18,10 @@ def _u32(n, device=DEV):
     return torch.empty(int(n), dtype=torch.int32, device=device)
 
 
+def _on_current(stream) -> bool:
+    return stream is None or stream.cuda_stream == torch.cuda.current_stream().cuda_stream
+
+
 def status_word(device=DEV) -> torch.Tensor:
     return torch.zeros(1, dtype=torch.int32, device=device)
 
@@ -221,19 +225,26 @@ def cache_sim_batch(geoms: list[Geom], traces, pairs=None, stream=None):
     offs[1:] = np.cumsum([(x + 31) // 32 for x in lens])
     bitmaps = _u32(max(1, int(offs[-1])))
     counts = torch.empty(2 * max(1, n_items), dtype=torch.int64, device=DEV)
-    d_offs = torch.from_numpy(offs[:-1].astype(np.int64)).to(DEV)
-    need = ctypes.c_size_t(0)
-    args = (ctypes.addressof(ga), len(geoms), ctypes.addressof(ta), len(traces),
-            ctypes.addressof(pa) if pa is not None else None, len(pairs) if pairs is not None else 0,
-            C.ptr(bitmaps), C.ptr(d_offs), C.ptr(counts), None)
-    rc = L.cache_sim_batch(*args, None, ctypes.byref(need), C.stream_handle(stream))
-    if rc != C.ERANGE:
-        C.check(rc)
-    ws = torch.empty(need.value + 256, dtype=torch.uint8, device=DEV)
-    wp = (C.ptr(ws) + 255) & ~255
-    have = ctypes.c_size_t(need.value)
-    C.check(L.cache_sim_batch(*args, wp, ctypes.byref(have), C.stream_handle(stream)))
-    torch.cuda.current_stream().synchronize()
+    # plan, upload, run, as cache_sim_batch in C does, but planned once: the C
+    # call plans a first time to say how much workspace it needs.  The plan's own
+    # bitmap layout is `offs`.
+    h = ctypes.c_void_p()
+    C.check(L.pchase_sim_plan_create(
+        ctypes.addressof(ga), len(geoms), ctypes.addressof(ta), len(traces),
+        ctypes.addressof(pa) if pa is not None else None, len(pairs) if pairs is not None else 0,
+        None, ctypes.byref(h)))
+    try:
+        need = int(L.pchase_sim_plan_workspace_bytes(h))
+        ws = torch.empty(need + 256, dtype=torch.uint8, device=DEV)
+        wp = (C.ptr(ws) + 255) & ~255
+        st = C.stream_handle(stream)
+        if not _on_current(stream):  # what the current stream makes is ready first
+            torch.cuda.current_stream().synchronize()
+        C.check(L.pchase_sim_plan_upload(h, wp, need, st))
+        C.check(L.pchase_sim_run(h, wp, C.ptr(bitmaps), None, C.ptr(counts), None, st))
+        (torch.cuda.current_stream() if stream is None else stream).synchronize()
+    finally:
+        L.pchase_sim_plan_destroy(h)
     return bitmaps, counts.view(-1, 2)[:n_items], offs
 
 
@@ -246,10 +257,13 @@ def pchase_classify(lats: list[torch.Tensor], stream=None):
     offs[1:] = np.cumsum(n)
     w = np.zeros(len(lats), dtype=np.int64)
     w[1:] = np.cumsum([(x + 31) // 32 for x in n])[:-1]
-    flat = torch.cat([x.float().reshape(-1) for x in lats]) if lats else torch.zeros(1, device=DEV)
+    flat = (torch.cat([x if x.dim() == 1 and x.dtype == torch.float32 else x.float().reshape(-1)
+                       for x in lats]) if lats else torch.zeros(1, device=DEV))
     max_len = max(n) if n else 0
-    d_offs = torch.from_numpy(offs).to(DEV)
-    d_w = torch.from_numpy(w).to(DEV)
+    # both offset arrays in one copy, which waits for the device only when the
+    # call goes to another stream than the one that makes its inputs
+    d_both = torch.from_numpy(np.concatenate([offs, w])).to(DEV, non_blocking=_on_current(stream))
+    d_offs, d_w = d_both[:len(offs)], d_both[len(offs):]
     nwords = int(sum((x + 31) // 32 for x in n))
     bits = _u32(max(1, nwords))
     thr = torch.empty(max(1, len(lats)), dtype=torch.float32, device=DEV)
