@@ -60,14 +60,14 @@ struct ObsMeta {
 // 16K-64K latencies take @@ us against 288 us as four launches, one CTA per
 // observation; one of 177K latencies, as the matcher pools, @@ against 458 us.
 constexpr uint32_t kGapBuckets = 4096;
-constexpr uint32_t kClusterThreads = 1024;
+constexpr uint32_t kClusterThreads = 512;
 constexpr uint32_t kClusterMaxKeys = 49152;  // of one CTA (192 KB, beside 33 KB of buckets)
 constexpr uint32_t kClusterMax = 8;
 
 struct ClusterShared {
     uint4 bucket4[kGapBuckets / 2];  // uint2 {min key, max key} per bucket; the histogram's bins before
     unsigned long long best;
-    uint32_t warp_v[32];
+    uint32_t warp_v[kClusterThreads / 32];
     uint32_t prefix, k, min_key, carry, found;
     float gap, lo, hi, thr;
 };
@@ -92,7 +92,7 @@ __device__ __forceinline__ uint32_t block_exclusive(uint32_t v, uint32_t id, uin
     return lane ? op(before, up) : before;
 }
 
-__global__ void __launch_bounds__(kClusterThreads)
+__global__ void __launch_bounds__(kClusterThreads, 2)
     classify_cluster_kernel(const float *__restrict__ lat, const uint64_t *__restrict__ offsets,
                             uint64_t max_len, ObsMeta *meta, float *thresh_out, uint32_t *bits,
                             const uint64_t *__restrict__ word_offsets) {
@@ -155,25 +155,28 @@ __global__ void __launch_bounds__(kClusterThreads)
         }
         cluster.sync();
         if (rank == 0) {
-            // two bins a thread (one in the last pass), all CTAs' counts
-            uint32_t c0 = 0, c1 = 0;
-            if (2 * tid < bins)
+            // four bins a thread, all CTAs' counts
+            uint32_t m[4] = {0, 0, 0, 0};
+            if (4 * tid < bins)
                 for (uint32_t c = 0; c < C; ++c) {
-                    const uint2 v = *reinterpret_cast<const uint2 *>(
-                        cluster.map_shared_rank(hist, c) + 2 * tid);
-                    c0 += v.x;
-                    c1 += v.y;
+                    const uint4 v = *reinterpret_cast<const uint4 *>(
+                        cluster.map_shared_rank(hist, c) + 4 * tid);
+                    m[0] += v.x;
+                    m[1] += v.y;
+                    m[2] += v.z;
+                    m[3] += v.w;
                 }
-            const uint32_t before =
-                block_exclusive(c0 + c1, 0u, S.warp_v, [](uint32_t a, uint32_t b) { return a + b; });
+            uint32_t before = block_exclusive(m[0] + m[1] + m[2] + m[3], 0u, S.warp_v,
+                                              [](uint32_t a, uint32_t b) { return a + b; });
             const uint32_t k = S.k;
             __syncthreads();
-            if (before < k && k <= before + c0) {
-                S.prefix = prefix | ((2 * tid) << shift);
-                S.k = k - before;
-            } else if (before + c0 < k && k <= before + c0 + c1) {
-                S.prefix = prefix | ((2 * tid + 1) << shift);
-                S.k = k - before - c0;
+#pragma unroll
+            for (uint32_t e = 0; e < 4; ++e) {
+                if (before < k && k <= before + m[e]) {
+                    S.prefix = prefix | ((4 * tid + e) << shift);
+                    S.k = k - before;
+                }
+                before += m[e];
             }
             if (pass == 0 && tid < C) atomicMin(&S.min_key, cluster.map_shared_rank(&S, tid)->min_key);
         }
@@ -203,18 +206,21 @@ __global__ void __launch_bounds__(kClusterThreads)
             }
             cluster.sync();
             if (rank == 0) {
-                uint2 m[4];
+                constexpr uint32_t B = kGapBuckets / kClusterThreads;  // buckets a thread
+                uint2 m[B];
+                uint32_t top = 0;
 #pragma unroll
-                for (int e = 0; e < 4; ++e) m[e] = make_uint2(0xFFFFFFFFu, 0u);
+                for (uint32_t e = 0; e < B; ++e) m[e] = make_uint2(0xFFFFFFFFu, 0u);
                 for (uint32_t c = 0; c < C; ++c) {
-                    const uint4 *const r = cluster.map_shared_rank(S.bucket4, c) + 2 * tid;
-                    const uint4 a = r[0], b = r[1];
-                    m[0] = make_uint2(min(m[0].x, a.x), max(m[0].y, a.y));
-                    m[1] = make_uint2(min(m[1].x, a.z), max(m[1].y, a.w));
-                    m[2] = make_uint2(min(m[2].x, b.x), max(m[2].y, b.y));
-                    m[3] = make_uint2(min(m[3].x, b.z), max(m[3].y, b.w));
+                    const uint4 *const r = cluster.map_shared_rank(S.bucket4, c) + B / 2 * tid;
+#pragma unroll
+                    for (uint32_t e = 0; e < B; e += 2) {
+                        const uint4 a = r[e / 2];
+                        m[e] = make_uint2(min(m[e].x, a.x), max(m[e].y, a.y));
+                        m[e + 1] = make_uint2(min(m[e + 1].x, a.z), max(m[e + 1].y, a.w));
+                        top = max(top, max(a.y, a.w));
+                    }
                 }
-                const uint32_t top = max(max(m[0].y, m[1].y), max(m[2].y, m[3].y));
                 const auto larger = [](uint32_t a, uint32_t b) { return max(a, b); };
                 uint32_t prev = max(block_exclusive(top, 0u, S.warp_v, larger), S.carry);
                 if (tid == 0) S.best = 0;
@@ -222,7 +228,7 @@ __global__ void __launch_bounds__(kClusterThreads)
                 float g = 0.0f, lo = 0.0f, hi = 0.0f;
                 uint32_t at = 0;
 #pragma unroll
-                for (uint32_t e = 0; e < 4; ++e) {
+                for (uint32_t e = 0; e < B; ++e) {
                     if (m[e].x == 0xFFFFFFFFu) continue;
                     if (prev) {
                         const float a = fval(prev), c = fval(m[e].x), d = c - a;
@@ -230,7 +236,7 @@ __global__ void __launch_bounds__(kClusterThreads)
                             g = d;
                             lo = a;
                             hi = c;
-                            at = 4 * tid + e;
+                            at = B * tid + e;
                         }
                     }
                     prev = m[e].y;
@@ -287,17 +293,22 @@ __global__ void __launch_bounds__(kClusterThreads)
     cluster.sync();  // rank 0's shared memory outlives the others' reads
 }
 
-// CTAs of an observation's cluster (0: too long for one), and its launch.
-uint32_t cluster_ctas(uint64_t max_len) {
+// CTAs of an observation's cluster (0: too long for one), and its launch: as
+// few as hold it, more while its CTAs have above 8K latencies each and the
+// call's CTAs still fit the GPU side by side, two to an SM (every CTA more
+// shortens the passes and lengthens rank 0's sums: 64 observations of up to
+// 64K latencies took 131 us with eight CTAs of 1024 threads each).
+uint32_t cluster_ctas(uint64_t max_len, uint64_t n_obs, int sms) {
     uint32_t c = 1;
-    while (c < kClusterMax && max_len > 8192ull * c) c *= 2;
+    while (c < kClusterMax && (max_len > (uint64_t)c * (kClusterMaxKeys - 32) ||
+                               (max_len > 8192ull * c && n_obs * c <= (uint64_t)std::max(sms, 1))))
+        c *= 2;
     return max_len <= (uint64_t)c * (kClusterMaxKeys - 32) ? c : 0;
 }
 
 cudaError_t launch_cluster(const float *lat, const uint64_t *offsets, uint32_t n_obs, uint64_t max_len,
                            ObsMeta *meta, float *thresh_out, uint32_t *bits,
-                           const uint64_t *word_offsets, cudaStream_t st) {
-    const uint32_t C = cluster_ctas(max_len);
+                           const uint64_t *word_offsets, cudaStream_t st, uint32_t C) {
     const size_t per = ((max_len + C - 1) / C + 31) & ~size_t(31);
     const size_t smem = kClusterSmemBase + 4 * per;
     cudaError_t e = cudaFuncSetAttribute(classify_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -558,8 +569,8 @@ cudaError_t classify_thresholds(const float *lat, const uint64_t *offsets, uint3
                                 float *thresh_out, cudaStream_t st, int sms) {
     ObsMeta *meta = static_cast<ObsMeta *>(meta_mem);
     uint2 *bk = static_cast<uint2 *>(bucket_mem);
-    if (cluster_ctas(max_len))
-        return launch_cluster(lat, offsets, n_obs, max_len, meta, thresh_out, nullptr, nullptr, st);
+    if (const uint32_t C = cluster_ctas(max_len, n_obs, sms))
+        return launch_cluster(lat, offsets, n_obs, max_len, meta, thresh_out, nullptr, nullptr, st, C);
     select_cut_kernel<<<n_obs, 1024, 0, st>>>(lat, offsets, max_len, meta, bk);
     uint32_t gx = (uint32_t)((max_len + 255) / 256);
     const uint32_t cap = (uint32_t)(sms > 0 ? sms : 1) * 8;
@@ -588,9 +599,9 @@ cudaError_t classify_bits(const float *lat, const uint64_t *seg_offsets, int per
 cudaError_t classify_all(const float *lat, const uint64_t *offsets, uint32_t n_obs, uint64_t max_len,
                          void *meta_mem, void *bucket_mem, float *thresh_out, uint32_t *bits,
                          const uint64_t *word_offsets, cudaStream_t st, int sms) {
-    if (cluster_ctas(max_len))
+    if (const uint32_t C = cluster_ctas(max_len, n_obs, sms))
         return launch_cluster(lat, offsets, n_obs, max_len, static_cast<ObsMeta *>(meta_mem), thresh_out, bits,
-                              word_offsets, st);
+                              word_offsets, st, C);
     cudaError_t e = classify_thresholds(lat, offsets, n_obs, max_len, meta_mem, bucket_mem, thresh_out, st, sms);
     if (e == cudaSuccess)
         e = classify_bits(lat, offsets, 1, n_obs, max_len, meta_mem, bits, word_offsets, st, sms);

@@ -71,13 +71,18 @@ struct Chain {
         T = it.kcnt > 1 ? it.gsets : it.sets;
         a = it.ways;
         m = (it.lsh >> 8) & 255u;
-        uint32_t x = st % T, y = T;  // gcd(st, T)
-        while (x) {
-            const uint32_t r = y % x;
-            y = x;
-            x = r;
+        // T / gcd(st, T); a line step is mostly a power of two
+        if ((st & (st - 1u)) == 0u) {
+            Tp = T >> min(__ffs(st) - 1, __ffs(T) - 1);
+        } else {
+            uint32_t x = st % T, y = T;
+            while (x) {
+                const uint32_t r = y % x;
+                y = x;
+                x = r;
+            }
+            Tp = T / y;
         }
-        Tp = T / y;
         const uint64_t room = (uint64_t)a * Tp;
         thr = nl > room ? (uint32_t)min((uint64_t)Tp, nl - room) : 0u;
         rnd = it.policy >= PCHASE_RANDOM && a > 1;
@@ -91,6 +96,21 @@ struct Chain {
         if (strided) {
             // every access is a head; x: its line's class
             uint32_t x = k % Tp;
+            if (Tp >= 8u) {
+                // runs of overflowing classes and of the others, a few a word
+                for (uint32_t i = 0; i < 32u;) {
+                    const bool cold = t0 + i < per, miss = cold || (!held && (all || x < thr));
+                    uint32_t r = cold || all || held ? 32u : x < thr ? thr - x : Tp - x;
+                    r = min(min(r, per - k), 32u - i);
+                    bits |= (miss ? kFull >> (32u - r) : 0u) << i;
+                    i += r;
+                    k += r;
+                    x += r;
+                    if (k == per) k = x = 0;
+                    if (x >= Tp) x = cold || all || held ? x % Tp : 0u;
+                }
+                return bits;
+            }
 #pragma unroll 8
             for (uint32_t i = 0; i < 32; ++i) {
                 const bool miss = t0 + i < per || (!held && (all || x < thr));
