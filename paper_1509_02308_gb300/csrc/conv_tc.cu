@@ -62,38 +62,51 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
 // producer warps straight from the trace's 512 FP32 inputs (rounded to BF16
 // as the unfused path rounds them): row 8G + i of plane pl holds layer-1
 // position q = 32i + 2G - 2 + pl, channels in 16-byte chunks with the
-// 128-byte swizzle, zeros outside 0 <= q < 256.  The other eight warps issue
-// the MMAs (one thread) and run the epilogue (bias, GELU, BF16 store).  The two
-// roles meet on mbarriers: slab_full (the producers' 256 arrivals after a
-// proxy fence), slab_empty (tcgen05.commit once the MMAs that read a slab
-// are done; three slabs in flight) and acc_full (two TMEM accumulators).
+// 128-byte swizzle, zeros outside 0 <= q < 256.  Eight more warps run the
+// epilogue (bias, GELU, BF16 store) and one thread of the last warp issues the
+// MMAs.  The roles meet on mbarriers: slab_full (the producers' 256 arrivals
+// after a proxy fence), slab_empty (tcgen05.commit once the MMAs that read a
+// slab are done; three slabs in flight), acc_full and acc_empty (two TMEM
+// accumulators).
+// The output tile goes through shared memory and leaves as one TMA store: a
+// lane of the accumulator holds half a row, and 32 such rows stored from
+// registers are 32 pieces of 16 bytes an instruction (65,536 traces 925 us with
+// them, 793 us so).  What bounds it: no one pipe; FMA, tanh and shared-memory
+// wavefronts each take 43-45 % of the cycles and issue 49 %, and a second group
+// of producer warps adds nothing.
 // Every wait gives up after 2 s: the CTA then ORs PCHASE_DEV_TIMEOUT into
-// *status, each role leaves its loop at its next group barrier, the MMAs
-// already issued are waited for, and TMEM is freed.
-constexpr int kFusedThreads = 512;
+// *status, each role leaves its loop at its next wait or group barrier, the
+// MMAs already issued are waited for, and TMEM is freed.
+constexpr uint32_t kOutTile = kTileRows * 128;  // a trace's 128 output positions, 16 KB
+constexpr int kFusedThreads = 256 + 256 + 32;  // producers, epilogue, an MMA warp
+constexpr int kFusedSlabs = 3;
 constexpr uint32_t kFusedXs = 520;  // staged inputs: xs[q + 2] = x[q], zeros around
 // two buffers of staged inputs, a trace's and the next one's
-constexpr uint32_t kFusedSmem = 1024 + kWBytes + kSlabs * kSlabBytes + 2 * 4 * kFusedXs + 128;
+constexpr uint32_t kFusedSmem =
+    1024 + kWBytes + kFusedSlabs * kSlabBytes + 2 * kOutTile + 2 * 4 * kFusedXs + 4 * kCh + 128;
 
 __global__ void __launch_bounds__(kFusedThreads, 1)
     conv12_tc_kernel(const float *__restrict__ x, int nb, const __nv_bfloat16 *__restrict__ W1,
                      const float *__restrict__ bias1, const __nv_bfloat16 *__restrict__ W2,
-                     const float *__restrict__ bias2, __nv_bfloat16 *__restrict__ out,
+                     const float *__restrict__ bias2, const __grid_constant__ CUtensorMap omap,
                      uint32_t *__restrict__ status) {
-    constexpr int kLin = 512, kL1 = 256, kL2 = 128;
+    constexpr int kLin = 512, kL1 = 256;
     extern __shared__ uint8_t dsm[];
     const uint32_t raw = smem_u32(dsm);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *const gbase = dsm + (base - raw);
     const uint32_t sW = base;
     const uint32_t sSlab = base + kWBytes;
-    float *const xs = reinterpret_cast<float *>(gbase + kWBytes + kSlabs * kSlabBytes);
-    const uint32_t sBar = base + kWBytes + kSlabs * kSlabBytes + 2 * 4 * kFusedXs;
-    // barriers: slab_full[3] at sBar + 8b, slab_empty[3] at sBar + 24 + 8b,
-    // acc_full[2] at sBar + 48 + 8a; then the TMEM address and the abort flag
-    uint32_t *const tslot = reinterpret_cast<uint32_t *>(gbase + (sBar - base) + 64);
+    const uint32_t sOut = sSlab + kFusedSlabs * kSlabBytes;  // two output tiles
+    float *const xs = reinterpret_cast<float *>(gbase + (sOut - base) + 2 * kOutTile);
+    float *const sBias2 = xs + 2 * kFusedXs;
+    const uint32_t sBar = sOut + 2 * kOutTile + 2 * 4 * kFusedXs + 4 * kCh;
+    // barriers: slab_full[4] at sBar + 8b, slab_empty[4] at sEmpty + 8b,
+    // acc_full[2] at sAcc + 8a, acc_empty[2] at sFree + 8a; then the TMEM
+    // address and the abort flag
+    const uint32_t sEmpty = sBar + 8u * kFusedSlabs, sAcc = sEmpty + 8u * kFusedSlabs, sFree = sAcc + 16u;
+    uint32_t *const tslot = reinterpret_cast<uint32_t *>(gbase + (sFree - base) + 16);
     volatile uint32_t *const abort_flag = tslot + 1;
-    volatile uint32_t *const last_issued = tslot + 2;  // tiles whose MMAs were issued
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ntiles = nb;
@@ -106,23 +119,29 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
     }
     cp_async_commit();
     if (tid == 0) {
-        for (int q = 0; q < 3; ++q) {
+        for (int q = 0; q < kFusedSlabs; ++q) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 256;" ::"r"(sBar + 8 * q) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sBar + 24 + 8 * q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sEmpty + 8 * q)
                          : "memory");
         }
-        for (int a = 0; a < 2; ++a)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sBar + 48 + 8 * a)
+        for (int a = 0; a < 2; ++a) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sAcc + 8 * a)
                          : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;" ::"r"(sFree + 8 * a)
+                         : "memory");
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         *abort_flag = 0;
-        *last_issued = 0;
     }
-    if (tid < 2) xs[tid] = xs[kFusedXs + tid] = 0.0f;
-    if (tid < (int)kFusedXs - kLin - 2) xs[kLin + 2 + tid] = xs[kFusedXs + kLin + 2 + tid] = 0.0f;
+    if (tid < kCh) sBias2[tid] = bias2[tid];
+    if (tid < 2 * (int)(kFusedXs - kLin)) {
+        // the padding of each buffer: 2 words before the inputs, the rest after
+        const int u = tid / (int)(kFusedXs - kLin), e = tid % (int)(kFusedXs - kLin);
+        xs[u * (int)kFusedXs + (e < 2 ? e : kLin + e)] = 0.0f;
+    }
     // slab rows of positions -2, -1 (row 0 of each plane) and 256, 257 (row
     // 8 * 17 + 7) are zero padding, written once: the producers never write them
-    for (int e = tid; e < kSlabs * 2 * 2 * 8; e += kFusedThreads) {
+    for (int e = tid; e < kFusedSlabs * 2 * 2 * 8; e += kFusedThreads) {
         const int sb = e / 32, pl = (e / 16) & 1, which = (e / 8) & 1, c = e & 7;
         const int row = which ? 8 * 17 + 7 : 0;
         uint4 *d = reinterpret_cast<uint4 *>(gbase + kWBytes + (size_t)sb * kSlabBytes +
@@ -169,9 +188,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
         for (int j = 0;; ++j) {
             const int t = blockIdx.x + j * (int)gridDim.x;
             if (t >= ntiles) break;
-            const int b = j % kSlabs;
+            const int b = j % kFusedSlabs;
             bool ok = true;
-            if (j >= kSlabs) ok = mbar_wait(sBar + 24 + 8 * b, (uint32_t)(j / kSlabs - 1) & 1u);
+            if (j >= kFusedSlabs) ok = mbar_wait(sEmpty + 8 * b, (uint32_t)(j / kFusedSlabs - 1) & 1u);
             // this trace's inputs into buffer j mod 2 (every producer finished
             // trace j - 2, the last user of that buffer, before the barrier of
             // trace j - 1), then one barrier: the inputs are in, and no wait
@@ -235,92 +254,114 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
             asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(sBar + 8 * b)
                          : "memory");
         }
-    } else {
-        // ---------------- MMA issue and epilogue (barrier id 1)
-        const int g = tid - 256, gw = warp - 8;
-        bool bad = false;  // an accumulator wait of this thread gave up
+    } else if (warp < 16) {
+        // ---------------- epilogue: tile j from accumulator j mod 2, handed
+        // back as soon as its values are in registers.  Warp w reads TMEM lane
+        // quarter w mod 4 (its hardware quarter), column half w / 4
+        const int gw = warp - 8, quarter = gw & 3, half = gw >> 2;
+        const int r = quarter * 32 + lane;  // TMEM lane r: output position 16 (r & 7) + (r >> 3)
+        const ulonglong2 *const b2 = reinterpret_cast<const ulonglong2 *>(sBias2 + half * 32);
         for (int j = 0;; ++j) {
             const int t = blockIdx.x + j * (int)gridDim.x;
-            const bool have = t < ntiles;
-            tc_fence_before();
-            const bool stop = group_any(1, bad || *abort_flag != 0);
+            if (t >= ntiles) break;
+            // (a wait that gives up is told to the others at the tile's barrier)
+            const bool bad = !mbar_wait(sAcc + 8 * (j & 1), (uint32_t)(j >> 1) & 1u);
+            __syncwarp();
             tc_fence_after();
-            if (stop) {
-                if (bad) *abort_flag = 1;
+            const uint32_t taddr = tmem + (uint32_t)(j & 1) * 64u + (uint32_t)half * 32u +
+                                   ((uint32_t)(quarter * 32) << 16);
+            uint32_t v[2][16];
+#pragma unroll
+            for (int qq = 0; qq < 2; ++qq) tmem_ld16(taddr + qq * 16, v[qq]);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            tc_fence_before();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(sFree + 8 * (j & 1))
+                             : "memory");
+            // the tile in shared memory, row r as it comes (the store's tensor map
+            // puts it at its position), 128-byte swizzle: 8 lanes write 8 chunks
+            const uint32_t row = sOut + (uint32_t)(j & 1) * kOutTile + (uint32_t)r * 128u;
+            auto put = [&](int c, const uint32_t *q) {
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                                 row + (uint32_t)(((half * 4 + c) ^ (r & 7)) << 4)),
+                             "r"(q[0]), "r"(q[1]), "r"(q[2]), "r"(q[3])
+                             : "memory");
+            };
+#pragma unroll
+            for (int qq = 0; qq < 2; ++qq) {
+                uint32_t pk[8];
+#pragma unroll
+                for (int e = 0; e < 16; e += 4) {
+                    const ulonglong2 bb = b2[qq * 4 + (e >> 2)];
+                    pk[e >> 1] = gelu2_bf16(add2(f2(__uint_as_float(v[qq][e]), __uint_as_float(v[qq][e + 1])), bb.x));
+                    pk[(e >> 1) + 1] =
+                        gelu2_bf16(add2(f2(__uint_as_float(v[qq][e + 2]), __uint_as_float(v[qq][e + 3])), bb.y));
+                }
+                put(2 * qq, pk);
+                put(2 * qq + 1, pk + 4);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            // the tile before this one has left its buffer (issued a tile ago),
+            // which the warps fill after this barrier
+            if (gw == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            if (group_any(1, bad || *abort_flag != 0)) {
+                if (lane == 0) *abort_flag = 1;
                 break;
             }
-            if (have && g == 0) {
-                const int b = j % kSlabs;
-                if (!mbar_wait(sBar + 8 * b, (uint32_t)(j / kSlabs) & 1u)) {
-                    *abort_flag = 1;
-                } else {
-                    tc_fence_after();
-                    const uint32_t d = tmem + (uint32_t)(j & 1) * 64u;
-                    const uint32_t slab = sSlab + (uint32_t)b * kSlabBytes;
-#pragma unroll
-                    for (int k = 0; k < kTaps; ++k) {
-                        const uint32_t a0 = slab + (uint32_t)(k & 1) * kPlaneBytes + (uint32_t)(k >> 1) * 1024u;
-                        const uint32_t b0 = sW + (uint32_t)k * 8192u;
-#pragma unroll
-                        for (int s = 0; s < 4; ++s)
-                            mma_bf16(d, sw128_desc(a0 + 32u * s), sw128_desc(b0 + 32u * s),
-                                     (k | s) != 0 ? 1u : 0u);
-                    }
-                    asm volatile(
-                        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                            sBar + 48u + 8u * (uint32_t)(j & 1))
-                        : "memory");
-                    asm volatile(
-                        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                            sBar + 24u + 8u * (uint32_t)b)
-                        : "memory");
-                    *last_issued = (uint32_t)(j + 1);
-                }
+            if (gw == 0 && lane == 0) {
+                asm volatile(
+                    "cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::
+                        "l"(reinterpret_cast<uint64_t>(&omap)), "r"(0), "r"(0), "r"(0), "r"(t),
+                    "r"(sOut + (uint32_t)(j & 1) * kOutTile)
+                    : "memory");
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
-            if (j > 0) {
-                // epilogue of tile j - 1 (issued: tile j - 1 had its MMAs unless aborted)
-                const int jp = j - 1;
-                if (!mbar_wait(sBar + 48 + 8 * (jp & 1), (uint32_t)(jp >> 1) & 1u)) bad = true;
-                tc_fence_after();
-                const int tp = t - (int)gridDim.x;
-                const int quarter = gw & 3, half = gw >> 2;
-                const uint32_t taddr = tmem + (uint32_t)(jp & 1) * 64u + (uint32_t)half * 32u +
-                                       ((uint32_t)(quarter * 32) << 16);
-                uint32_t v[2][16];
+        }
+        if (gw == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    } else if (lane == 0) {
+        // ---------------- MMA issue: one thread, ahead of the epilogue by one
+        // tile (two accumulators)
+        uint64_t da[kTaps], db[kTaps];  // tap k in slab 0, and its weights
 #pragma unroll
-                for (int qq = 0; qq < 2; ++qq) tmem_ld16(taddr + qq * 16, v[qq]);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                const int r = quarter * 32 + lane;
-                const int m = 16 * (r & 7) + (r >> 3);  // output position of TMEM lane r
-                uint4 *o4 = reinterpret_cast<uint4 *>(out + ((size_t)tp * kL2 + m) * kCh + half * 32);
-#pragma unroll
-                for (int qq = 0; qq < 2; ++qq) {
-                    uint32_t pk[8];
-#pragma unroll
-                    for (int e = 0; e < 16; e += 2) {
-                        const int n = half * 32 + qq * 16 + e;
-                        pk[e >> 1] = gelu2_bf16(add2(f2(__uint_as_float(v[qq][e]),
-                                                        __uint_as_float(v[qq][e + 1])),
-                                                     f2(__ldg(bias2 + n), __ldg(bias2 + n + 1))));
-                    }
-                    o4[2 * qq] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                    o4[2 * qq + 1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-                }
+        for (int q = 0; q < kTaps; ++q) {
+            da[q] = sw128_desc(sSlab + (uint32_t)(q & 1) * kPlaneBytes + (uint32_t)(q >> 1) * 1024u);
+            db[q] = sw128_desc(sW + (uint32_t)q * 8192u);
+        }
+        int issued = 0;
+        for (int j = 0;; ++j) {
+            const int t = blockIdx.x + j * (int)gridDim.x;
+            if (t >= ntiles || *abort_flag) break;
+            const int b = j % kFusedSlabs;
+            // the epilogue has tile j - 2's values, and slab j is written
+            if ((j >= 2 && !mbar_wait(sFree + 8 * (j & 1), (uint32_t)((j >> 1) - 1) & 1u)) ||
+                !mbar_wait(sBar + 8 * b, (uint32_t)(j / kFusedSlabs) & 1u)) {
+                *abort_flag = 1;
+                break;
             }
-            if (!have) break;
+            tc_fence_after();
+            const uint32_t d = tmem + (uint32_t)(j & 1) * 64u;
+            const uint64_t off = (uint64_t)((uint32_t)b * kSlabBytes >> 4);  // slab b's, in 16 bytes
+#pragma unroll
+            for (int q = 0; q < kTaps; ++q)
+#pragma unroll
+                for (int s = 0; s < 4; ++s)
+                    mma_bf16(d, da[q] + off + 2u * s, db[q] + 2u * s, (q | s) != 0 ? 1u : 0u);
+            asm volatile(
+                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                    sAcc + 8u * (uint32_t)(j & 1))
+                : "memory");
+            asm volatile(
+                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                    sEmpty + 8u * (uint32_t)b)
+                : "memory");
+            issued = j + 1;
         }
-        if (bad) *abort_flag = 1;
-        // every commit's arrival lands before the CTA leaves (the last tiles'
-        // slab_empty arrivals have no producer waiting for them; after a
-        // timeout, MMAs issued but never waited for must also finish before
-        // TMEM is freed)
-        if (g == 0) {
-            const uint32_t li = *last_issued;
-            if (li && *abort_flag)
-                mbar_wait(sBar + 48 + 8 * ((li - 1) & 1), (uint32_t)((li - 1) >> 1) & 1u);
-            for (uint32_t jj = li > (uint32_t)kSlabs ? li - kSlabs : 0u; jj < li; ++jj)
-                mbar_wait(sBar + 24 + 8 * (jj % kSlabs), (jj / kSlabs) & 1u);
-        }
+        // every commit's arrival lands, and every MMA issued finishes, before
+        // TMEM is freed and the CTA leaves
+        for (int jj = issued > kFusedSlabs ? issued - kFusedSlabs : 0; jj < issued; ++jj)
+            mbar_wait(sEmpty + 8 * (jj % kFusedSlabs), (uint32_t)(jj / kFusedSlabs) & 1u);
+        for (int jj = issued > 2 ? issued - 2 : 0; jj < issued; ++jj)
+            mbar_wait(sAcc + 8 * (jj & 1), (uint32_t)(jj >> 1) & 1u);
     }
     tc_fence_before();
     __syncthreads();
@@ -775,6 +816,21 @@ cudaError_t conv34_tc(const __nv_bfloat16 *x, int nb, const __nv_bfloat16 *W3, c
     return cudaGetLastError();
 }
 
+// Layer 2's outputs [nb][128][64] BF16 as a 4-D tensor (channel, position / 16,
+// position mod 16, trace): a box is a trace's tile with its rows in the order
+// of the accumulator's lanes, lane 8g + i holding position 16i + g
+static bool conv12_out_map(__nv_bfloat16 *out, int nb, CUtensorMap *map) {
+    const PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
+    if (!encode) return false;
+    const cuuint64_t dims[4] = {64, 8, 16, (cuuint64_t)nb};
+    const cuuint64_t strides[3] = {16 * 128, 128, 128 * 128};
+    const cuuint32_t box[4] = {64, 8, 16, 1};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, out, dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 cudaError_t conv12_tc(const float *x, int nb, const __nv_bfloat16 *W1, const float *bias1,
                       const __nv_bfloat16 *W2, const float *bias2, __nv_bfloat16 *out,
                       uint32_t *status, int sms, cudaStream_t st) {
@@ -785,7 +841,9 @@ cudaError_t conv12_tc(const float *x, int nb, const __nv_bfloat16 *W1, const flo
                                          (int)kFusedSmem);
     if (e != cudaSuccess) return e;
     const int grid = std::min(nb, std::max(1, sms));
-    conv12_tc_kernel<<<grid, kFusedThreads, kFusedSmem, st>>>(x, nb, W1, bias1, W2, bias2, out,
+    CUtensorMap omap;
+    if (!conv12_out_map(out, nb, &omap)) return cudaErrorInvalidValue;
+    conv12_tc_kernel<<<grid, kFusedThreads, kFusedSmem, st>>>(x, nb, W1, bias1, W2, bias2, omap,
                                                                status);
     return cudaGetLastError();
 }
