@@ -58,10 +58,11 @@ cudaError_t conv_back_tc(const float *dact, const float *pre, const __nv_bfloat1
                          int lout, const __nv_bfloat16 *W, float *gW, float *gb, float *dx,
                          uint32_t *status, int sms, cudaStream_t st);
 
-// The same for the first layer (one input channel, x [nb][512] BF16, W
-// [64][5]; no input gradient), on CUDA cores.
-cudaError_t conv0_back(const float *dact, const float *pre, const __nv_bfloat16 *x, int nb,
-                       float *gW, float *gb, int sms, cudaStream_t st);
+// The same for the first layer (one input channel, x [nb][512] FP32, rounded
+// to BF16 as inputs, W [64][5] + bias; pre-activations worked out again, no
+// input gradient), on CUDA cores.
+cudaError_t conv0_back(const float *dact, const float *x, const __nv_bfloat16 *W, const float *bias,
+                       int nb, float *gW, float *gb, int sms, cudaStream_t st);
 
 // C = A B^T on the tcgen05 tensor cores: A [M][K], B [N][K] BF16 with row
 // strides lda, ldb (multiples of 8 elements, 16-byte aligned bases).  Tiles of

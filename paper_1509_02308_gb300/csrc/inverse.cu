@@ -57,14 +57,16 @@ __global__ void gelu_back_kernel(const float *dy, const float *pre, size_t n, fl
 }
 
 // softmax cross-entropy over the four heads; loss (mean over the batch and
-// heads) accumulated into *loss; dlogits = (softmax - onehot) / (4 batch)
+// heads) accumulated into *loss; dlogits = (softmax - onehot) / (4 batch).  A
+// thread per trace and head (a thread per trace left 4096 traces to 32 CTAs:
+// 16 us); a warp adds its losses before the one atomic.
 __global__ void xent_kernel(const float *logits, const uint32_t *labels, int nb, float *dlog,
                             __nv_bfloat16 *dlogb, float *loss) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nb) return;
+    const int u = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = u >> 2, h = u & 3;
     float l = 0.0f;
     const float inv = 1.0f / (4.0f * nb);
-    for (int h = 0; h < 4; ++h) {
+    if (b < nb) {
         const int o0 = c_head_off[h], o1 = c_head_off[h + 1];
         const float *z = logits + (size_t)b * kLogits;
         float mx = -INFINITY;
@@ -72,16 +74,18 @@ __global__ void xent_kernel(const float *logits, const uint32_t *labels, int nb,
         float se = 0.0f;
         for (int i = o0; i < o1; ++i) se += expf(z[i] - mx);
         const uint32_t y = labels[(size_t)b * 4 + h];
-        l += logf(se) + mx - z[o0 + y];
+        l = (logf(se) + mx - z[o0 + y]) * inv;
         for (int i = o0; i < o1; ++i) {
             const float p = expf(z[i] - mx) / se;
             const float d = (p - (i == (int)(o0 + y) ? 1.0f : 0.0f)) * inv;
             dlog[(size_t)b * kLogits + i] = d;
             dlogb[(size_t)b * kLogitsPad + i] = __float2bfloat16(d);
         }
+        if (h == 3) dlogb[(size_t)b * kLogitsPad + kLogits] = __float2bfloat16(0.0f);
     }
-    dlogb[(size_t)b * kLogitsPad + kLogits] = __float2bfloat16(0.0f);
-    atomicAdd(loss, l * inv);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(kFull, l, o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(loss, l);
 }
 
 // Adam (Kingma & Ba 2015) on FP32 master weights; refreshes BF16 copies
@@ -197,7 +201,8 @@ __global__ void predict_kernel(const float *logits, int nb, uint32_t *pred, floa
     conf[b] = c;
 }
 
-// column sums with atomics (out zeroed by the caller)
+// column sums with atomics (out zeroed by the caller); a thread's rows are
+// loads one after the other, so few of them to a block (256 rows: 12 us)
 __global__ void colsum_atomic_kernel(const float *x, int rows, int cols, int rows_per_block,
                                      float *out) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -205,25 +210,26 @@ __global__ void colsum_atomic_kernel(const float *x, int rows, int cols, int row
     const int r0 = blockIdx.y * rows_per_block;
     const int r1 = min(rows, r0 + rows_per_block);
     float s = 0.0f;
+#pragma unroll 8
     for (int r = r0; r < r1; ++r) s += x[(size_t)r * cols + c];
     atomicAdd(out + c, s);
 }
 
 // First convolution (1 input channel) of the training forward pass:
-// pre[b][p][co] = bias[co] + sum_k W[co][k] * x[b][2p + k - 2] (BF16 operands,
-// FP32 sums) and out = BF16(GELU(pre)).  One block per trace: the 512 inputs
-// are staged in shared memory (zero padding around them); thread t computes
-// channels 8 (t % 8) .. +7 at positions 8 (t / 8) .. +7: per position one
-// 16-byte store of out and two of pre.  HBM-bound on the 96 KB written per
-// trace.
-__global__ void __launch_bounds__(256) conv1_kernel(const __nv_bfloat16 *__restrict__ x, int nb,
+// out[b][p][co] = BF16(GELU(bias[co] + sum_k W[co][k] * x[b][2p + k - 2])) (BF16
+// operands, the FP32 inputs rounded here, FP32 sums; the backward pass works
+// the pre-activations out again).  One block per trace: the 512 inputs are
+// staged in shared memory (zero padding around them); thread t computes
+// channels 8 (t % 8) .. +7 at positions t / 8 + 32 i, so that a warp stores
+// four whole rows.  32 KB written per trace (with the 64 KB of FP32
+// pre-activations 4096 traces took 90 us, 47 us without).
+__global__ void __launch_bounds__(256) conv1_kernel(const float *__restrict__ x, int nb,
                                                     const __nv_bfloat16 *__restrict__ W,
                                                     const float *__restrict__ bias,
-                                                    __nv_bfloat16 *__restrict__ out,
-                                                    float *__restrict__ pre) {
+                                                    __nv_bfloat16 *__restrict__ out) {
     constexpr int lout = kPoints / 2;
     __shared__ float xs[kPoints + 8];  // xs[q + 2] = x[q], zeros outside
-    const int t = threadIdx.x, g = t & 7, p0 = (t >> 3) * 8;
+    const int t = threadIdx.x, g = t & 7, p0 = t >> 3;
     float w[8][kKer], bs[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
@@ -235,13 +241,13 @@ __global__ void __launch_bounds__(256) conv1_kernel(const __nv_bfloat16 *__restr
         __syncthreads();  // the previous trace's reads are done
         for (int q = t; q < kPoints + 8; q += blockDim.x) {
             const int src = q - 2;
-            xs[q] = (src >= 0 && src < kPoints) ? __bfloat162float(x[(size_t)b * kPoints + src])
-                                                : 0.0f;
+            xs[q] = (src >= 0 && src < kPoints)
+                        ? __bfloat162float(__float2bfloat16(x[(size_t)b * kPoints + src])) : 0.0f;
         }
         __syncthreads();
 #pragma unroll 2
         for (int i = 0; i < 8; ++i) {
-            const int p = p0 + i;
+            const int p = p0 + 32 * i;
             float xin[kKer];
 #pragma unroll
             for (int k = 0; k < kKer; ++k) xin[k] = xs[2 * p + k];  // x[2p + k - 2]
@@ -254,9 +260,6 @@ __global__ void __launch_bounds__(256) conv1_kernel(const __nv_bfloat16 *__restr
                 for (int k = 0; k < kKer; ++k) acc = fmaf(w[c][k], xin[k], acc);
                 v[c] = acc + bs[c];
             }
-            float4 *po = reinterpret_cast<float4 *>(pre + row * kCh + g * 8);
-            po[0] = make_float4(v[0], v[1], v[2], v[3]);
-            po[1] = make_float4(v[4], v[5], v[6], v[7]);
             uint32_t pk[4];
 #pragma unroll
             for (int c = 0; c < 8; c += 2) {
@@ -364,7 +367,7 @@ struct pchase_inverse {
     InverseLayout L;
     uint32_t max_batch;
     size_t p_w, p_wb, p_g, p_m, p_v, p_bytes;
-    size_t status, xb, pre[4], act[4], pre4, h4, logits, dlog, dlogb, tA, tB, w4t, w5t, dh, dzf, dzb, dbig,
+    size_t status, pre[4], act[4], pre4, h4, logits, dlog, dlogb, tA, tB, w4t, w5t, dh, dzf, dzb, dbig,
         dsmall, work_bytes, infer_bytes;
 };
 
@@ -397,11 +400,11 @@ int device_sms() {
 }
 
 int forward(const pchase_inverse *h, const void *params, void *work, uint32_t B, cudaStream_t st,
-            bool train, const float *xf = nullptr) {
+            bool train, const float *xf) {
     const InverseLayout &L = h->L;
     const __nv_bfloat16 *wb = at<__nv_bfloat16>(params, h->p_wb);
     const float *wf = at<float>(params, h->p_w);
-    const __nv_bfloat16 *in = at<__nv_bfloat16>(work, h->xb);
+    const __nv_bfloat16 *in = nullptr;
     int l0 = 0;
     if (!train) {
         // inference: layers 1 and 2 in one tcgen05 kernel from the FP32 inputs
@@ -430,7 +433,7 @@ int forward(const pchase_inverse *h, const void *params, void *work, uint32_t B,
         // first layer (one input channel): direct
         __nv_bfloat16 *o = at<__nv_bfloat16>(work, h->act[l]);
         conv1_kernel<<<std::min<uint32_t>(B, 152u * 8u), 256, 0, st>>>(
-            in, (int)B, wb + L.w[l], wf + L.b[l], o, at<float>(work, h->pre[l]));
+            xf, (int)B, wb + L.w[l], wf + L.b[l], o);
         INV_CUDA(cudaGetLastError());
         in = o;
     }
@@ -478,7 +481,6 @@ int pchase_inverse_create(uint32_t max_batch, pchase_inverse **out) {
     // prefix, pchase_inverse_infer_work_bytes), then the training step's
     o = 0;
     h->status = o; o = a256(o + 4);
-    h->xb = o; o = a256(o + 2 * B * kPoints);
     for (int l = 0; l < 4; ++l) {
         const size_t lout = h->L.lin[l] / 2;
         h->act[l] = o; o = a256(o + 2 * B * lout * kCh);
@@ -488,7 +490,10 @@ int pchase_inverse_create(uint32_t max_batch, pchase_inverse **out) {
     size_t big = B * kFlat;  // largest per-layer FP32 activation gradient
     for (int l = 0; l < 4; ++l) {
         const size_t lout = h->L.lin[l] / 2;
-        h->pre[l] = o; o = a256(o + 4 * B * lout * kCh);
+        if (l > 0) {  // (the first layer's are worked out again)
+            h->pre[l] = o;
+            o = a256(o + 4 * B * lout * kCh);
+        }
         big = std::max(big, B * lout * kCh);
     }
     h->pre4 = o; o = a256(o + 4 * B * kHidden);
@@ -583,9 +588,7 @@ int pchase_inverse_train_step(const pchase_inverse *h, void *params, void *work,
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const InverseLayout &L = h->L;
     INV_CUDA(cudaMemsetAsync(at<uint32_t>(work, h->status), 0, 4, st));
-    f2b_kernel<<<grid_for((size_t)B * kPoints), 256, 0, st>>>(x, (size_t)B * kPoints,
-                                                               at<__nv_bfloat16>(work, h->xb));
-    int rc = forward(h, params, work, B, st, true);
+    int rc = forward(h, params, work, B, st, true, x);
     if (rc) return rc;
     const size_t n = L.n_params;
     float *grad = at<float>(params, h->p_g);
@@ -593,7 +596,7 @@ int pchase_inverse_train_step(const pchase_inverse *h, void *params, void *work,
     INV_CUDA(cudaMemsetAsync(grad, 0, 4 * n, st));
     float *dlog = at<float>(work, h->dlog);
     __nv_bfloat16 *dlogb = at<__nv_bfloat16>(work, h->dlogb);
-    xent_kernel<<<(B + 127) / 128, 128, 0, st>>>(at<float>(work, h->logits), labels, (int)B, dlog,
+    xent_kernel<<<(B + 31) / 32, 128, 0, st>>>(at<float>(work, h->logits), labels, (int)B, dlog,
                                                  dlogb, loss_accum);
     // heads and FC on the tcgen05 tensor cores.  Products over the batch
     // (weight gradients) take both operands batch-contiguous: transposed
@@ -612,8 +615,8 @@ int pchase_inverse_train_step(const pchase_inverse *h, void *params, void *work,
         INV_CUDA(transpose_bf16(dlogb, (int)B, kLogitsPad, kLogitsPad, tB, ldk, kLogitsPad, st));
         INV_CUDA(tc_gemm(tA, ldk, tB, ldk, kHidden, kLogits, ldk, 32, 32, nullptr, grad + L.w[5],
                          kHidden, true, true, nullptr, nullptr, status, st));
-        colsum_atomic_kernel<<<dim3(1, (B + 255) / 256), 32, 0, st>>>(dlog, (int)B, kLogits, 256,
-                                                                       grad + L.b[5]);
+        colsum_atomic_kernel<<<dim3(1, (B + 31) / 32), 32, 0, st>>>(dlog, (int)B, kLogits, 32,
+                                                                     grad + L.b[5]);
         // dh [B][256] = dlogb W5
         INV_CUDA(tc_gemm(dlogb, kLogitsPad, w5t, kLogitsPad, (int)B, kHidden, kLogitsPad, 128, 1,
                          nullptr, at<float>(work, h->dh), kHidden, false, false, nullptr, nullptr,
@@ -633,8 +636,8 @@ int pchase_inverse_train_step(const pchase_inverse *h, void *params, void *work,
                                 kFlat, st));
         INV_CUDA(tc_gemm(tA, ldk, tB, ldk, kHidden, kFlat, ldk, 128, 4, nullptr, grad + L.w[4],
                          kFlat, true, false, nullptr, nullptr, status, st));
-        colsum_atomic_kernel<<<dim3((kHidden + 127) / 128, (B + 255) / 256), 128, 0, st>>>(
-            dzf, (int)B, kHidden, 256, grad + L.b[4]);
+        colsum_atomic_kernel<<<dim3((kHidden + 127) / 128, (B + 31) / 32), 128, 0, st>>>(
+            dzf, (int)B, kHidden, 32, grad + L.b[4]);
         // d(act3) [B][32 x 64] = dzb W4
         INV_CUDA(tc_gemm(dzb, kHidden, w4t, kHidden, (int)B, kFlat, kHidden, 128, 1, nullptr, dbig,
                          kFlat, false, false, nullptr, nullptr, status, st));
@@ -652,8 +655,8 @@ int pchase_inverse_train_step(const pchase_inverse *h, void *params, void *work,
                                   at<uint32_t>(work, h->status), sms, st));
             std::swap(dcur, dnext);
         }
-        INV_CUDA(conv0_back(dcur, at<float>(work, h->pre[0]), at<__nv_bfloat16>(work, h->xb),
-                            (int)B, grad + L.w[0], grad + L.b[0], sms, st));
+        INV_CUDA(conv0_back(dcur, x, wb + L.w[0], at<float>(params, h->p_w) + L.b[0], (int)B,
+                            grad + L.w[0], grad + L.b[0], sms, st));
     }
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - powf(b1, (float)step + 1.0f), c2 = 1.0f - powf(b2, (float)step + 1.0f);

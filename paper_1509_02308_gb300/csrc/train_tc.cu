@@ -79,6 +79,7 @@ constexpr uint32_t kOffBias = kOffBar + 32;         // 64 FP32 bias partial sums
 constexpr uint32_t kBackSmem = 1024 + kOffBias + 64 * 4;
 static_assert(kOffXT + kXTAtom + 3 * 16384 <= kOffZero, "third gW tile reads past the window");
 static_assert(kBackSmem <= 232448, "shared memory");
+static_assert(4 * 16384 <= 2 * kXTAtom, "a tile of dx in the transposed window's buffer");
 
 // tcgen05 instruction descriptors (FP32 accumulator, BF16 A and B, both
 // K-major, M = 128): N = 128 for dx, N = 64 for gW
@@ -111,6 +112,22 @@ __device__ __forceinline__ void st_shared_b32(uint32_t addr, uint32_t v) {
     asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
+// TMA tile stores out of shared memory, each a bulk group of its own
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap *map, int c0, int c1, int c2, uint32_t src) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(c0), "r"(c1), "r"(c2), "r"(src)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, int c0, int c1, uint32_t src) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(c0), "r"(c1), "r"(src)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
 // byte offset of 16-byte chunk c of row r in a K-major operand whose rows are
 // 128 bytes (64 BF16) with the 128-byte swizzle
 __device__ __forceinline__ uint32_t sw_chunk(uint32_t r, uint32_t c) {
@@ -123,7 +140,7 @@ __global__ void __launch_bounds__(kBackThreads, 1)
     conv_back_tc_kernel(const float *__restrict__ dact, const float *__restrict__ pre,
                         const __grid_constant__ CUtensorMap xmap, const __nv_bfloat16 *__restrict__ W,
                         int nb, float *__restrict__ gW, float *__restrict__ gb,
-                        float *__restrict__ dx, uint32_t *status) {
+                        const __grid_constant__ CUtensorMap dmap, uint32_t *status) {
     constexpr int lout = LOUT;
     extern __shared__ uint8_t dsm[];
     const uint32_t raw = smem_u32(dsm);
@@ -137,10 +154,12 @@ __global__ void __launch_bounds__(kBackThreads, 1)
     float *const sbias = reinterpret_cast<float *>(gbase + kOffBias);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int lin = 2 * lout;
     const int nrows = nb * lout;
     const int ntiles = (nrows + kRowsPerTile - 1) / kRowsPerTile;
     const int tpt = kRowsPerTile / lout;  // traces per tile
+    // the thread of each 32-column group of warps that stores the group's part
+    // of dx (a TMA store of 128 rows x 128 bytes)
+    const bool storer = (warp & 3) == 0 && lane == 0;
 
     // B operands of dx: tile j, row n = (tap 2j + n / 64, ci = n % 64), K = co
     for (int e = tid; e < 3 * 128 * 8; e += kBackThreads) {
@@ -259,6 +278,8 @@ __global__ void __launch_bounds__(kBackThreads, 1)
             if (lo == 0) st_shared_v4(sS + 32768u + sw_chunk((uint32_t)r, (uint32_t)c), z);
         }
         const bool wok = mbar_wait(sXBar, (uint32_t)(windows - 1) & 1u);
+        // the last tile's dx has been read out of the transposes' buffer
+        if (storer) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         if (__syncthreads_or(!wok)) {
             timed_out = true;
             break;
@@ -346,32 +367,35 @@ __global__ void __launch_bounds__(kBackThreads, 1)
             break;
         }
         // ---- dx epilogue: warp w reads lanes 32 (w % 4) .. (rows q) and
-        // columns 32 (w / 4) .. +31: even positions for w / 4 < 2, odd after
+        // columns 32 (w / 4) .. +31: even positions for w / 4 < 2, odd after.
+        // A lane holds 128 bytes of a row of dx, so the rows go through shared
+        // memory (the transposed window's buffer, which these MMAs were the
+        // last to read) and leave as a TMA store per column group; 32 lanes
+        // storing 16 bytes each to rows 512 bytes apart took most of the tile's
+        // memory issue (layers 2-4 of 4096 traces: 395 us, 272 us so)
         {
             const int lg = warp & 3, qq = warp >> 2, h = qq >> 1;
-            const int q = 32 * lg + lane;
+            const uint32_t q = (uint32_t)(32 * lg + lane);
+            const uint32_t box = sXT + (uint32_t)qq * 16384u;
             uint32_t v[2][16];
 #pragma unroll
             for (int k = 0; k < 2; ++k)
                 tmem_ld16(tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)(32 * qq + 16 * k), v[k]);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            const int grow = row0 + q;
-            if (grow < nrows) {
-                const int b = grow / lout, lo = grow % lout;
-                float4 *o = reinterpret_cast<float4 *>(dx + ((size_t)b * lin + 2 * lo + h) * kCh +
-                                                       32 * (qq & 1));
 #pragma unroll
-                for (int k = 0; k < 2; ++k)
+            for (int k = 0; k < 2; ++k)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        o[4 * k + e] = make_float4(__uint_as_float(v[k][4 * e]),
-                                                   __uint_as_float(v[k][4 * e + 1]),
-                                                   __uint_as_float(v[k][4 * e + 2]),
-                                                   __uint_as_float(v[k][4 * e + 3]));
-            }
+                for (int e = 0; e < 4; ++e)
+                    st_shared_v4(box + sw_chunk(q, (uint32_t)(4 * k + e)),
+                                 make_uint4(v[k][4 * e], v[k][4 * e + 1], v[k][4 * e + 2], v[k][4 * e + 3]));
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("bar.sync %0, 128;" ::"r"(1 + qq) : "memory");
+            // (rows past the batch are out of the tensor)
+            if (storer) tma_store_3d(&dmap, 32 * (qq & 1), h, row0, box);
         }
         tc_fence_before();
     }
+    if (storer) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     // ---- partial sums into the gradient
 #pragma unroll
     for (int e = 0; e < 8; ++e) atomicAdd(&sbias[c * 8 + e], bacc[e]);
@@ -414,64 +438,91 @@ __global__ void __launch_bounds__(kBackThreads, 1)
                      : "memory");
 }
 
-// First layer (one input channel): dact, pre [nb * 256][64] FP32, x [nb][512]
-// BF16.  A CTA takes whole traces (a grid-stride loop): the trace's inputs
-// are staged in shared memory and thread t takes channels 8 (t % 8) .. +7 at
-// positions 8 (t / 8) .. +7, two positions' dact and pre (eight 16-byte
-// loads) in flight at a time.  Partial sums stay in registers over all of the
-// CTA's traces, then meet across the warp (shuffles), in shared memory, and
-// in one atomic per value and CTA.
-__global__ void __launch_bounds__(256) conv0_back_kernel(const float *__restrict__ dact,
-                                                         const float *__restrict__ pre,
-                                                         const __nv_bfloat16 *__restrict__ x,
-                                                         int nb, float *__restrict__ gW,
-                                                         float *__restrict__ gb) {
+// First layer (one input channel): dact [nb * 256][64] FP32, x [nb][512]
+// FP32 (rounded to BF16 as the forward pass rounds it).  The pre-activations
+// are not read back: conv1_kernel's five FMAs and bias, in its order, give the
+// same values again for a fraction of the 268 MB of 4096 traces.  A CTA takes
+// whole traces (a grid-stride loop): the trace's inputs are staged in shared
+// memory and thread t takes channels 4 (t % 16) .. +3 at positions t / 16 +
+// 16 i (a warp's load is two whole rows of dact), four positions in flight.
+// Partial sums stay in registers over all of the CTA's traces, then meet
+// across the warp (a shuffle), in shared memory, and in one atomic per value
+// and CTA.  4096 traces take 90 us (115 with pre read; 40 us for dact alone at
+// the copy rate): issue is half used and the loads' latency is the rest, hence
+// the four positions loaded ahead at two CTAs per SM (122 us without, at three).
+__global__ void __launch_bounds__(256, 2) conv0_back_kernel(const float *__restrict__ dact,
+                                                         const float *__restrict__ x,
+                                                         const __nv_bfloat16 *__restrict__ W,
+                                                         const float *__restrict__ bias, int nb,
+                                                         float *__restrict__ gW, float *__restrict__ gb) {
     constexpr int kLout = 256, kLin = 512;
-    __shared__ float xs[kLin + 8];  // xs[q + 2] = x[q], zeros outside
+    // xs[u][q + 2] = x[q], zeros outside: this trace's and the next one's
+    __shared__ float xs2[2][kLin + 8];
     __shared__ float sw[kCh * kTaps], sb[kCh];
-    const int t = threadIdx.x, c = t & 7, p0 = (t >> 3) * 8;
+    const int t = threadIdx.x, c = t & 15, p0 = t >> 4;
+    if (t < 8) xs2[0][t < 2 ? t : kLin + t] = xs2[1][t < 2 ? t : kLin + t] = 0.0f;
+    auto fetch = [&](int b, float (&v)[2]) {
+        v[0] = b < nb ? x[(size_t)b * kLin + t] : 0.0f;
+        v[1] = b < nb ? x[(size_t)b * kLin + 256 + t] : 0.0f;
+    };
+    float xn[2];
+    fetch(blockIdx.x, xn);
     for (int e = t; e < kCh * kTaps; e += blockDim.x) sw[e] = 0.0f;
     if (t < kCh) sb[t] = 0.0f;
-    float aw[8][kTaps], ab[8];
+    float w[4][kTaps], bs[4], aw[4][kTaps], ab[4];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
+    for (int e = 0; e < 4; ++e) {
         ab[e] = 0.0f;
+        bs[e] = bias[c * 4 + e];
 #pragma unroll
-        for (int k = 0; k < kTaps; ++k) aw[e][k] = 0.0f;
-    }
-    for (int b = blockIdx.x; b < nb; b += gridDim.x) {
-        __syncthreads();  // the previous trace's reads are done
-        for (int q = t; q < kLin + 8; q += blockDim.x) {
-            const int src = q - 2;
-            xs[q] = (src >= 0 && src < kLin) ? __bfloat162float(x[(size_t)b * kLin + src]) : 0.0f;
+        for (int k = 0; k < kTaps; ++k) {
+            aw[e][k] = 0.0f;
+            w[e][k] = __bfloat162float(W[(c * 4 + e) * kTaps + k]);
         }
-        __syncthreads();
-#pragma unroll 1
-        for (int i = 0; i < 8; i += 2) {
-            float4 a[2][2], pr[2][2];
+    }
+    float4 an[4];
+    if ((int)blockIdx.x < nb) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const size_t row = (size_t)b * kLout + p0 + i + h;
-                const float4 *da = reinterpret_cast<const float4 *>(dact + row * kCh + c * 8);
-                const float4 *pa = reinterpret_cast<const float4 *>(pre + row * kCh + c * 8);
-                a[h][0] = __ldg(da);
-                a[h][1] = __ldg(da + 1);
-                pr[h][0] = __ldg(pa);
-                pr[h][1] = __ldg(pa + 1);
+        for (int h = 0; h < 4; ++h)
+            an[h] = __ldcs(reinterpret_cast<const float4 *>(dact + (size_t)blockIdx.x * kLout * kCh) + c +
+                           (p0 + 16 * h) * (kCh / 4));
+    }
+    int u = 0;
+    for (int b = blockIdx.x; b < nb; b += gridDim.x, u ^= 1) {
+        // (the barrier of the trace before was after the last reads of this buffer)
+        float *const xs = xs2[u];
+        xs[2 + t] = __bfloat162float(__float2bfloat16(xn[0]));
+        xs[258 + t] = __bfloat162float(__float2bfloat16(xn[1]));
+        __syncthreads();
+        fetch(b + (int)gridDim.x, xn);
+        const float4 *const da = reinterpret_cast<const float4 *>(dact + (size_t)b * kLout * kCh) + c;
+#pragma unroll 1
+        for (int i = 0; i < kLout / 16; i += 4) {
+            // the next four positions' loads (the next trace's first ones at the
+            // end of this one) go out before this four's arithmetic
+            float4 a[4];
+#pragma unroll
+            for (int h = 0; h < 4; ++h) a[h] = an[h];
+            const bool same = i + 4 < kLout / 16;
+            if (same || b + (int)gridDim.x < nb) {
+                const float4 *const dn = same ? da + 16 * (i + 4) * (kCh / 4)
+                                              : da + (size_t)gridDim.x * kLout * (kCh / 4);
+#pragma unroll
+                for (int h = 0; h < 4; ++h) an[h] = __ldcs(dn + (p0 + 16 * h) * (kCh / 4));
             }
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int p = p0 + i + h;
+            for (int h = 0; h < 4; ++h) {
+                const int p = p0 + 16 * (i + h);
                 float xv[kTaps];
 #pragma unroll
                 for (int k = 0; k < kTaps; ++k) xv[k] = xs[2 * p + k];  // x[2p + k - 2]
-                const float av[8] = {a[h][0].x, a[h][0].y, a[h][0].z, a[h][0].w,
-                                     a[h][1].x, a[h][1].y, a[h][1].z, a[h][1].w};
-                const float pv[8] = {pr[h][0].x, pr[h][0].y, pr[h][0].z, pr[h][0].w,
-                                     pr[h][1].x, pr[h][1].y, pr[h][1].z, pr[h][1].w};
+                const float av[4] = {a[h].x, a[h].y, a[h].z, a[h].w};
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const float d = av[e] * gelu_grad_t(pv[e]);
+                for (int e = 0; e < 4; ++e) {
+                    float acc = 0.0f;
+#pragma unroll
+                    for (int k = 0; k < kTaps; ++k) acc = fmaf(w[e][k], xv[k], acc);
+                    const float d = av[e] * gelu_grad_t(acc + bs[e]);
                     ab[e] += d;
                     const float db = __bfloat162float(__float2bfloat16(d));
 #pragma unroll
@@ -480,24 +531,20 @@ __global__ void __launch_bounds__(256) conv0_back_kernel(const float *__restrict
             }
         }
     }
-    // lanes l, l ^ 8, l ^ 16, l ^ 24 hold the same channels
+    // lanes l and l ^ 16 hold the same channels
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        ab[e] += __shfl_xor_sync(0xffffffffu, ab[e], 8);
+    for (int e = 0; e < 4; ++e) {
         ab[e] += __shfl_xor_sync(0xffffffffu, ab[e], 16);
 #pragma unroll
-        for (int k = 0; k < kTaps; ++k) {
-            aw[e][k] += __shfl_xor_sync(0xffffffffu, aw[e][k], 8);
-            aw[e][k] += __shfl_xor_sync(0xffffffffu, aw[e][k], 16);
-        }
+        for (int k = 0; k < kTaps; ++k) aw[e][k] += __shfl_xor_sync(0xffffffffu, aw[e][k], 16);
     }
     __syncthreads();
-    if ((t & 31) < 8) {
+    if ((t & 31) < 16) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            atomicAdd(&sb[c * 8 + e], ab[e]);
+        for (int e = 0; e < 4; ++e) {
+            atomicAdd(&sb[c * 4 + e], ab[e]);
 #pragma unroll
-            for (int k = 0; k < kTaps; ++k) atomicAdd(&sw[(c * 8 + e) * kTaps + k], aw[e][k]);
+            for (int k = 0; k < kTaps; ++k) atomicAdd(&sw[(c * 4 + e) * kTaps + k], aw[e][k]);
         }
     }
     __syncthreads();
@@ -529,8 +576,8 @@ template <int LOUT>
 __global__ void __launch_bounds__(kFwdThreads, 1)
     conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap xmap, int nb,
                        const __nv_bfloat16 *__restrict__ W, const float *__restrict__ bias,
-                       float *__restrict__ pre, __nv_bfloat16 *__restrict__ out,
-                       uint32_t *status) {
+                       const __grid_constant__ CUtensorMap pmap,
+                       const __grid_constant__ CUtensorMap omap, uint32_t *status) {
     constexpr int tpt = kRowsPerTile / LOUT;
     extern __shared__ uint8_t dsm[];
     const uint32_t raw = smem_u32(dsm);
@@ -589,18 +636,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     int j = 0, last_load = (int)blockIdx.x < ntiles ? 0 : -1;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++j) {
         const int s = j & 1;
-        if (j > 0) {
-            // every thread is done with the previous tile's accumulator
-            tc_fence_before();
-            __syncthreads();
-            tc_fence_after();
-        }
         if (tid == 0) {
-            // buffer s ^ 1 was last read by tile j - 1's MMAs, complete
-            if (t + (int)gridDim.x < ntiles) {
-                load(t + gridDim.x, s ^ 1);
-                last_load = j + 1;
-            }
             if (mbar_wait(sBar + 16u + 8u * (uint32_t)s, (uint32_t)(j >> 1) & 1u)) {
                 tc_fence_after();
                 const uint32_t a0 = sA + (uint32_t)s * kFwdA;
@@ -620,6 +656,13 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
                 "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                     sBar + 8u * (uint32_t)s)
                 : "memory");
+            // buffer s ^ 1: tile j - 1's MMAs are complete, and its outputs,
+            // staged there, have been read by their stores
+            if (t + (int)gridDim.x < ntiles) {
+                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                load(t + gridDim.x, s ^ 1);
+                last_load = j + 1;
+            }
         }
         const bool got = mbar_wait(sBar + 8u * (uint32_t)s, (uint32_t)(j >> 1) & 1u);
         tc_fence_after();
@@ -630,22 +673,43 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
         uint32_t v[16];
         tmem_ld16(tmem + ((uint32_t)(32 * lg) << 16) + 64u * (uint32_t)s + 16u * (uint32_t)qq, v);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        const int grow = t * kRowsPerTile + 32 * lg + lane;
-        if (grow < nrows) {
-            float4 *po = reinterpret_cast<float4 *>(pre + (size_t)grow * kCh + 16 * qq);
-            uint4 *ao = reinterpret_cast<uint4 *>(out + (size_t)grow * kCh + 16 * qq);
+        // a lane holds 16 channels of a row: the tile goes through the operand
+        // buffer its MMAs have just read and leaves as three TMA stores (FP32
+        // pre-activations in two 32-channel halves, BF16 outputs); rows past
+        // the batch are out of the tensors
+        {
+            const uint32_t q = (uint32_t)(32 * lg + lane);
+            const uint32_t st = sA + (uint32_t)s * kFwdA;
+            const uint32_t ph = st + (uint32_t)(qq >> 1) * 16384u, c0 = 4u * (uint32_t)(qq & 1);
             float y[16];
 #pragma unroll
             for (int e = 0; e < 16; ++e) y[e] = __uint_as_float(v[e]) + bq[e];
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                po[e] = make_float4(y[4 * e], y[4 * e + 1], y[4 * e + 2], y[4 * e + 3]);
-            ao[0] = make_uint4(pack_bf16(gelu_t(y[0]), gelu_t(y[1])), pack_bf16(gelu_t(y[2]), gelu_t(y[3])),
-                               pack_bf16(gelu_t(y[4]), gelu_t(y[5])), pack_bf16(gelu_t(y[6]), gelu_t(y[7])));
-            ao[1] = make_uint4(pack_bf16(gelu_t(y[8]), gelu_t(y[9])), pack_bf16(gelu_t(y[10]), gelu_t(y[11])),
-                               pack_bf16(gelu_t(y[12]), gelu_t(y[13])), pack_bf16(gelu_t(y[14]), gelu_t(y[15])));
+                st_shared_v4(ph + sw_chunk(q, c0 + (uint32_t)e),
+                             make_uint4(__float_as_uint(y[4 * e]), __float_as_uint(y[4 * e + 1]),
+                                        __float_as_uint(y[4 * e + 2]), __float_as_uint(y[4 * e + 3])));
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                st_shared_v4(st + 32768u + sw_chunk(q, 2u * (uint32_t)qq + (uint32_t)e),
+                             make_uint4(pack_bf16(gelu_t(y[8 * e]), gelu_t(y[8 * e + 1])),
+                                        pack_bf16(gelu_t(y[8 * e + 2]), gelu_t(y[8 * e + 3])),
+                                        pack_bf16(gelu_t(y[8 * e + 4]), gelu_t(y[8 * e + 5])),
+                                        pack_bf16(gelu_t(y[8 * e + 6]), gelu_t(y[8 * e + 7]))));
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        // every thread is done with this tile's accumulator and has written
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        if (tid == 0) {
+            const uint32_t st = sA + (uint32_t)s * kFwdA;
+            tma_store_2d(&pmap, 0, t * kRowsPerTile, st);
+            tma_store_2d(&pmap, 32, t * kRowsPerTile, st + 16384u);
+            tma_store_2d(&omap, 0, t * kRowsPerTile, st + 32768u);
         }
     }
+    if (tid == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     if (!ok && tid == 0) {
         atomicOr(status, PCHASE_DEV_TIMEOUT);
         // loads and MMAs still in flight land before the CTA leaves
@@ -899,6 +963,23 @@ cudaError_t launch_tc_gemm(const TcGemm &g, int slices, cudaStream_t st) {
 
 }  // namespace
 
+// a row-major FP32 (BF16 when bf16) tensor written in boxes of 128-byte rows,
+// 128-byte swizzle in shared memory
+static bool store_map(void *p, bool bf16, int rank, const cuuint64_t *dims, const cuuint64_t *strides,
+                      const cuuint32_t *box, CUtensorMap *map) {
+    const PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
+    if (!encode || (reinterpret_cast<uintptr_t>(p) & 15)) return false;
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return encode(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+                  (cuuint32_t)rank, p, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+static bool fp32_store_map(float *p, int rank, const cuuint64_t *dims, const cuuint64_t *strides,
+                           const cuuint32_t *box, CUtensorMap *map) {
+    return store_map(p, false, rank, dims, strides, box, map);
+}
+
 // x [nb][2 lout][64] BF16 as the 4-D tensor (channel, parity, pair, trace)
 // with boxes of 64 channels x 1 parity x lout pairs x (128 / lout) traces,
 // 128-byte swizzle: the rows of one parity plane of a 128-row tile
@@ -923,9 +1004,17 @@ cudaError_t conv_back_tc(const float *dact, const float *pre, const __nv_bfloat1
     if (nb <= 0) return cudaSuccess;
     if (lout != 128 && lout != 64 && lout != 32) return cudaErrorInvalidValue;
     if (reinterpret_cast<uintptr_t>(x) & 15) return cudaErrorInvalidValue;
-    alignas(64) CUtensorMap map;
+    alignas(64) CUtensorMap map, dmap;
     const cudaError_t me = x_plane_map(x, nb, lout, &map);
     if (me != cudaSuccess) return me;
+    {
+        // dx [nb][2 lout][64] FP32 as (channel, parity, pair): the rows of a
+        // tile, 32 channels of one parity a box
+        const cuuint64_t dims[3] = {(cuuint64_t)kCh, 2, (cuuint64_t)nb * lout};
+        const cuuint64_t strides[2] = {kCh * 4, 2 * kCh * 4};
+        const cuuint32_t box[3] = {32, 1, (cuuint32_t)kRowsPerTile};
+        if (!fp32_store_map(dx, 3, dims, strides, box, &dmap)) return cudaErrorInvalidValue;
+    }
     static bool attr = false;
     if (!attr) {
         for (auto k : {conv_back_tc_kernel<128>, conv_back_tc_kernel<64>, conv_back_tc_kernel<32>}) {
@@ -938,19 +1027,19 @@ cudaError_t conv_back_tc(const float *dact, const float *pre, const __nv_bfloat1
     const int ntiles = (nb * lout + kRowsPerTile - 1) / kRowsPerTile;
     const int grid = std::max(1, std::min(ntiles, sms));
     if (lout == 128)
-        conv_back_tc_kernel<128><<<grid, kBackThreads, kBackSmem, st>>>(dact, pre, map, W, nb, gW, gb, dx, status);
+        conv_back_tc_kernel<128><<<grid, kBackThreads, kBackSmem, st>>>(dact, pre, map, W, nb, gW, gb, dmap, status);
     else if (lout == 64)
-        conv_back_tc_kernel<64><<<grid, kBackThreads, kBackSmem, st>>>(dact, pre, map, W, nb, gW, gb, dx, status);
+        conv_back_tc_kernel<64><<<grid, kBackThreads, kBackSmem, st>>>(dact, pre, map, W, nb, gW, gb, dmap, status);
     else
-        conv_back_tc_kernel<32><<<grid, kBackThreads, kBackSmem, st>>>(dact, pre, map, W, nb, gW, gb, dx, status);
+        conv_back_tc_kernel<32><<<grid, kBackThreads, kBackSmem, st>>>(dact, pre, map, W, nb, gW, gb, dmap, status);
     return cudaGetLastError();
 }
 
-cudaError_t conv0_back(const float *dact, const float *pre, const __nv_bfloat16 *x, int nb,
-                       float *gW, float *gb, int sms, cudaStream_t st) {
+cudaError_t conv0_back(const float *dact, const float *x, const __nv_bfloat16 *W, const float *bias,
+                       int nb, float *gW, float *gb, int sms, cudaStream_t st) {
     if (nb <= 0) return cudaSuccess;
-    const int grid = std::max(1, std::min(nb, sms * 4));
-    conv0_back_kernel<<<grid, 256, 0, st>>>(dact, pre, x, nb, gW, gb);
+    const int grid = std::max(1, std::min(nb, sms * 2));
+    conv0_back_kernel<<<grid, 256, 0, st>>>(dact, x, W, bias, nb, gW, gb);
     return cudaGetLastError();
 }
 
@@ -993,9 +1082,16 @@ cudaError_t conv_fwd_tc(const __nv_bfloat16 *x, int nb, int lout, const __nv_bfl
     if (lout != 128 && lout != 64 && lout != 32) return cudaErrorInvalidValue;
     if ((reinterpret_cast<uintptr_t>(x) & 15) || (reinterpret_cast<uintptr_t>(W) & 15))
         return cudaErrorInvalidValue;
-    alignas(64) CUtensorMap map;
+    alignas(64) CUtensorMap map, pmap, omap;
     const cudaError_t me = x_plane_map(x, nb, lout, &map);
     if (me != cudaSuccess) return me;
+    {
+        const cuuint64_t dims[2] = {(cuuint64_t)kCh, (cuuint64_t)nb * lout};
+        const cuuint64_t ps[1] = {kCh * 4}, os[1] = {kCh * 2};
+        const cuuint32_t pbox[2] = {32, (cuuint32_t)kRowsPerTile}, obox[2] = {64, (cuuint32_t)kRowsPerTile};
+        if (!store_map(pre, false, 2, dims, ps, pbox, &pmap) || !store_map(out, true, 2, dims, os, obox, &omap))
+            return cudaErrorInvalidValue;
+    }
     static bool attr = false;
     if (!attr) {
         for (auto k : {conv_fwd_tc_kernel<128>, conv_fwd_tc_kernel<64>, conv_fwd_tc_kernel<32>}) {
@@ -1008,11 +1104,11 @@ cudaError_t conv_fwd_tc(const __nv_bfloat16 *x, int nb, int lout, const __nv_bfl
     const int ntiles = (nb * lout + kRowsPerTile - 1) / kRowsPerTile;
     const int grid = std::max(1, std::min(ntiles, sms));
     if (lout == 128)
-        conv_fwd_tc_kernel<128><<<grid, kFwdThreads, kFwdSmem, st>>>(map, nb, W, bias, pre, out, status);
+        conv_fwd_tc_kernel<128><<<grid, kFwdThreads, kFwdSmem, st>>>(map, nb, W, bias, pmap, omap, status);
     else if (lout == 64)
-        conv_fwd_tc_kernel<64><<<grid, kFwdThreads, kFwdSmem, st>>>(map, nb, W, bias, pre, out, status);
+        conv_fwd_tc_kernel<64><<<grid, kFwdThreads, kFwdSmem, st>>>(map, nb, W, bias, pmap, omap, status);
     else
-        conv_fwd_tc_kernel<32><<<grid, kFwdThreads, kFwdSmem, st>>>(map, nb, W, bias, pre, out, status);
+        conv_fwd_tc_kernel<32><<<grid, kFwdThreads, kFwdSmem, st>>>(map, nb, W, bias, pmap, omap, status);
     return cudaGetLastError();
 }
 
