@@ -529,8 +529,8 @@ int pchase::set_last_error(int code, const char *msg) { return fail(code, msg); 
 struct pchase_sim_plan {
     std::vector<SimItem> items;
     SlotLayout layout{};
-    SlotLayout ulayout{};  // layout with the homes of a run whose analytic uniform
-                           // chains are not the units' work
+    SlotLayout ulayout{};  // layout with the slot mix and homes of a run whose analytic
+                           // uniform chains are not the units' work
     SlotLayout jumbo{};   // items too large for the main slot mix (nwarps 0: none)
     SlotLayout gpool{};   // units with global set state, one pool region per warp
     uint32_t pool_warps = 0;    // warps (and state regions) of the pool launch
@@ -553,7 +553,7 @@ struct pchase_sim_plan {
     double est_sum = 0.0, est_critical = 0.0, est_target = 0.0, est_max_unit = 0.0;
     bool filtered = false;  // every unit queued (pchase_sim_run_filtered)
     // runtime state, set on the first run
-    int device = -1, sms = 0, grid = 0, jgrid = 0, ggrid = 0;
+    int device = -1, sms = 0, grid = 0, ugrid = 0, jgrid = 0, ggrid = 0;
     uint64_t n_isolated = 0;  // units given an SM of their own (in the jumbo launch)
     uint64_t n_gmem = 0;        // units with their set state in global memory
     uint64_t gstate_bytes = 0;  // their state area (workspace, after the pooled offsets)
@@ -798,9 +798,13 @@ int plan_runtime(pchase_sim_plan *p) {
         p->grid = (int)std::max<uint64_t>(
             1, std::min<uint64_t>((uint64_t)per * (p->sms - jsms), p->n_units - p->n_jumbo));
         const uint32_t sites = (uint32_t)std::max(1, std::min(p->grid, p->sms - jsms));
-        p->ulayout = p->layout;
         set_homes(p->layout, p->gwork_main, p->affinity, sites);
-        set_homes(p->ulayout, p->gwork_live, p->affinity, sites);
+        const int uper = sim_max_ctas_per_sm(p->ulayout);
+        if (uper <= 0) return fail(PCHASE_ECUDA, "simulator kernel cannot be resident");
+        p->ugrid = (int)std::max<uint64_t>(
+            1, std::min<uint64_t>((uint64_t)uper * (p->sms - jsms), p->n_units - p->n_jumbo));
+        set_homes(p->ulayout, p->gwork_live, p->affinity,
+                  (uint32_t)std::max(1, std::min(p->ugrid, p->sms - jsms)));
     }
     if (p->jumbo.nwarps) {
         const int per = sim_max_ctas_per_sm(p->jumbo);
@@ -923,7 +927,8 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
         PCHASE_CUDA(cudaEventRecord(p->join, p->side), "cudaEventRecord");
     }
     if (units && p->layout.nwarps)
-        PCHASE_CUDA(launch_sim(items, uni ? p->ulayout : p->layout, queues, p->grid, o, st),
+        PCHASE_CUDA(launch_sim(items, uni ? p->ulayout : p->layout, queues, uni ? p->ugrid : p->grid, o,
+                               st),
                     "simulator launch");
     if (jside) PCHASE_CUDA(cudaStreamWaitEvent(st, p->join, 0), "cudaStreamWaitEvent");
     if (units && p->gpool.nwarps)
@@ -1050,6 +1055,8 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
     }
     uint64_t word = 0;
     double total = 0.0;
+    // done outside the units in most runs (an analytic uniform chain)
+    auto certain = [](const SimItem &it) { return !it.idx && ((it.lsh >> kUniformBit) & 1u); };
     const uint32_t max_split = std::max<uint32_t>(1, tn.max_split);
     for (uint64_t i = 0; i < n_items; ++i) {
         uint32_t g, t;
@@ -1471,7 +1478,8 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
     SlotLayout &L = p->layout;
     memset(&L, 0, sizeof L);
     std::vector<double> work(ncap, 0.0);
-    std::vector<double> gwork[kUnitGroups], glive[kUnitGroups];
+    // (live: what analytic uniform chains leave to the units)
+    std::vector<double> gwork[kUnitGroups], glive[kUnitGroups], wlive(ncap, 0.0);
     for (auto &v : gwork) v.assign(ncap, 0.0);
     for (auto &v : glive) v.assign(ncap, 0.0);
     uint32_t nclass = 0;
@@ -1500,8 +1508,10 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
                         ++count;
                         work[q] += cost[order[k]];
                         gwork[g][q] += cost[order[k]];
-                        const SimItem &it = items[order[k]];
-                        if (it.idx || !((it.lsh >> kUniformBit) & 1u)) glive[g][q] += cost[order[k]];
+                        if (!certain(items[order[k]])) {
+                            glive[g][q] += cost[order[k]];
+                            wlive[q] += cost[order[k]];
+                        }
                     }
                 L.cls_first[g][q] = (uint32_t)(count ? first : 0);
                 L.cls_count[g][q] = (uint32_t)count;
@@ -1513,7 +1523,7 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
         // are added one at a time to minimise the estimated makespan
         // max_q (work of classes >= q) / (slots that can hold class q), since a
         // slot also serves every smaller class.
-        std::vector<uint32_t> caps(nclass), slots(nclass, 0);
+        std::vector<uint32_t> caps(nclass);
         for (uint32_t q = 0; q < nclass; ++q) caps[q] = kCaps[present[q]];
         p->class_caps = caps;
         const uint32_t budget = tn.smem_budget_bytes;
@@ -1521,66 +1531,110 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
         for (uint32_t q = 0; q < nclass; ++q)
             if (caps[q] * 2 <= budget) main_top = (int)q;
         p->jumbo_first_class = (uint32_t)(main_top + 1);
-        auto makespan = [&](const std::vector<uint32_t> &sl) {
-            double worst = 0.0, wsum = 0.0;
-            uint32_t ssum = 0;
-            for (int q = main_top; q >= 0; --q) {
-                wsum += work[q];
-                ssum += sl[q];
-                if (wsum > 0.0) worst = std::max(worst, ssum ? wsum / ssum : 1e300);
+        auto slot_mix = [&](SlotLayout &L, const std::vector<double> &work, int main_top) {
+            std::vector<uint32_t> slots(nclass, 0);
+            auto makespan = [&](const std::vector<uint32_t> &sl) {
+                double worst = 0.0, wsum = 0.0;
+                uint32_t ssum = 0;
+                for (int q = main_top; q >= 0; --q) {
+                    wsum += work[q];
+                    ssum += sl[q];
+                    if (wsum > 0.0) worst = std::max(worst, ssum ? wsum / ssum : 1e300);
+                }
+                return worst;
+            };
+            uint32_t used = 0, nw = 0;
+            if (main_top >= 0) {
+                // the least makespan t whose slots fit: from the largest class
+                // down, a class gets as many as bring the work of the classes
+                // so far under t per slot
+                auto fill = [&](double t) {
+                    std::fill(slots.begin(), slots.end(), 0u);
+                    slots[main_top] = 1;
+                    used = caps[main_top];
+                    nw = 1;
+                    double wsum = 0.0;
+                    for (int q = main_top; q >= 0; --q) {
+                        wsum += work[q];
+                        const double need = std::ceil(wsum / t - 1e-9);
+                        while (nw < need) {
+                            if (nw == tn.max_warps_per_cta || used + caps[q] > budget) return false;
+                            slots[q] += 1;
+                            used += caps[q];
+                            nw += 1;
+                        }
+                    }
+                    return true;
+                };
+                double lo = 0.0, hi = 0.0;
+                for (int q = main_top; q >= 0; --q) hi += work[q];
+                if (hi > 0.0) {
+                    for (int k = 0; k < 40; ++k) {
+                        const double mid = 0.5 * (lo + hi);
+                        (fill(mid) ? hi : lo) = mid;
+                    }
+                }
+                fill(hi > 0.0 ? hi : 1.0);
+                // extra large slots (big_slots - 1 of them, each the largest class
+                // that leaves half of what is left), for whoever asks for them
+                for (uint32_t k = 1; k < tn.big_slots && nw < tn.max_warps_per_cta; ++k) {
+                    int q2 = -1;
+                    for (int q = main_top; q >= 0; --q)
+                        if (caps[q] <= (budget - used) / 2 && work[q] > 0.0) { q2 = q; break; }
+                    if (q2 < 0) break;
+                    slots[q2] += 1;
+                    used += caps[q2];
+                    nw += 1;
+                }
+                while (nw < tn.max_warps_per_cta) {
+                    int best = -1;
+                    double best_ms = makespan(slots);
+                    for (int q = 0; q <= main_top; ++q) {
+                        if (used + caps[q] > budget) continue;
+                        slots[q] += 1;
+                        const double ms = makespan(slots);
+                        slots[q] -= 1;
+                        if (ms < best_ms * (1.0 - 1e-9)) { best_ms = ms; best = q; }
+                    }
+                    if (best < 0) {
+                        // no slot lowers the makespan, which one class sets: the
+                        // one that most lowers the other classes' (their sum of
+                        // squares; the smallest class's slots, taken here before,
+                        // stand idle once its units are done)
+                        double least = 1e300;
+                        for (int q = 0; q <= main_top; ++q) {
+                            if (used + caps[q] > budget) continue;
+                            slots[q] += 1;
+                            double sum = 0.0, wsum = 0.0;
+                            uint32_t ssum = 0;
+                            for (int r = main_top; r >= 0; --r) {
+                                wsum += work[r];
+                                ssum += slots[r];
+                                sum += ssum ? (wsum / ssum) * (wsum / ssum) : 0.0;
+                            }
+                            slots[q] -= 1;
+                            // (slots of classes without units hold the smaller ones')
+                            if (sum < least) { least = sum; best = q; }
+                        }
+                        if (best < 0) break;
+                    }
+                    slots[best] += 1;
+                    used += caps[best];
+                    nw += 1;
+                }
             }
-            return worst;
+            uint32_t off = 0, w = 0;
+            for (int q = main_top; q >= 0; --q)
+                for (uint32_t k = 0; k < slots[q]; ++k) {
+                    L.warp_class[w] = (uint32_t)q;
+                    L.warp_off[w] = off;
+                    off += caps[q];
+                    ++w;
+                }
+            L.nwarps = w;
+            L.smem_bytes = off;
         };
-        uint32_t used = 0, nw = 0;
-        if (main_top >= 0) {
-            slots[main_top] = 1;
-            used = caps[main_top];
-            nw = 1;
-            // extra large slots first (big_slots - 1 of them, each the largest
-            // class that leaves half of what is left to the greedy fill): the
-            // greedy alone spends the budget on small slots before the large
-            // classes' work, which only the first slot holds, would pay
-            for (uint32_t k = 1; k < tn.big_slots && nw < tn.max_warps_per_cta; ++k) {
-                int q2 = -1;
-                for (int q = main_top; q >= 0; --q)
-                    if (caps[q] <= (budget - used) / 2 && work[q] > 0.0) { q2 = q; break; }
-                if (q2 < 0) break;
-                slots[q2] += 1;
-                used += caps[q2];
-                nw += 1;
-            }
-            while (nw < tn.max_warps_per_cta) {
-                int best = -1;
-                double best_ms = makespan(slots);
-                for (int q = 0; q <= main_top; ++q) {
-                    if (used + caps[q] > budget) continue;
-                    slots[q] += 1;
-                    const double ms = makespan(slots);
-                    slots[q] -= 1;
-                    if (ms < best_ms * (1.0 - 1e-9)) { best_ms = ms; best = q; }
-                }
-                if (best < 0) {
-                    // no slot lowers the makespan: spend what is left on the
-                    // smallest class with work (more warps to hide latency)
-                    for (int q = 0; q <= main_top; ++q)
-                        if (work[q] > 0.0 && used + caps[q] <= budget) { best = q; break; }
-                    if (best < 0) break;
-                }
-                slots[best] += 1;
-                used += caps[best];
-                nw += 1;
-            }
-        }
-        uint32_t off = 0, w = 0;
-        for (int q = main_top; q >= 0; --q)
-            for (uint32_t k = 0; k < slots[q]; ++k) {
-                L.warp_class[w] = (uint32_t)q;
-                L.warp_off[w] = off;
-                off += caps[q];
-                ++w;
-            }
-        L.nwarps = w;
-        L.smem_bytes = off;
+        slot_mix(L, work, main_top);
         // first-pop stagger: 4 us per slot for plans of long units, a
         // 2000th of the longest unit's estimate below that
         L.stagger_ns = (uint32_t)std::min(4000.0, p->est_max_unit / 2000.0);
@@ -1590,6 +1644,17 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
                 p->gwork_live[g] += glive[g][q];
             }
         p->affinity = tn.kind_affinity != 0;
+        // The same for runs whose analytic uniform chains are done elsewhere:
+        // their estimates would buy slots that stand idle (the 512-point plan:
+        // 448 chains beside 64 index arrays whose line tables need 70-110 KB
+        // each; 3.6 warps active per SM, 14.1 ms a table of 64 candidates; 10.5 ms
+        // with this and the slots above).
+        p->ulayout = L;
+        {
+            double live = 0.0;
+            for (int q = 0; q <= main_top; ++q) live += wlive[q];
+            if (live > 0.0) slot_mix(p->ulayout, wlive, main_top);
+        }
         // jumbo layout: one warp, the largest jumbo arena; serves jumbo classes
         SlotLayout &J = p->jumbo;
         memset(&J, 0, sizeof J);
@@ -1809,6 +1874,13 @@ size_t pchase_sim_plan_describe(const pchase_sim_plan *plan, char *buf, size_t b
             snprintf(tmp, sizeof tmp, " uniform=%llu,%zu", (unsigned long long)plan->n_uniform,
                      plan->utasks.size());
             d += tmp;
+            d += " live_slots=";
+            for (uint32_t w = 0; w < plan->ulayout.nwarps; ++w) {
+                const uint32_t next = w + 1 < plan->ulayout.nwarps ? plan->ulayout.warp_off[w + 1]
+                                                                   : plan->ulayout.smem_bytes;
+                snprintf(tmp, sizeof tmp, "%s%u", w ? "," : "", next - plan->ulayout.warp_off[w]);
+                d += tmp;
+            }
         }
         if (!plan->jobs.empty()) {
             // head streams: split items, their parts, entries (8 bytes each);
