@@ -126,6 +126,9 @@ constexpr double kAffinityMinNsPerSm = 20.0e6;
 // launch): the costliest kIsolateMax within kIsolateFrac of the costliest.
 constexpr double kIsolateFrac = 0.6;
 constexpr size_t kIsolateMax = 12;
+// ... in plans whose longest unit takes this long: a second launch beside the
+// main one, forked and joined, costs the host and the GPU some 6 us.
+constexpr double kIsolateMinNs = 1.0e5;
 // Way scans over set state in global memory (L2-resident) against shared memory.
 constexpr double kGlobalScanFactor = 2.0;
 // A time part's backward read of 32 accesses while it rebuilds the recency
@@ -848,8 +851,7 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
     // uniform chains, unless the run filters accesses, records a timeline of
     // the units, or may stop its candidates early
     const bool uni = p->uniform && !o.filter && !o.timeline && (!o.dist || o.stop_above == ~0ull);
-    PCHASE_CUDA(cudaMemsetAsync(w, 0, kQueueHeader + (uni ? 4ull * p->n_trace : 0), st),
-                "cudaMemsetAsync(queues)");
+    if (!uni) PCHASE_CUDA(cudaMemsetAsync(w, 0, kQueueHeader, st), "cudaMemsetAsync(queues)");
     if (!o.status) o.status = reinterpret_cast<uint32_t *>(w + kStatusOffset);
     o.gstate = w + p->off_gstate;
     const SimItem *items = reinterpret_cast<const SimItem *>(w + p->off_items);
@@ -860,10 +862,10 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
         o.uniform_bad = bad;
         o.uniform_live = reinterpret_cast<uint32_t *>(w + kLiveOffset);
         PCHASE_CUDA(launch_uniform_prep(items, reinterpret_cast<const uint32_t *>(w + p->off_tunit),
-                                        p->n_trace, p->n_explicit, p->n_items, o.miss_counts, bad,
-                                        p->sms, st),
+                                        p->n_trace, p->n_explicit, p->max_trace_len, p->n_items,
+                                        o.miss_counts, reinterpret_cast<uint32_t *>(w), bad, p->sms, st),
                     "uniform check");
-        PCHASE_CUDA(launch_uniform_out(items, p->n_units, p->sms, o,
+        PCHASE_CUDA(launch_uniform_out(items, p->n_units, p->max_trace_len, p->sms, o,
                                        reinterpret_cast<uint32_t *>(w + kLiveOffset), st),
                     "uniform words");
         const UniformTask *const tasks = reinterpret_cast<const UniformTask *>(w + p->off_utasks);
@@ -1386,7 +1388,7 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
             if (cost[i] >= kIsolateFrac * cmax) top.push_back(i);
         std::sort(top.begin(), top.end(), [&](uint64_t x, uint64_t y) { return cost[x] > cost[y]; });
         if (top.size() > kIsolateMax) top.resize(kIsolateMax);
-        if (csum > 64.0 * cmax) {
+        if (csum > 64.0 * cmax && cmax >= kIsolateMinNs) {
             for (uint64_t i : top) cls[i] = ncap - 1;
             p->n_isolated = top.size();
         }

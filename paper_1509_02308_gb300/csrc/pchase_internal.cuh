@@ -294,13 +294,15 @@ int sim_max_ctas_per_sm(const SlotLayout &layout);
 // current device: once per plan, with the same constants from every plan.
 cudaError_t prepare_sim(uint32_t smem_bytes);
 cudaError_t prepare_uniform(uint32_t smem_bytes);
-// Uniform chains: traces checked and counts cleared, the words of every item,
-// the tasks of one shared-memory class.
+// Uniform chains: traces checked, the workspace's counters (head: kQueueHeader
+// bytes, bad right behind them) and the counts cleared; the words of every item;
+// the tasks of one shared-memory class.  max_len: the longest trace.
 cudaError_t launch_uniform_prep(const SimItem *items, const uint32_t *trace_unit, uint32_t n_trace,
-                                uint64_t n_explicit, uint64_t n_items, uint64_t *counts,
-                                uint32_t *bad, int sms, cudaStream_t st);
-cudaError_t launch_uniform_out(const SimItem *items, uint64_t n_units, int sms, const SimOut &out,
-                               uint32_t *live, cudaStream_t st);
+                                uint64_t n_explicit, uint64_t max_len, uint64_t n_items,
+                                uint64_t *counts, uint32_t *head, uint32_t *bad, int sms,
+                                cudaStream_t st);
+cudaError_t launch_uniform_out(const SimItem *items, uint64_t n_units, uint64_t max_len, int sms,
+                               const SimOut &out, uint32_t *live, cudaStream_t st);
 cudaError_t launch_uniform_play(const SimItem *items, const UniformTask *tasks, uint32_t n_tasks,
                                 uint32_t smem_bytes, const SimOut &out, cudaStream_t st);
 // The head streams of a plan's split items (three launches on `st`).

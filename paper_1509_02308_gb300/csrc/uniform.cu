@@ -178,9 +178,11 @@ __global__ void __launch_bounds__(256) uniform_prep_kernel(const SimItem *__rest
                                                            const uint32_t *__restrict__ trace_unit,
                                                            uint32_t n_trace, uint32_t parts,
                                                            uint64_t n_items, uint64_t *counts,
-                                                           uint32_t *bad) {
+                                                           uint32_t *bad, uint32_t *head) {
     const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     const uint64_t nthr = (uint64_t)gridDim.x * blockDim.x;
+    if (head)  // the workspace's counters, unless a memset cleared them
+        for (uint64_t i = tid; i < kQueueHeader / 4; i += nthr) head[i] = 0;
     if (counts)
         for (uint64_t i = tid; i < 2 * n_items; i += nthr) counts[i] = 0;
     const uint32_t lane = threadIdx.x & 31u;
@@ -188,7 +190,10 @@ __global__ void __launch_bounds__(256) uniform_prep_kernel(const SimItem *__rest
     for (uint64_t task = tid >> 5; task < tasks; task += nthr >> 5) {
         const uint32_t tr = (uint32_t)(task / parts), part = (uint32_t)(task % parts);
         const uint32_t unit = trace_unit[tr];
-        if (unit == 0xFFFFFFFFu) continue;
+        if (unit == 0xFFFFFFFFu) {
+            if (parts == 1u && lane == 0) bad[tr] = 0;
+            continue;
+        }
         const SimItem &it = items[unit];
         const uint32_t *const p = it.idx;
         const uint32_t len = it.len, s = it.stride;
@@ -233,7 +238,10 @@ __global__ void __launch_bounds__(256) uniform_prep_kernel(const SimItem *__rest
             k += inc;
             k -= k >= per ? per : 0u;
         }
-        if (wrong) atomicOr(bad + tr, 1u);
+        // (a warp that has the trace to itself says so either way)
+        const bool any = __any_sync(kFull, wrong);
+        if (lane == 0 && parts == 1u) bad[tr] = any ? 1u : 0u;
+        else if (lane == 0 && any) atomicOr(bad + tr, 1u);
     }
 }
 
@@ -662,25 +670,35 @@ __global__ void __launch_bounds__(32) uniform_play_kernel(const SimItem *__restr
 }  // namespace
 
 cudaError_t launch_uniform_prep(const SimItem *items, const uint32_t *trace_unit, uint32_t n_trace,
-                                uint64_t n_explicit, uint64_t n_items, uint64_t *counts,
-                                uint32_t *bad, int sms, cudaStream_t st) {
-    // warps to a trace: enough of them to fill the GPU when traces are few
+                                uint64_t n_explicit, uint64_t max_len, uint64_t n_items,
+                                uint64_t *counts, uint32_t *head, uint32_t *bad, int sms,
+                                cudaStream_t st) {
+    // warps to a trace: enough of them to fill the GPU when traces are few, of
+    // 2048 accesses at least; with one each, the launch needs nothing cleared
+    // before it (97 traces of 432 accesses: 2 us of memset and 2 of idle CTAs)
     const uint64_t full = (uint64_t)std::max(sms, 1) * 64;
     uint32_t parts = 1;
-    while (parts < 64 && n_explicit && n_explicit * parts < 4 * full) parts *= 2;
+    while (parts < 64 && n_explicit && n_explicit * parts < 4 * full && max_len > 2048ull * parts) parts *= 2;
+    const bool alone = parts == 1 && n_explicit;
+    if (!alone) {
+        const cudaError_t e = cudaMemsetAsync(head, 0, kQueueHeader + 4ull * n_trace, st);
+        if (e != cudaSuccess) return e;
+    }
     const uint64_t warps = std::max<uint64_t>(n_explicit ? (uint64_t)n_trace * parts : 1,
                                               counts ? (2 * n_items + 31) / 32 : 1);
     const uint64_t blocks = std::min<uint64_t>((warps + 7) / 8, (uint64_t)std::max(sms, 1) * 8);
     uniform_prep_kernel<<<(unsigned)blocks, 256, 0, st>>>(items, trace_unit, n_explicit ? n_trace : 0u,
-                                                          parts, n_items, counts, bad);
+                                                          parts, n_items, counts, bad,
+                                                          alone ? head : nullptr);
     return cudaGetLastError();
 }
 
-cudaError_t launch_uniform_out(const SimItem *items, uint64_t n_units, int sms, const SimOut &out,
-                               uint32_t *live, cudaStream_t st) {
+cudaError_t launch_uniform_out(const SimItem *items, uint64_t n_units, uint64_t max_len, int sms,
+                               const SimOut &out, uint32_t *live, cudaStream_t st) {
+    // (a part is 32 words at least)
     const uint64_t full = (uint64_t)std::max(sms, 1) * 64;
     uint32_t parts = 1;
-    while (parts < 32 && n_units * parts < 2 * full) parts *= 2;
+    while (parts < 32 && n_units * parts < 2 * full && max_len > 1024ull * parts) parts *= 2;
     const uint64_t warps = n_units * parts;
     const uint64_t blocks = std::min<uint64_t>((warps + 7) / 8, (uint64_t)std::max(sms, 1) * 8);
     uniform_out_kernel<<<(unsigned)blocks, 256, 0, st>>>(items, n_units, parts, out, live);
