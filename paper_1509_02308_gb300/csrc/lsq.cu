@@ -10,23 +10,32 @@
 // Sums over 512 points for every trace x candidate pair are a contraction, but
 // the answer is defined by FP32 sums in point order (dyr, dr, drr below), and
 // two candidates' residuals may be closer than another order's rounding.  So
-// the work is in two parts:
-//   1. estimates of every pair's residual on the tcgen05 tensor cores, from
-//      centred rows split into BF16 high and low parts (three products for the
-//      covariance; the dropped points' share of the row's sum and square sum),
-//      accurate to about 1e-5 of Var_y.  Each trace lists the candidates whose
-//      estimate is within a margin of its best one: 1e-3 Var_y, far above both
-//      the estimates' error and the FP32 sums', plus 2^-14 of the trace's
-//      square sum, which takes over when Var_y is small against it (then FP32
-//      sums cancel, the list overflows and every candidate is evaluated);
-//   2. the listed candidates' residuals by the FP32 sums themselves, a lane
-//      each, and the smallest of them.  Rows that are nearly constant (their
-//      variance below 1/64 of their mean square), whose FP32 variance cancels,
-//      are evaluated for every trace.
+// the work is in three parts:
+//   1. every pair's covariance on the tcgen05 tensor cores, from centred rows
+//      split into BF16 high and low parts (three products, accurate to about
+//      1e-5 of Var_y).  Dropped points are zeros in the trace's row, so the
+//      covariance needs no mask; Var_r does, but it lies between the row's
+//      whole square sum and that less its five largest squares, which bounds
+//      the residual from both sides without looking at the pair's points.  A
+//      trace lists the candidates whose lower bound is within a margin of the
+//      smallest upper bound seen;
+//   2. the listed candidates' residuals from the covariance and the five
+//      dropped points' rates.  The margin is 1e-3 Var_y, far above both these
+//      estimates' error and the FP32 sums', plus 2^-14 of the trace's square
+//      sum, which takes over when Var_y is small against it (then FP32 sums
+//      cancel, the list overflows and every candidate is evaluated);
+//   3. the residuals of the candidates within the margin of the best estimate
+//      by the FP32 sums themselves, and the smallest of them.  Rows that are
+//      nearly constant (their variance below 1/64 of their mean square), whose
+//      FP32 variance cancels, are evaluated for every trace.
 // Evaluating every pair on the CUDA cores (three FP32 accumulators, 64 x 64
 // tiles) took 1388 us for 8192 traces x 1308 candidates, 80 % of it FP32 issue
-// and shared-memory loads; the two parts take 233 us.  What bounds them:
-// the operand tiles' L2 reads (0.9 MB per 128 x 128 tile).
+// and shared-memory loads; with the dropped points' sums as three more tensor
+// products per pair, a 128 x 128 tile's load, MMA and epilogue one after the
+// other and a trace to a warp in part 3, 232 us (150 the estimates, 66 part 3).
+// Now 98 us: 37 the covariances (287 MB of operand tiles from L2 at 7.7 TB/s,
+// tensor pipe 41 % active), 42 parts 2 and 3 (latency: 512 dependent adds a
+// candidate, 19 % of issue slots used), 14 the traces' rows, 5 the candidates'.
 #include <algorithm>
 
 #include <cuda_bf16.h>
@@ -42,23 +51,31 @@ namespace {
 constexpr int kPoints = 512;
 constexpr int kKeep = kPoints - 5;
 constexpr uint32_t kLsqChunk = 2048;   // candidates converted at a time
-constexpr uint32_t kLsqList = 32;      // listed candidates of a trace
+constexpr uint32_t kLsqList = 128;     // listed candidates of a trace
 constexpr uint32_t kLsqIll = 4096;     // nearly constant rows
-constexpr int kYCols = 3 * kPoints;    // a trace's operand row: high, low, dropped mask
-constexpr int kRCols = 4 * kPoints;    // a candidate's: high, low, square's high, low
+constexpr int kDrop = kPoints - kKeep; // points a trace drops, at most
+constexpr int kCols = 2 * kPoints;     // an operand row: high parts, low parts
 
-struct RowStats {
+struct __align__(16) RowStats {
     float thr, cnt, sy, syy;  // kept: v <= thr; their count, sum and square sum
     float mean, var;          // of the kept points, from centred sums
-    float margin, pad;
+    float margin;
+    uint32_t n_drop;
+    uint16_t drop[8];         // the dropped points
 };
-struct Listed {
-    float res;
+struct __align__(16) Listed {
+    float cov;  // then the residual's estimate
     uint32_t g;
+    float mean, s2;  // the candidate's mean and centred square sum
+};
+struct __align__(16) Cand {
+    float inv_low, inv_s2;  // 1 / the least and the whole centred square sum
+    float mean, s2;
 };
 struct Flags {
     uint32_t all;    // 1: evaluate every candidate (a wait gave up, too many flat rows)
     uint32_t n_ill;  // nearly constant rows
+    uint32_t n_every;  // traces that evaluate every candidate
 };
 
 // The workspace: per trace operands, statistics, best estimate, list; then a
@@ -66,9 +83,9 @@ struct Flags {
 struct LsqWork {
     __nv_bfloat16 *Y, *R;
     RowStats *stats;
-    uint32_t *best, *count, *ill;
+    uint32_t *best, *count, *ill, *every;
     Listed *list;
-    float2 *cand;  // {sum, square sum} of the centred row
+    Cand *cand;
     Flags *flags;
     size_t bytes;
     LsqWork(void *base, size_t n) {
@@ -79,13 +96,14 @@ struct LsqWork {
             o = (o + b + 255) & ~size_t(255);
             return q;
         };
-        Y = reinterpret_cast<__nv_bfloat16 *>(take(n * kYCols * 2));
+        Y = reinterpret_cast<__nv_bfloat16 *>(take(n * kCols * 2));
         stats = reinterpret_cast<RowStats *>(take(n * sizeof(RowStats)));
         best = reinterpret_cast<uint32_t *>(take(n * 4));
         count = reinterpret_cast<uint32_t *>(take(n * 4));
         list = reinterpret_cast<Listed *>(take(n * kLsqList * sizeof(Listed)));
-        R = reinterpret_cast<__nv_bfloat16 *>(take((size_t)kLsqChunk * kRCols * 2));
-        cand = reinterpret_cast<float2 *>(take((size_t)kLsqChunk * sizeof(float2)));
+        R = reinterpret_cast<__nv_bfloat16 *>(take((size_t)kLsqChunk * kCols * 2));
+        cand = reinterpret_cast<Cand *>(take((size_t)kLsqChunk * sizeof(Cand)));
+        every = reinterpret_cast<uint32_t *>(take(n * 4));
         ill = reinterpret_cast<uint32_t *>(take(kLsqIll * 4));
         flags = reinterpret_cast<Flags *>(take(sizeof(Flags)));
         bytes = o;
@@ -120,21 +138,22 @@ __global__ void __launch_bounds__(256) lsq_rows_kernel(const float *__restrict__
         for (int q = 0; q < 4; ++q)
 #pragma unroll
             for (int e = 0; e < 4; ++e) v[4 * q + e] = row[4 * lane + 128 * q + e];
-        uint32_t out = 0;  // values taken out
-        uint32_t kth = 0;
-        for (int round = 0; round < kPoints - kKeep + 1; ++round) {
-            uint32_t top = 0, at = 0;
+        uint32_t key[16], kth = 0;  // (a value taken out has key 0)
 #pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const uint32_t k = order_key(v[e]);
-                if (!((out >> e) & 1u) && k >= top) {
-                    top = k;
-                    at = (uint32_t)e;
-                }
-            }
+        for (int e = 0; e < 16; ++e) key[e] = order_key(v[e]);
+        for (int round = 0; round < kDrop + 1; ++round) {
+            uint32_t top = 0;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) top = max(top, key[e]);
             kth = __reduce_max_sync(kFull, top);
             const uint32_t who = __ballot_sync(kFull, top == kth);
-            if (lane == (uint32_t)(__ffs(who) - 1)) out |= 1u << at;
+            bool mine = lane == (uint32_t)(__ffs(who) - 1);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                const bool hit = mine && key[e] == kth;
+                key[e] = hit ? 0u : key[e];
+                mine = mine && !hit;
+            }
         }
         const float thr = key_value(kth);
         float c = 0.0f, sy = 0.0f, syy = 0.0f;
@@ -150,10 +169,10 @@ __global__ void __launch_bounds__(256) lsq_rows_kernel(const float *__restrict__
         syy = warp_sum(syy);
         const float mean = sy / c;
         float var = 0.0f;
-        __nv_bfloat16 *o = w.Y + (size_t)i * kYCols;
+        __nv_bfloat16 *o = w.Y + (size_t)i * kCols;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            __nv_bfloat16 hi[4], lo[4], d[4];
+            __nv_bfloat16 hi[4], lo[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const bool kept = v[4 * q + e] <= thr;
@@ -161,16 +180,23 @@ __global__ void __launch_bounds__(256) lsq_rows_kernel(const float *__restrict__
                 var += z * z;
                 hi[e] = __float2bfloat16(z);
                 lo[e] = __float2bfloat16(z - __bfloat162float(hi[e]));
-                d[e] = __float2bfloat16(kept ? 0.0f : 1.0f);
             }
             const uint32_t p = 4 * lane + 128 * q;
             *reinterpret_cast<uint2 *>(o + p) = *reinterpret_cast<const uint2 *>(hi);
             *reinterpret_cast<uint2 *>(o + kPoints + p) = *reinterpret_cast<const uint2 *>(lo);
-            *reinterpret_cast<uint2 *>(o + 2 * kPoints + p) = *reinterpret_cast<const uint2 *>(d);
         }
         var = warp_sum(var);
+        uint32_t nd = 0;  // dropped points (more than kDrop: values that compare with nothing)
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const bool gone = !(v[e] <= thr);
+            const uint32_t who = __ballot_sync(kFull, gone);
+            const uint32_t at = nd + (uint32_t)__popc(who & ((1u << lane) - 1u));
+            if (gone && at < 8u) w.stats[i].drop[at] = (uint16_t)(4 * lane + 128 * (e >> 2) + (e & 3));
+            nd += (uint32_t)__popc(who);
+        }
         if (lane == 0) {
-            RowStats s;
+            RowStats &s = w.stats[i];
             s.thr = thr;
             s.cnt = c;
             s.sy = sy;
@@ -178,15 +204,15 @@ __global__ void __launch_bounds__(256) lsq_rows_kernel(const float *__restrict__
             s.mean = mean;
             s.var = var;
             s.margin = 1e-3f * var + syy * (1.0f / 16384.0f);
-            s.pad = 0.0f;
-            w.stats[i] = s;
+            s.n_drop = min(nd, (uint32_t)kDrop);
             w.best[i] = 0x7F800000u;
-            w.count[i] = 0;
+            w.count[i] = nd > (uint32_t)kDrop ? kLsqList + 1u : 0u;
         }
     }
 }
 
-// One warp per candidate of the chunk: centred row, split, and its sums.
+// One warp per candidate of the chunk: centred row, split, its square sum and
+// what is left of that without its five largest squares.
 __global__ void __launch_bounds__(256) lsq_rates_kernel(const float *__restrict__ rates, uint32_t g0,
                                                         uint32_t ng, LsqWork w) {
     const uint32_t lane = threadIdx.x & 31u;
@@ -205,30 +231,51 @@ __global__ void __launch_bounds__(256) lsq_rates_kernel(const float *__restrict_
         }
     const float mean = warp_sum(sum) * (1.0f / kPoints);
     raw = warp_sum(raw);
-    float s1 = 0.0f, s2 = 0.0f;
-    __nv_bfloat16 *o = w.R + (size_t)k * kRCols;
+    float s2 = 0.0f, zz[16];
+    __nv_bfloat16 *o = w.R + (size_t)k * kCols;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        __nv_bfloat16 t[4][4];
+        __nv_bfloat16 hi[4], lo[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const float z = v[4 * q + e] - mean, zz = z * z;
-            s1 += z;
-            s2 += zz;
-            t[0][e] = __float2bfloat16(z);
-            t[1][e] = __float2bfloat16(z - __bfloat162float(t[0][e]));
-            t[2][e] = __float2bfloat16(zz);
-            t[3][e] = __float2bfloat16(zz - __bfloat162float(t[2][e]));
+            const float z = v[4 * q + e] - mean;
+            zz[4 * q + e] = z * z;
+            s2 += z * z;
+            hi[e] = __float2bfloat16(z);
+            lo[e] = __float2bfloat16(z - __bfloat162float(hi[e]));
         }
-#pragma unroll
-        for (int h = 0; h < 4; ++h)
-            *reinterpret_cast<uint2 *>(o + h * kPoints + 4 * lane + 128 * q) =
-                *reinterpret_cast<const uint2 *>(t[h]);
+        const uint32_t p = 4 * lane + 128 * q;
+        *reinterpret_cast<uint2 *>(o + p) = *reinterpret_cast<const uint2 *>(hi);
+        *reinterpret_cast<uint2 *>(o + kPoints + p) = *reinterpret_cast<const uint2 *>(lo);
     }
-    s1 = warp_sum(s1);
     s2 = warp_sum(s2);
+    float top = 0.0f;
+    uint32_t out = 0;
+    for (int round = 0; round < kDrop; ++round) {
+        float mx = -1.0f;
+        int at = 0;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            if (!((out >> e) & 1u) && zz[e] > mx) {
+                mx = zz[e];
+                at = e;
+            }
+        }
+        const uint32_t all = __reduce_max_sync(kFull, mx < 0.0f ? 0u : __float_as_uint(mx));
+        const uint32_t who = __ballot_sync(kFull, mx >= 0.0f && __float_as_uint(mx) == all);
+        if (lane == (uint32_t)(__ffs(who) - 1)) out |= 1u << at;
+        top += __uint_as_float(all);
+    }
     if (lane == 0) {
-        w.cand[k] = make_float2(s1, s2);
+        // a trace's Var_r is s2 less its dropped points' squares and less
+        // (their sum)^2 / 507, below a hundredth of their squares
+        const float low = s2 * (1.0f - 1e-5f) - 1.02f * top;
+        Cand c;
+        c.inv_low = low > 1e-3f * s2 && low > 1e-9f ? 1.0f / low : __int_as_float(0x7F800000);
+        c.inv_s2 = low > 1e-9f ? 1.0f / s2 : 0.0f;
+        c.mean = mean;
+        c.s2 = s2;
+        w.cand[k] = c;
         // (also rows whose sums are not finite)
         if (!(64.0f * s2 >= raw)) {
             const uint32_t at = atomicAdd(&w.flags->n_ill, 1u);
@@ -238,36 +285,77 @@ __global__ void __launch_bounds__(256) lsq_rates_kernel(const float *__restrict_
     }
 }
 
-// Estimates: persistent CTAs over 128 x 128 tiles (traces x candidates), the
-// three sums side by side in TMEM (128 columns each).  A K block of 64 points
-// is seven TMA tiles (112 KB) in one of two stages and 24 MMAs; one thread
-// issues both.  Epilogue: a thread per trace and column half, first its best
-// estimate, then the candidates to list.
-constexpr uint32_t kTile = 128 * 128;  // bytes of a 128 x 64 BF16 tile
-constexpr uint32_t kLsqStage = 7 * kTile;
-constexpr uint32_t kLsqSmem = 1024 + 2 * kLsqStage + 128 * 8 + 64;
-// M 128, N 128, BF16 operands, FP32 sums
-constexpr uint32_t kIdescLsq = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+// A pair's residual from its covariance (a positive one's square), the
+// candidate's mean and centred square sum, and its rates at the trace's
+// dropped points.
+__device__ __forceinline__ float estimate(float cov2, float mean, float s2, const float *__restrict__ row,
+                                          const RowStats &s) {
+    float dr = 0.0f, dq = 0.0f;
+#pragma unroll
+    for (uint32_t k = 0; k < (uint32_t)kDrop; ++k) {
+        if (k < s.n_drop) {
+            const float r = __ldg(row + s.drop[k]) - mean;
+            dr += r;
+            dq += r * r;
+        }
+    }
+    const float var_r = (s2 - dq) - dr * dr / s.cnt;
+    return var_r > 1e-12f ? fmaxf(s.var - cov2 / var_r, 0.0f) : s.var;
+}
 
-__global__ void __launch_bounds__(256)
+// Covariances and lists: persistent CTAs over tiles of 128 traces x N
+// candidates, candidate-major, so that the first tiles leave most traces an
+// upper bound for the others to list by.  A K block of 64 points is four TMA
+// tiles (32 KB of traces, N / 4 KB of candidates) in a ring of stages and 12
+// MMAs; the sums are double buffered in TMEM (columns 0 and 256), so the next
+// tile's MMAs run under this one's epilogue.  Warps 0-7: epilogue, a thread per
+// trace and column half; warp 8: loads; warp 9: MMAs (one thread each).
+//
+// N: bytes read per tile are 256 (N + 128) a K row, and a wave is a tile on
+// every SM, so the N with the least waves (N + 128) (8192 x 1308: 192, three
+// waves).
+constexpr uint32_t kTile = 128 * 128;  // bytes of a 128 x 64 BF16 tile
+constexpr uint32_t kLsqMaxN = 256, kLsqMaxStages = 5, kLsqRing = 200 * 1024;
+constexpr uint32_t kLsqBars = 16;      // loaded, free [stages]; sums ready, read [2]
+constexpr uint32_t kLsqSmem = 1024 + kLsqRing + kLsqMaxN * 16 + kLsqBars * 8 + 16;
+constexpr uint32_t kLsqThreads = 320;
+// M 128, BF16 operands, FP32 sums; N is added
+constexpr uint32_t kIdescLsq = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
+
+__host__ __device__ constexpr uint32_t lsq_stage_bytes(uint32_t N) { return 2 * kTile + 2 * N * 128; }
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(kLsqThreads, 1)
     lsq_estimate_kernel(const __grid_constant__ CUtensorMap ymap, const __grid_constant__ CUtensorMap rmap,
-                        uint32_t n, const uint32_t *n_dev, uint32_t g0, uint32_t ng, LsqWork w) {
+                        const float *__restrict__ rates, uint32_t n, const uint32_t *n_dev, uint32_t g0,
+                        uint32_t ng, uint32_t N, LsqWork w) {
     extern __shared__ uint8_t dsm[];
     const uint32_t raw = smem_u32(dsm);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *const gbase = dsm + (base - raw);
-    float2 *const cand = reinterpret_cast<float2 *>(gbase + 2 * kLsqStage);
-    // mbarriers: stage loaded [2], stage's MMAs done [2]
-    const uint32_t full0 = base + 2 * kLsqStage + 128 * 8, done0 = full0 + 16u;
-    uint32_t *const tslot = reinterpret_cast<uint32_t *>(gbase + 2 * kLsqStage + 128 * 8 + 32);
+    Cand *const cand = reinterpret_cast<Cand *>(gbase + kLsqRing);
+    const uint32_t bars = base + kLsqRing + kLsqMaxN * 16;
+    const uint32_t full0 = bars, free0 = bars + 8 * kLsqMaxStages, ready0 = free0 + 8 * kLsqMaxStages,
+                   read0 = ready0 + 16;
+    uint32_t *const tslot = reinterpret_cast<uint32_t *>(gbase + kLsqRing + kLsqMaxN * 16 + kLsqBars * 8);
     volatile uint32_t *const abort_flag = tslot + 1;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (n_dev && *n_dev < n) n = *n_dev;
-    const uint32_t gt = (ng + 127u) / 128u, tiles = (n + 127u) / 128u * gt;
+    const uint32_t stage = lsq_stage_bytes(N), S = min(kLsqMaxStages, kLsqRing / stage);
+    const uint32_t mt = (n + 127u) / 128u, tiles = mt * ((ng + N - 1u) / N);
     constexpr int kBlocks = kPoints / 64;
     if (tid == 0) {
-        for (int q = 0; q < 4; ++q)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8 * q) : "memory");
+        for (uint32_t q = 0; q < 2 * kLsqMaxStages + 2; ++q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bars + 8 * q) : "memory");
+        for (uint32_t q = 0; q < 2; ++q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;" ::"r"(read0 + 8 * q) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         *abort_flag = 0;
     }
@@ -282,233 +370,390 @@ __global__ void __launch_bounds__(256)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
-    // K blocks are numbered through all of this CTA's tiles: block b uses stage
-    // b mod 2, whose barriers it completes for the (b / 2)-th time
-    auto load = [&](uint32_t tile, int kb, uint32_t b) {
-        const uint32_t q = b & 1u, st = base + q * kLsqStage, bar = full0 + 8u * q;
-        const int m0 = (int)(tile / gt) * 128, c0 = (int)(tile % gt) * 128, k0 = kb * 64;
-        mbar_expect_tx(bar, kLsqStage);
-#pragma unroll
-        for (int h = 0; h < 3; ++h) tma_load_2d(st + h * kTile, &ymap, h * kPoints + k0, m0, bar);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) tma_load_2d(st + (3 + h) * kTile, &rmap, h * kPoints + k0, c0, bar);
-    };
-    uint32_t b = 0;        // blocks consumed (thread 0)
-    uint32_t loaded = 0;   // blocks requested (thread 0)
-    auto load_next = [&]() {
-        // block `loaded` of this CTA's sequence, if it has one
-        const uint64_t tile = (uint64_t)blockIdx.x + (uint64_t)(loaded / kBlocks) * gridDim.x;
-        if (tile < tiles) {
-            load((uint32_t)tile, (int)(loaded % kBlocks), loaded);
-            ++loaded;
-        }
-    };
-    if (tid == 0) {
-        load_next();
-        load_next();
-    }
-    bool ok = true;
-    uint32_t tno = 0;
-    for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++tno) {
-        if (tid < 128) {
-            const uint32_t g = tile % gt * 128u + (uint32_t)tid;
-            cand[tid] = g < ng ? w.cand[g] : make_float2(0.0f, 0.0f);
-        }
-        if (tid == 0) {
-            for (int kb = 0; kb < kBlocks; ++kb, ++b) {
-                const uint32_t q = b & 1u, par = (b >> 1) & 1u;
-                if (!mbar_wait(full0 + 8u * q, par)) {
-                    *abort_flag = 1;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t st = base + q * kLsqStage;
-#pragma unroll
-                for (int s = 0; s < 4; ++s) {
-                    const uint64_t yh = sw128_desc(st + 32u * s), yl = sw128_desc(st + kTile + 32u * s),
-                                   dm = sw128_desc(st + 2 * kTile + 32u * s),
-                                   rh = sw128_desc(st + 3 * kTile + 32u * s),
-                                   rl = sw128_desc(st + 4 * kTile + 32u * s),
-                                   qh = sw128_desc(st + 5 * kTile + 32u * s),
-                                   ql = sw128_desc(st + 6 * kTile + 32u * s);
-                    const uint32_t add = (kb | s) != 0 ? 1u : 0u;
-                    mma_bf16_id(tmem, yh, rh, kIdescLsq, add);
-                    mma_bf16_id(tmem, yh, rl, kIdescLsq, 1u);
-                    mma_bf16_id(tmem, yl, rh, kIdescLsq, 1u);
-                    mma_bf16_id(tmem + 128u, dm, rh, kIdescLsq, add);
-                    mma_bf16_id(tmem + 256u, dm, qh, kIdescLsq, add);
-                    mma_bf16_id(tmem + 256u, dm, ql, kIdescLsq, 1u);
-                }
-                asm volatile(
-                    "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                        done0 + 8u * q)
-                    : "memory");
-                // the other stage's block (its MMAs went out a step ago) is
-                // replaced once they are done
-                if (b > 0) {
-                    const uint32_t pb = b - 1u;
-                    if (!mbar_wait(done0 + 8u * (pb & 1u), (pb >> 1) & 1u)) {
+    // K blocks are numbered through all of this CTA's tiles: block b is in
+    // stage b mod S, whose barriers it completes for the (b / S)-th time
+    if (warp == 8) {
+        if (lane == 0) {
+            uint32_t b = 0, q = 0, par = 0;
+            for (uint32_t tile = blockIdx.x; tile < tiles && !*abort_flag; tile += gridDim.x) {
+                const int m0 = (int)(tile % mt) * 128, c0 = (int)(tile / mt * N);
+                for (int kb = 0; kb < kBlocks; ++kb, ++b) {
+                    if (!mbar_wait(free0 + 8u * q, par ^ 1u)) {
                         *abort_flag = 1;
                         break;
                     }
-                    load_next();
-                }
-            }
-        }
-        __syncthreads();
-        ok = *abort_flag == 0;
-        if (!ok) break;
-        const uint32_t lb = (tno + 1u) * kBlocks - 1u;  // the tile's last block
-        const bool got = mbar_wait(done0 + 8u * (lb & 1u), (lb >> 1) & 1u);
-        ok = __syncthreads_and(got);
-        if (!ok) break;
-        tc_fence_after();
-        // epilogue: warps w and w + 4 share TMEM lanes 32 (w % 4) .., a column
-        // half each
-        const uint32_t half = (uint32_t)warp >> 2;
-        const uint32_t i = tile / gt * 128u + 32u * ((uint32_t)warp & 3u) + (uint32_t)lane;
-        const uint32_t taddr = tmem + ((32u * ((uint32_t)warp & 3u)) << 16) + 64u * half;
-        const bool act = i < n;
-        RowStats s{};
-        if (act) s = w.stats[i];
-        const float inv = act ? 1.0f / s.cnt : 0.0f;
-        const uint32_t c0 = tile % gt * 128u + 64u * half;
-        auto estimate = [&](float cov, float dr, float dq, float2 c) {
-            const float d = c.x - dr, var = (c.y - dq) - d * d * inv;
-            const float r = var > 1e-12f && cov > 0.0f ? s.var - cov * cov / var : s.var;
-            return fmaxf(r, 0.0f);
-        };
-        float best = 3.0e38f;
-        for (int pass = 0; pass < 2; ++pass) {
-            float limit = 0.0f;
-            if (pass == 1) {
-                float all = best;
-                if (act) {
-                    const uint32_t old = atomicMin(w.best + i, __float_as_uint(best));
-                    all = fminf(best, __uint_as_float(old));
-                }
-                limit = all + s.margin;
-                if (!__any_sync(kFull, act && !(best > limit))) break;
-            }
-#pragma unroll 1
-            for (uint32_t q = 0; q < 4; ++q) {
-                uint32_t x[16], y[16], z[16];
-                __syncwarp();
-                tmem_ld16(taddr + 16u * q, x);
-                tmem_ld16(taddr + 128u + 16u * q, y);
-                tmem_ld16(taddr + 256u + 16u * q, z);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const uint32_t g = c0 + 16u * q + (uint32_t)e;
-                    const float r = estimate(__uint_as_float(x[e]), __uint_as_float(y[e]),
-                                             __uint_as_float(z[e]), cand[64u * half + 16u * q + e]);
-                    if (g >= ng) continue;
-                    if (pass == 0) {
-                        best = fminf(best, r);
-                    } else if (act && !(r > limit)) {
-                        const uint32_t at = atomicAdd(w.count + i, 1u);
-                        if (at < kLsqList) w.list[(size_t)i * kLsqList + at] = Listed{r, g0 + g};
+                    const uint32_t st = base + q * stage, bar = full0 + 8u * q;
+                    mbar_expect_tx(bar, stage);
+                    tma_load_2d(st, &ymap, kb * 64, m0, bar);
+                    tma_load_2d(st + kTile, &ymap, kPoints + kb * 64, m0, bar);
+                    tma_load_2d(st + 2 * kTile, &rmap, kb * 64, c0, bar);
+                    tma_load_2d(st + 2 * kTile + N * 128, &rmap, kPoints + kb * 64, c0, bar);
+                    if (++q == S) {
+                        q = 0;
+                        par ^= 1u;
                     }
                 }
             }
+            // loads in flight land before the CTA leaves
+            for (uint32_t k = b > S ? b - S : 0u; k < b; ++k) mbar_wait(full0 + 8u * (k % S), (k / S) & 1u);
         }
-        // every thread is done with the sums before the next tile's MMAs
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
+    } else if (warp == 9) {
+        if (lane == 0) {
+            const uint32_t idesc = kIdescLsq | ((N >> 3) << 17);
+            uint32_t b = 0, q = 0, par = 0, tno = 0;
+            bool ok = true;
+            for (uint32_t tile = blockIdx.x; ok && tile < tiles && !*abort_flag; tile += gridDim.x, ++tno) {
+                const uint32_t buf = tno & 1u, d = tmem + 256u * buf;
+                ok = mbar_wait(read0 + 8u * buf, ((tno >> 1) & 1u) ^ 1u);
+                tc_fence_after();
+                for (int kb = 0; ok && kb < kBlocks; ++kb) {
+                    ok = mbar_wait(full0 + 8u * q, par);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t st = base + q * stage;
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) {
+                        const uint64_t yh = sw128_desc(st + 32u * s), yl = sw128_desc(st + kTile + 32u * s),
+                                       rh = sw128_desc(st + 2 * kTile + 32u * s),
+                                       rl = sw128_desc(st + 2 * kTile + N * 128 + 32u * s);
+                        mma_bf16_id(d, yh, rh, idesc, (kb | s) != 0 ? 1u : 0u);
+                        mma_bf16_id(d, yh, rl, idesc, 1u);
+                        mma_bf16_id(d, yl, rh, idesc, 1u);
+                    }
+                    mma_commit(free0 + 8u * q);
+                    ++b;
+                    if (++q == S) {
+                        q = 0;
+                        par ^= 1u;
+                    }
+                }
+                if (ok) mma_commit(ready0 + 8u * buf);
+            }
+            if (!ok) *abort_flag = 1;
+            // and so do the MMAs
+            if (b) mbar_wait(free0 + 8u * ((b - 1u) % S), ((b - 1u) / S) & 1u);
+        }
+    } else {
+        // warps w and w + 4 share TMEM lanes 32 (w % 4) .., a column half each
+        const uint32_t quarter = (uint32_t)warp & 3u, half = (uint32_t)warp >> 2, cols = N / 2;
+        uint32_t tno = 0;
+        for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++tno) {
+            const uint32_t buf = tno & 1u, c0 = tile / mt * N;
+            // (every warp is done with the last tile's candidates)
+            if (group_any(1, *abort_flag != 0)) break;
+            for (uint32_t c = (uint32_t)tid; c < N; c += 256) {
+                float4 f = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (c0 + c < ng) f = *reinterpret_cast<const float4 *>(w.cand + c0 + c);
+                *reinterpret_cast<float4 *>(cand + c) = f;
+            }
+            const uint32_t i = tile % mt * 128u + 32u * quarter + (uint32_t)lane;
+            const bool act = i < n;
+            RowStats s{};
+            if (act) s = w.stats[i];
+            const bool got = mbar_wait(ready0 + 8u * buf, (tno >> 1) & 1u);
+            if (group_any(1, !got)) {
+                *abort_flag = 1;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t taddr = tmem + 256u * buf + ((32u * quarter) << 16) + half * cols;
+            const Cand *const cd = cand + half * cols;
+            // the residual is var - cov^2 / Var_r for a positive covariance
+            float top = 0.0f;
+            uint32_t arg = 0;
+#pragma unroll 1
+            for (uint32_t q = 0; q < cols; q += 16) {
+                uint32_t x[16];
+                __syncwarp();
+                tmem_ld16(taddr + q, x);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    const float cov = fmaxf(__uint_as_float(x[e]), 0.0f), gain = cov * cov * cd[q + e].inv_s2;
+                    if (gain > top) {
+                        top = gain;
+                        arg = q + (uint32_t)e;
+                    }
+                }
+            }
+            // the estimate of the one with the least upper bound: a third of
+            // the listed candidates that the bound itself lets through
+            float best = s.var;
+            if (act && top > 0.0f) {
+                const Cand f = cd[arg];
+                best = estimate(top * f.s2, f.mean, f.s2, rates + (size_t)(g0 + c0 + half * cols + arg) * kPoints,
+                                s);
+            }
+            if (act) best = fminf(best, __uint_as_float(atomicMin(w.best + i, __float_as_uint(best))));
+            const float need = s.var - (best + s.margin);
+            uint32_t take[kLsqMaxN / 64] = {}, found = 0;
+#pragma unroll
+            for (uint32_t h = 0; h < kLsqMaxN / 64; ++h) {
+                if (32 * h >= cols) break;
+#pragma unroll
+                for (uint32_t q = 0; q < 32; q += 16) {
+                    if (32 * h + q >= cols) break;
+                    uint32_t x[16];
+                    __syncwarp();
+                    tmem_ld16(taddr + 32 * h + q, x);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        const float cov = __uint_as_float(x[e]);
+                        const float gain = cov > 0.0f ? cov * cov * cd[32 * h + q + e].inv_low : 0.0f;
+                        if (!(gain < need)) take[h] |= 1u << (q + (uint32_t)e);
+                    }
+                }
+                // (columns past the last candidate)
+                const uint32_t c = c0 + half * cols + 32 * h;
+                if (!act || c >= ng) take[h] = 0;
+                else if (ng - c < 32) take[h] &= (1u << (ng - c)) - 1u;
+                found += (uint32_t)__popc(take[h]);
+            }
+            // one reservation a thread and tile: an atomic's round trip per
+            // listed candidate cost more than the tile's MMAs
+            uint32_t at = found ? atomicAdd(w.count + i, found) : 0u;
+            Listed *const list = w.list + (size_t)i * kLsqList;
+#pragma unroll
+            for (uint32_t h = 0; h < kLsqMaxN / 64; ++h) {
+                if (32 * h >= cols) break;
+#pragma unroll
+                for (uint32_t q = 0; q < 32; q += 16) {
+                    if (32 * h + q >= cols) break;
+                    if (!__any_sync(kFull, (take[h] >> q) & 0xFFFFu)) continue;
+                    uint32_t x[16];
+                    tmem_ld16(taddr + 32 * h + q, x);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        if ((take[h] >> (q + (uint32_t)e)) & 1u) {
+                            const uint32_t c = 32 * h + q + (uint32_t)e;
+                            if (at < kLsqList)
+                                list[at] = Listed{__uint_as_float(x[e]), g0 + c0 + half * cols + c, cd[c].mean,
+                                                  cd[c].s2};
+                            ++at;
+                        }
+                    }
+                }
+            }
+            // the sums are read; their columns may take the tile after next
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(read0 + 8u * buf);
+        }
     }
-    if (!ok && tid == 0) {
-        w.flags->all = 1u;
-        // loads and MMAs still in flight land before the CTA leaves
-        for (uint32_t k = loaded > 2u ? loaded - 2u : 0u; k < loaded; ++k)
-            mbar_wait(full0 + 8u * (k & 1u), (k >> 1) & 1u);
-        if (b > 0) mbar_wait(done0 + 8u * ((b - 1u) & 1u), ((b - 1u) >> 1) & 1u);
-    }
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (tid == 0 && *abort_flag) w.flags->all = 1u;
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
                      : "memory");
 }
 
-// One warp per trace: the listed candidates' residuals by FP32 sums in point
-// order, a candidate per lane; the smallest, then the lowest index.
-constexpr int kExactWarps = 8;
+// A candidate's residual by FP32 sums in point order: v the kept values (0 at
+// dropped points), kept a bit per point, both in shared memory.
+struct Trace {
+    float cnt, sy, var_y;
+};
+__device__ __forceinline__ float residual(const float *__restrict__ r1, bool vec, const float *v,
+                                          const uint32_t *kept, const Trace &t) {
+    float dyr = 0.0f, dr = 0.0f, drr = 0.0f;
+    auto load = [&](int q, float4 (&r)[8]) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float *const p = r1 + 32 * q + 4 * k;
+            r[k] = vec ? __ldg(reinterpret_cast<const float4 *>(p))
+                       : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+        }
+    };
+    auto add = [&](int q, const float4 (&r)[8]) {
+        const uint32_t bits = kept[q];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float4 y = *reinterpret_cast<const float4 *>(v + 32 * q + 4 * k);
+            const float rv[4] = {r[k].x, r[k].y, r[k].z, r[k].w}, yv[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float m = (bits >> (4 * k + e)) & 1u ? 1.0f : 0.0f;
+                dyr = fmaf(yv[e], rv[e], dyr);
+                dr = fmaf(m, rv[e], dr);
+                drr = fmaf(m, rv[e] * rv[e], drr);
+            }
+        }
+    };
+    // 128 bytes of the row ahead of the adds
+    float4 a[8], b[8];
+    load(0, a);
+#pragma unroll 1
+    for (int q = 0; q < kPoints / 32; q += 2) {
+        load(q + 1, b);
+        add(q, a);
+        if (q + 2 < kPoints / 32) load(q + 2, a);
+        add(q + 1, b);
+    }
+    const float cov = dyr - t.sy * dr / t.cnt;
+    const float var_r = drr - dr * dr / t.cnt;
+    float res = t.var_y;
+    if (var_r > 1e-12f && cov > 0.0f) res = t.var_y - cov * cov / var_r;
+    return fmaxf(res, 0.0f);
+}
+
+// the kept values and bits of trace i, by a warp
+__device__ __forceinline__ void load_trace(const float *__restrict__ y, uint32_t i, float thr, float *v,
+                                           uint32_t *kept, uint32_t lane) {
+#pragma unroll 4
+    for (uint32_t q = 0; q < kPoints / 32; ++q) {
+        const float x = y[(size_t)i * kPoints + 32 * q + lane], m = x <= thr ? 1.0f : 0.0f;
+        v[32 * q + lane] = m * x;
+        const uint32_t bits = __ballot_sync(kFull, x <= thr);
+        if (lane == 0) kept[q] = bits;
+    }
+}
+
+// What the warps of one left-over trace share, at the start of its list.
+struct Shared {
+    unsigned long long key;  // least residual, then candidate
+    uint32_t done;           // parts evaluated
+};
+
+// Eight lanes to a trace: its listed candidates' estimates, then the residuals
+// of those within the margin of the best (3 on average), a candidate per lane;
+// the smallest, then the lowest index.  A residual is a chain of 512 dependent
+// adds fed by 2 KB of its own row, so what counts is that every trace is in
+// flight at once and a lane's loads go out 128 bytes at a time.
+constexpr int kExactWarps = 4, kGroup = 8, kPerWarp = 32 / kGroup;
+constexpr int kRowPad = kPoints + 4, kKeptPad = kPoints / 32 + 1;  // (the groups' banks differ)
 __global__ void __launch_bounds__(kExactWarps * 32)
     lsq_exact_kernel(const float *__restrict__ y, uint32_t n, const uint32_t *n_dev,
-                     const float *__restrict__ rates, uint32_t G, LsqWork w, uint32_t *idx_out,
-                     float *res_out) {
-    __shared__ float2 sh[kExactWarps][kPoints];  // {kept value, kept}
+                     const float *__restrict__ rates, LsqWork w, uint32_t *idx_out, float *res_out) {
+    __shared__ __align__(16) float rows[kExactWarps][kPerWarp][kRowPad];
+    __shared__ uint32_t keeps[kExactWarps][kPerWarp][kKeptPad];
+    __shared__ uint32_t lists[kExactWarps][kPerWarp][kLsqList];
     if (n_dev && *n_dev < n) n = *n_dev;
-    const uint32_t lane = threadIdx.x & 31u;
-    float2 *const yv = sh[threadIdx.x >> 5];
+    const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, grp = lane / kGroup, l = lane % kGroup;
+    uint32_t *const near = lists[wid][grp];
     const uint32_t nw = gridDim.x * kExactWarps;
     const uint32_t n_ill = w.flags->n_ill;
+    const bool all = w.flags->all != 0;
     const bool vec = (reinterpret_cast<uintptr_t>(rates) & 15u) == 0;
-    for (uint32_t i = blockIdx.x * kExactWarps + (threadIdx.x >> 5); i < n; i += nw) {
-        const RowStats s = w.stats[i];
-        for (uint32_t p = lane; p < kPoints; p += 32) {
-            const float v = y[(size_t)i * kPoints + p], m = v <= s.thr ? 1.0f : 0.0f;
-            yv[p] = make_float2(m * v, m);
+    for (uint32_t t0 = (blockIdx.x * kExactWarps + wid) * kPerWarp; t0 < n; t0 += nw * kPerWarp) {
+        const uint32_t i = t0 + grp;
+        const uint32_t listed = i < n ? w.count[i] : 0u;
+        const bool every = all || listed > kLsqList || listed == 0;
+        if (i < n && every && l == 0) {
+            w.every[atomicAdd(&w.flags->n_every, 1u)] = i;
+            *reinterpret_cast<Shared *>(w.list + (size_t)i * kLsqList) = Shared{~0ull, 0u};
         }
-        const uint32_t listed = w.count[i];
-        const bool every = w.flags->all || listed > kLsqList || listed == 0;
-        const float limit = __uint_as_float(w.best[i]) + s.margin;
-        const uint32_t total = every ? G : listed + n_ill;
-        const float cnt = s.cnt, sy = s.sy, syy = s.syy;
-        const float var_y = syy - sy * sy / cnt;
-        __syncwarp();
-        unsigned long long best = ~0ull;
-        for (uint32_t c0 = 0; c0 < total; c0 += 32) {
-            const uint32_t c = c0 + lane;
-            uint32_t g = 0xFFFFFFFFu;
-            if (c < total) {
-                if (every) {
-                    g = c;
-                } else if (c < listed) {
-                    const Listed l = w.list[(size_t)i * kLsqList + c];
-                    if (!(l.res > limit)) g = l.g;
-                } else {
-                    g = w.ill[c - listed];
-                }
+        const bool act = i < n && !every;
+        if (!__any_sync(kFull, act)) continue;
+        RowStats s{};
+        if (act) s = w.stats[i];
+        __syncwarp();  // (the last traces' rows are read)
+#pragma unroll 1
+        for (uint32_t q = 0; q < kPerWarp; ++q) {
+            const float thr = __shfl_sync(kFull, s.thr, q * kGroup);
+            if (__shfl_sync(kFull, act ? 1u : 0u, q * kGroup))
+                load_trace(y, t0 + q, thr, rows[wid][q], keeps[wid][q], lane);
+        }
+        Listed *const list = w.list + (size_t)i * kLsqList;
+        float best = 3.0e38f;
+        if (act) {
+            for (uint32_t c = l; c < listed; c += kGroup) {
+                const Listed e = list[c];
+                const float est =
+                    e.cov > 0.0f ? estimate(e.cov * e.cov, e.mean, e.s2, rates + (size_t)e.g * kPoints, s) : s.var;
+                list[c].cov = est;
+                best = fminf(best, est);
             }
-            if (g == 0xFFFFFFFFu) continue;
-            const float *const r1 = rates + (size_t)g * kPoints;
-            float dyr = 0.0f, dr = 0.0f, drr = 0.0f;
-#pragma unroll 4
-            for (int p = 0; p < kPoints / 4; ++p) {
-                const float4 r = vec ? __ldg(reinterpret_cast<const float4 *>(r1) + p)
-                                     : make_float4(__ldg(r1 + 4 * p), __ldg(r1 + 4 * p + 1),
-                                                   __ldg(r1 + 4 * p + 2), __ldg(r1 + 4 * p + 3));
-                const float rv[4] = {r.x, r.y, r.z, r.w};
+        }
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 v = yv[4 * p + e];
-                    dyr = fmaf(v.x, rv[e], dyr);
-                    dr = fmaf(v.y, rv[e], dr);
-                    drr = fmaf(v.y, rv[e] * rv[e], drr);
-                }
+        for (int o = kGroup / 2; o; o >>= 1) best = fminf(best, __shfl_xor_sync(kFull, best, o));
+        const float limit = best + s.margin;
+        uint32_t n_near = 0;
+        const uint32_t trips = __reduce_max_sync(kFull, act ? listed : 0u);
+        for (uint32_t c = l; c < trips + l; c += kGroup) {
+            bool take = false;
+            uint32_t g = 0;
+            if (act && c < listed) {
+                take = !(list[c].cov > limit);
+                g = list[c].g;
             }
-            const float cov = dyr - sy * dr / cnt;
-            const float var_r = drr - dr * dr / cnt;
-            float res = var_y;
-            if (var_r > 1e-12f && cov > 0.0f) res = var_y - cov * cov / var_r;
-            res = fmaxf(res, 0.0f);
-            const unsigned long long key = ((unsigned long long)__float_as_uint(res) << 32) | g;
-            best = key < best ? key : best;
+            const uint32_t who = (__ballot_sync(kFull, take) >> (grp * kGroup)) & ((1u << kGroup) - 1u);
+            if (take) near[n_near + (uint32_t)__popc(who & ((1u << l) - 1u))] = g;
+            n_near += (uint32_t)__popc(who);
+        }
+        __syncwarp();
+        unsigned long long key = ~0ull;
+        if (act) {
+            const Trace t{s.cnt, s.sy, s.syy - s.sy * s.sy / s.cnt};
+            for (uint32_t c = l; c < n_near + n_ill; c += kGroup) {
+                const uint32_t g = c < n_near ? near[c] : w.ill[c - n_near];
+                const float res = residual(rates + (size_t)g * kPoints, vec, rows[wid][grp], keeps[wid][grp], t);
+                const unsigned long long k = ((unsigned long long)__float_as_uint(res) << 32) | g;
+                key = k < key ? k : key;
+            }
+        }
+#pragma unroll
+        for (int o = kGroup / 2; o; o >>= 1) {
+            const unsigned long long k = __shfl_xor_sync(kFull, key, o);
+            key = k < key ? k : key;
+        }
+        if (act && l == 0) {
+            idx_out[i] = (uint32_t)(key & 0xFFFFFFFFull);
+            if (res_out) res_out[i] = __uint_as_float((uint32_t)(key >> 32));
+        }
+    }
+}
+
+// The traces left over: every candidate's residual, 32 candidates at a time.
+// A trace's candidates are parted among the warps that there are for it (one
+// trace of 1308 candidates by one warp: 0.4 ms).
+constexpr int kEveryWarps = 8;
+__global__ void __launch_bounds__(kEveryWarps * 32, 2)
+    lsq_every_kernel(const float *__restrict__ y, const float *__restrict__ rates, uint32_t G, LsqWork w,
+                     uint32_t *idx_out, float *res_out) {
+    __shared__ __align__(16) float rows[kEveryWarps][kPoints];
+    __shared__ uint32_t keeps[kEveryWarps][kPoints / 32];
+    const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+    const uint32_t total = w.flags->n_every;
+    if (!total) return;
+    const uint32_t nw = gridDim.x * kEveryWarps, rounds = (G + 31u) / 32u;
+    const uint32_t most = min(rounds, max(nw / total, 1u)), each = (rounds + most - 1u) / most,
+                   parts = (rounds + each - 1u) / each;
+    const bool vec = (reinterpret_cast<uintptr_t>(rates) & 15u) == 0;
+    for (uint64_t k = blockIdx.x * kEveryWarps + wid; k < (uint64_t)total * parts; k += nw) {
+        const uint32_t i = w.every[k / parts], part = (uint32_t)(k % parts);
+        const RowStats s = w.stats[i];
+        __syncwarp();
+        load_trace(y, i, s.thr, rows[wid], keeps[wid], lane);
+        __syncwarp();
+        const Trace t{s.cnt, s.sy, s.syy - s.sy * s.sy / s.cnt};
+        unsigned long long key = ~0ull;
+        const uint32_t last = min(G, 32u * each * (part + 1u));
+        for (uint32_t g = 32u * each * part + lane; g < last; g += 32) {
+            const float res = residual(rates + (size_t)g * kPoints, vec, rows[wid], keeps[wid], t);
+            const unsigned long long x = ((unsigned long long)__float_as_uint(res) << 32) | g;
+            key = x < key ? x : key;
         }
 #pragma unroll
         for (int o = 16; o; o >>= 1) {
-            const unsigned long long v = __shfl_xor_sync(kFull, best, o);
-            best = v < best ? v : best;
+            const unsigned long long x = __shfl_xor_sync(kFull, key, o);
+            key = x < key ? x : key;
         }
         if (lane == 0) {
-            idx_out[i] = (uint32_t)(best & 0xFFFFFFFFull);
-            if (res_out) res_out[i] = __uint_as_float((uint32_t)(best >> 32));
+            Shared *const sh = reinterpret_cast<Shared *>(w.list + (size_t)i * kLsqList);
+            if (parts > 1) {
+                atomicMin(&sh->key, key);
+                __threadfence();
+                if (atomicAdd(&sh->done, 1u) + 1u < parts) continue;
+                __threadfence();
+                key = atomicMin(&sh->key, ~0ull);
+            }
+            idx_out[i] = (uint32_t)(key & 0xFFFFFFFFull);
+            if (res_out) res_out[i] = __uint_as_float((uint32_t)(key >> 32));
         }
-        __syncwarp();
     }
 }
 
@@ -527,20 +772,33 @@ cudaError_t lsq_run(const float *rates, uint32_t n_geoms, const float *y, uint32
     const uint32_t row_blocks = (n + 7u) / 8u;
     lsq_rows_kernel<<<std::min(row_blocks, full * 8u), 256, 0, st>>>(y, n, n_dev, w);
     CUtensorMap ymap, rmap;
-    if (!kmajor_map(w.Y, (int)n, kYCols, kYCols, 128, &ymap)) return cudaErrorInvalidValue;
+    if (!kmajor_map(w.Y, (int)n, kCols, kCols, 128, &ymap)) return cudaErrorInvalidValue;
     e = cudaFuncSetAttribute(lsq_estimate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kLsqSmem);
     if (e != cudaSuccess) return e;
+    const uint32_t mt = (n + 127u) / 128u;
     for (uint32_t g0 = 0; g0 < n_geoms; g0 += kLsqChunk) {
         const uint32_t ng = std::min(kLsqChunk, n_geoms - g0);
         lsq_rates_kernel<<<(ng + 7u) / 8u, 256, 0, st>>>(rates, g0, ng, w);
-        if (!kmajor_map(w.R, (int)ng, kRCols, kRCols, 128, &rmap)) return cudaErrorInvalidValue;
-        const uint64_t tiles = (uint64_t)((n + 127u) / 128u) * ((ng + 127u) / 128u);
-        lsq_estimate_kernel<<<(unsigned)std::min<uint64_t>(tiles, full), 256, kLsqSmem, st>>>(
-            ymap, rmap, n, n_dev, g0, ng, w);
+        uint32_t N = 0;
+        uint64_t least = ~0ull, tiles = 0;
+        for (uint32_t c = 32; c <= kLsqMaxN; c += 32) {
+            const uint64_t t = (uint64_t)mt * ((ng + c - 1u) / c), cost = (t + full - 1u) / full * (c + 128u);
+            if (cost < least) {
+                least = cost;
+                N = c;
+                tiles = t;
+            }
+        }
+        if (!kmajor_map(w.R, (int)ng, kCols, kCols, (int)N, &rmap)) return cudaErrorInvalidValue;
+        lsq_estimate_kernel<<<(unsigned)std::min<uint64_t>(tiles, full), kLsqThreads, kLsqSmem, st>>>(
+            ymap, rmap, rates, n, n_dev, g0, ng, N, w);
     }
-    lsq_exact_kernel<<<std::min((n + kExactWarps - 1u) / kExactWarps, full * 8u), kExactWarps * 32, 0, st>>>(
-        y, n, n_dev, rates, n_geoms, w, best_out, resid_out);
+    constexpr uint32_t kPerBlock = kExactWarps * kPerWarp;
+    lsq_exact_kernel<<<std::min((n + kPerBlock - 1u) / kPerBlock, full * 16u), kExactWarps * 32, 0, st>>>(
+        y, n, n_dev, rates, w, best_out, resid_out);
+    lsq_every_kernel<<<full * 2u, kEveryWarps * 32, 0, st>>>(
+        y, rates, n_geoms, w, best_out, resid_out);
     return cudaGetLastError();
 }
 

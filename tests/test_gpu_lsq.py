@@ -83,3 +83,25 @@ def test_judge_at_tile_edges(n, G, shift):
     buf[1:] = torch.from_numpy(rates.reshape(-1)).cuda()
     b2, r2 = INV.lsq_match(buf[1:].view(G, R.POINTS), torch.from_numpy(y).cuda())
     assert np.array_equal(b2.cpu().numpy(), best) and np.array_equal(r2.cpu().numpy().astype(np.float64), res)
+
+
+@pytest.mark.parametrize("n,G", [(3, 33), (16, 200), (130, 161), (40, 2100)])
+def test_judge_by_few_points(n, G):
+    """Rows that a trace's five dropped points can take most or all of (their
+    residuals' lower bounds say nothing), and traces that fit so many rows
+    equally well that their list overflows, between traces that do not."""
+    rng = np.random.Generator(np.random.PCG64(77 * n + G))
+    rates = _rows(G, rng)
+    for k in range(0, G, 2):
+        rates[k] = 0.0
+        rates[k, rng.integers(0, R.POINTS, 1 + k // 2 % 12)] = rng.choice([0.25, 0.5, 1.0])
+    y = rates[rng.integers(0, G, n)] + 0.02 * rng.standard_normal((n, R.POINTS))
+    y[1::3] = rng.standard_normal((len(y[1::3]), R.POINTS)) + 500.0
+    y = y.astype(np.float32)
+    best, res = INV.lsq_match(torch.from_numpy(rates).cuda(), torch.from_numpy(y).cuda())
+    best, res = best.cpu().numpy(), res.cpu().numpy().astype(np.float64)
+    assert best.min() >= 0 and best.max() < G
+    want, bound = _exact(rates, y)
+    i = np.arange(n)
+    assert (np.abs(res - want[i, best]) <= bound[i, best]).all()
+    assert (res <= (want + bound).min(1)).all()
