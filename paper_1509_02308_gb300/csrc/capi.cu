@@ -126,6 +126,9 @@ constexpr double kAffinityMinNsPerSm = 20.0e6;
 // launch): the costliest kIsolateMax within kIsolateFrac of the costliest.
 constexpr double kIsolateFrac = 0.6;
 constexpr size_t kIsolateMax = 12;
+// A matcher's groups are one launch more (2 us): worth it from a few candidates
+// to a group on (1308 candidates x 108 traces: 312 -> 188 us a match).
+constexpr uint32_t kUniformGroupGeoms = 16;
 // ... in plans whose longest unit takes this long: a second launch beside the
 // main one, forked and joined, costs the host and the GPU some 6 us.
 constexpr double kIsolateMinNs = 1.0e5;
@@ -580,7 +583,11 @@ struct pchase_sim_plan {
     std::vector<UniformTask> utasks;
     uint32_t uclass[kUniformClasses] = {};
     std::vector<uint32_t> trace_unit;
-    size_t off_bad = 0, off_utasks = 0, off_tunit = 0;
+    // a matcher's plan: groups of items with the same words, their candidates,
+    // and the units of the other items
+    std::vector<UniformGroup> ugroups;
+    std::vector<uint32_t> ucands, urest;
+    size_t off_bad = 0, off_utasks = 0, off_tunit = 0, off_ugroups = 0, off_ucands = 0, off_urest = 0;
     double gwork_live[kUnitGroups] = {};  // (ulayout's)
     double gwork_main[kUnitGroups] = {};  // estimated work of each unit group in the
                                           // slot-mix launch
@@ -656,6 +663,46 @@ uint32_t uniform_bits(const pchase_geom &G, const SimItem &it) {
     return it.len <= kUniformMatchLen ? both : 1u << kUniformBit;
 }
 
+// The matcher's groups: by trace, line size, and whether the later passes miss
+// nothing (or only in played sets) or everything.
+void plan_uniform_groups(pchase_sim_plan *p) {
+    constexpr uint32_t kKinds = 64;  // 32 line sizes x 2
+    std::vector<uint32_t> count((size_t)p->n_trace * kKinds), first;
+    std::vector<std::pair<uint32_t, uint32_t>> in;  // {group key, unit}
+    for (size_t k = 0; k < p->items.size(); ++k) {
+        const SimItem &it = p->items[k];
+        if (!it.lead) continue;
+        const uint32_t lb = it.lsh & 255u;
+        bool grouped = ((it.lsh >> kUniformMatchBit) & 1u) && !((it.lsh >> 8) & 255u) && lb < 32;
+        uint32_t kind = 0;
+        if (grouped) {
+            const HostChain c(it, p->geoms[it.cand].sets);
+            kind = (it.policy >= PCHASE_RANDOM && it.ways > 1) || c.over == 0 ? 0u : 1u;
+            grouped = kind == 0 || c.over == c.Tp;
+        }
+        if (!grouped) {
+            p->urest.push_back((uint32_t)k);
+            continue;
+        }
+        const uint32_t key = it.obs * kKinds + 2u * lb + kind;
+        count[key] += 1;
+        in.push_back({key, (uint32_t)k});
+    }
+    first.assign(count.size(), 0);
+    uint32_t at = 0;
+    for (size_t key = 0; key < count.size(); ++key) {
+        first[key] = at;
+        at += count[key];
+    }
+    std::vector<uint32_t> next = first;
+    p->ucands.resize(in.size());
+    for (const auto &e : in) {
+        uint32_t &to = next[e.first];
+        if (to == first[e.first]) p->ugroups.push_back({e.second, to, count[e.first]});
+        p->ucands[to++] = p->items[e.second].cand;
+    }
+}
+
 // Tasks of the played sets, and the traces to check.
 void plan_uniform(pchase_sim_plan *p) {
     struct Costed {
@@ -724,6 +771,7 @@ void plan_uniform(pchase_sim_plan *p) {
         p->utasks.push_back(c.t);
         p->uclass[c.cls] += 1;
     }
+    if (p->cross && p->n_geom >= kUniformGroupGeoms) plan_uniform_groups(p);
 }
 
 // Unit-group homes of the slot-mix launch: `sites` SMs (CTA b sits on site
@@ -827,11 +875,13 @@ int plan_runtime(pchase_sim_plan *p) {
     }
     // played sets run beside the simulator's units, the large ones beside the
     // small ones (where every item may be a uniform chain the units mostly have
-    // nothing to do, and one stream less is needed)
+    // nothing to do, and one stream less is needed), and beside the matcher's
+    // other launches
     const bool large = p->utasks.size() > p->uclass[0];
-    if (!p->utasks.empty() && (large || !p->uniform_every))
+    const bool beside = !p->uniform_every || !p->ugroups.empty();
+    if (!p->utasks.empty() && (large || beside))
         PCHASE_CUDA(cudaEventCreateWithFlags(&p->ufork, cudaEventDisableTiming), "cudaEventCreate");
-    if (p->uclass[0] && !p->uniform_every) {
+    if (p->uclass[0] && beside) {
         PCHASE_CUDA(cudaStreamCreateWithFlags(&p->uside, cudaStreamNonBlocking), "cudaStreamCreate");
         PCHASE_CUDA(cudaEventCreateWithFlags(&p->ujoin, cudaEventDisableTiming), "cudaEventCreate");
     }
@@ -865,11 +915,25 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
                                         p->n_trace, p->n_explicit, p->max_trace_len, p->n_items,
                                         o.miss_counts, reinterpret_cast<uint32_t *>(w), bad, p->sms, st),
                     "uniform check");
-        PCHASE_CUDA(launch_uniform_out(items, p->n_units, p->max_trace_len, p->sms, o,
-                                       reinterpret_cast<uint32_t *>(w + kLiveOffset), st),
+        uint32_t *const live = reinterpret_cast<uint32_t *>(w + kLiveOffset);
+        // the played sets add bits to the words, or (the matcher) only to the
+        // distances, beside the launches that work these out: 188 -> 177 us a
+        // match of 1308 candidates x 108 traces
+        if (p->ufork && o.dist) PCHASE_CUDA(cudaEventRecord(p->ufork, st), "cudaEventRecord");
+        const bool grouped = o.dist && !p->ugroups.empty();
+        if (grouped)
+            PCHASE_CUDA(launch_uniform_match(items, reinterpret_cast<const UniformGroup *>(w + p->off_ugroups),
+                                             (uint32_t)p->ugroups.size(),
+                                             reinterpret_cast<const uint32_t *>(w + p->off_ucands), p->sms,
+                                             o, live, st),
+                        "uniform groups");
+        PCHASE_CUDA(launch_uniform_out(items,
+                                       grouped ? reinterpret_cast<const uint32_t *>(w + p->off_urest) : nullptr,
+                                       grouped ? p->urest.size() : p->n_units, p->max_trace_len, p->sms, o,
+                                       live, st),
                     "uniform words");
         const UniformTask *const tasks = reinterpret_cast<const UniformTask *>(w + p->off_utasks);
-        if (p->ufork) PCHASE_CUDA(cudaEventRecord(p->ufork, st), "cudaEventRecord");
+        if (p->ufork && !o.dist) PCHASE_CUDA(cudaEventRecord(p->ufork, st), "cudaEventRecord");
         if (p->uside2) {
             PCHASE_CUDA(cudaStreamWaitEvent(p->uside2, p->ufork, 0), "cudaStreamWaitEvent");
             uint32_t first = (uint32_t)p->utasks.size();
@@ -1733,6 +1797,12 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
     off = align256(off + p->utasks.size() * sizeof(UniformTask));
     p->off_tunit = off;
     off = align256(off + p->trace_unit.size() * sizeof(uint32_t));
+    p->off_ugroups = off;
+    off = align256(off + p->ugroups.size() * sizeof(UniformGroup));
+    p->off_ucands = off;
+    off = align256(off + p->ucands.size() * sizeof(uint32_t));
+    p->off_urest = off;
+    off = align256(off + p->urest.size() * sizeof(uint32_t));
     p->ws_bytes = off;
     *plan_out = p;
     return PCHASE_OK;
@@ -1746,6 +1816,8 @@ size_t pchase_sim_plan_upload_bytes(const pchase_sim_plan *plan) {
            plan->seg_offsets.size() * sizeof(uint64_t) +
            plan->obs_word_offsets.size() * sizeof(uint64_t) + 2 * sizeof(uint64_t) +
            plan->utasks.size() * sizeof(UniformTask) + plan->trace_unit.size() * sizeof(uint32_t) +
+           plan->ugroups.size() * sizeof(UniformGroup) +
+           (plan->ucands.size() + plan->urest.size()) * sizeof(uint32_t) +
            (plan->jobs.empty() ? 0
                                : plan->jobs.size() * sizeof(StreamJob) +
                                      plan->seg_job.size() * sizeof(uint32_t) +
@@ -1946,6 +2018,18 @@ int pchase_sim_plan_upload(const pchase_sim_plan *plan, void *workspace, size_t 
                                     plan->trace_unit.size() * sizeof(uint32_t),
                                     cudaMemcpyHostToDevice, st),
                     "upload uniform traces");
+    if (!plan->ugroups.empty()) {
+        PCHASE_CUDA(cudaMemcpyAsync(w + plan->off_ugroups, plan->ugroups.data(),
+                                    plan->ugroups.size() * sizeof(UniformGroup), cudaMemcpyHostToDevice, st),
+                    "upload uniform groups");
+        PCHASE_CUDA(cudaMemcpyAsync(w + plan->off_ucands, plan->ucands.data(),
+                                    plan->ucands.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, st),
+                    "upload uniform candidates");
+    }
+    if (!plan->urest.empty())
+        PCHASE_CUDA(cudaMemcpyAsync(w + plan->off_urest, plan->urest.data(),
+                                    plan->urest.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, st),
+                    "upload ungrouped units");
     if (!plan->jobs.empty()) {
         PCHASE_CUDA(cudaMemcpyAsync(w + plan->off_jobs, plan->jobs.data(),
                                     plan->jobs.size() * sizeof(StreamJob), cudaMemcpyHostToDevice, st),

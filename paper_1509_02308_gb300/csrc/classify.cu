@@ -57,8 +57,8 @@ struct ObsMeta {
 // or where the bucket arithmetic is not regular, the 2 * keep buckets of the
 // pigeonhole method follow, kGapBuckets of them at a time.  Bound by the
 // passes over shared memory and a dozen cluster barriers: 64 observations of
-// 16K-64K latencies take @@ us against 288 us as four launches, one CTA per
-// observation; one of 177K latencies, as the matcher pools, @@ against 458 us.
+// 16K-64K latencies take 40 us against 288 us as four launches, one CTA per
+// observation; one of 177K latencies, as the matcher pools, 39 against 458 us.
 constexpr uint32_t kGapBuckets = 4096;
 constexpr uint32_t kClusterThreads = 512;
 constexpr uint32_t kClusterMaxKeys = 49152;  // of one CTA (192 KB, beside 33 KB of buckets)

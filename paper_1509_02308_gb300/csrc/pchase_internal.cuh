@@ -248,6 +248,12 @@ struct UniformTask {
     uint32_t count;
     uint32_t lanes;
 };
+// Matcher items whose words are the same: one trace, one line size, and every
+// run head of the later passes missing or none.
+struct UniformGroup {
+    uint32_t unit;          // of any of them
+    uint32_t first, count;  // their candidates in the plan's list
+};
 
 // Head streams (streams.cu).  Every item split by sets into K parts is one
 // job: its trace is cut into segments of kSegAccesses accesses, one warp per
@@ -301,8 +307,14 @@ cudaError_t launch_uniform_prep(const SimItem *items, const uint32_t *trace_unit
                                 uint64_t n_explicit, uint64_t max_len, uint64_t n_items,
                                 uint64_t *counts, uint32_t *head, uint32_t *bad, int sms,
                                 cudaStream_t st);
-cudaError_t launch_uniform_out(const SimItem *items, uint64_t n_units, uint64_t max_len, int sms,
-                               const SimOut &out, uint32_t *live, cudaStream_t st);
+// (units: the n_units units to do, NULL for all)
+cudaError_t launch_uniform_out(const SimItem *items, const uint32_t *units, uint64_t n_units,
+                               uint64_t max_len, int sms, const SimOut &out, uint32_t *live,
+                               cudaStream_t st);
+// The distances of the matcher's groups, every observation's.
+cudaError_t launch_uniform_match(const SimItem *items, const UniformGroup *groups, uint32_t n_groups,
+                                 const uint32_t *cands, int sms, const SimOut &out, uint32_t *live,
+                                 cudaStream_t st);
 cudaError_t launch_uniform_play(const SimItem *items, const UniformTask *tasks, uint32_t n_tasks,
                                 uint32_t smem_bytes, const SimOut &out, cudaStream_t st);
 // The head streams of a plan's split items (three launches on `st`).

@@ -25,10 +25,10 @@
 // kernel writes a bit per access; the played sets are chains of dependent
 // events, so they are cut into one warp per set (or 32 small sets) and the
 // costliest start first.  Against stepping the same items in the units, the
-// 4096-item batch (0.64 G accesses, index arrays) went from 43.3 to 18.0 ms
-// (what is left is the longest played sets), a 384-item batch of short traces
-// from 519 to 179 us, matching 1308 candidates against 108 traces from 3.54 to
-// 0.88 ms.
+// 4096-item batch (0.64 G accesses, index arrays) went from 43.3 to 13.9 ms
+// (12.7 of them the longest played sets), a 384-item batch of short traces
+// from 519 to 155 us, matching 1308 candidates against 108 traces from 3.54 to
+// 0.18 ms.
 #include <algorithm>
 
 #include "pchase_internal.cuh"
@@ -250,9 +250,10 @@ __global__ void __launch_bounds__(256) uniform_prep_kernel(const SimItem *__rest
 // other one is cleared for the simulator's units.  A warp takes 32 words at a
 // time, one per lane.  A lane goes through its word's run heads (its accesses,
 // where each is one): up to 32 short turns for 32 words, where a vote per word
-// took 32 longer ones (texture and Fermi sweeps of 9.6K items: 239 us with the
-// votes, @@ so; the 4096-item batch 1519 -> @@ us).
+// took 32 longer ones (a pass over the texture and Fermi sweeps of 9.6K items
+// 284 -> 91 us; this kernel on the 4096-item batch 1519 -> 421 us).
 __global__ void __launch_bounds__(256) uniform_out_kernel(const SimItem *__restrict__ items,
+                                                          const uint32_t *__restrict__ units,
                                                           uint64_t n_units, uint32_t parts,
                                                           SimOut out, uint32_t *live) {
     const uint32_t lane = threadIdx.x & 31u;
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(256) uniform_out_kernel(const SimItem *__restr
          task < n_units * parts; task += nw) {
         const uint64_t ui = task / parts;
         const uint32_t part = (uint32_t)(task % parts);
-        const SimItem it = items[ui];
+        const SimItem it = items[units ? units[ui] : ui];
         if (!it.lead) continue;
         const bool mine = taken(it, out.uniform_bad) &&
                           (!ham || ((it.lsh >> kUniformMatchBit) & 1u));
@@ -337,6 +338,57 @@ __global__ void __launch_bounds__(256) uniform_out_kernel(const SimItem *__restr
                 if (aft) atomicAdd(mc + 1, (unsigned long long)aft);
             }
         }
+    }
+}
+
+// The matcher's groups: a candidate's capacity decides only whether the run
+// heads after the first pass all miss, all hit or are split by class, so most
+// candidates of one line size predict the same words for a trace (1308
+// candidates x 108 traces, 141K items: 864 groups).  A CTA works out a group's
+// distance from one observation and adds it to its candidates' (161 us item by
+// item; 8 us so, and 30 for the items that have a word of their own).
+__global__ void __launch_bounds__(256) uniform_match_kernel(const SimItem *__restrict__ items,
+                                                            const UniformGroup *__restrict__ groups,
+                                                            uint32_t n_groups,
+                                                            const uint32_t *__restrict__ cands,
+                                                            SimOut out, uint32_t *live) {
+    __shared__ uint32_t sums[8];
+    const uint32_t tid = threadIdx.x, rep = blockIdx.y;
+    const uint32_t *const observed = out.observed + rep * out.rep_obs_stride;
+    unsigned long long *const dist =
+        reinterpret_cast<unsigned long long *>(out.dist + rep * out.rep_dist_stride);
+    for (uint32_t b = blockIdx.x; b < n_groups; b += gridDim.x) {
+        const UniformGroup g = groups[b];
+        const SimItem &it = items[g.unit];
+        if (!taken(it, out.uniform_bad)) {
+            if (tid == 0) atomicOr(live, 1u);
+            continue;
+        }
+        Chain ch(it);
+        ch.prepare_first();
+        const bool held = ch.rnd || ch.thr == 0, all = !held;
+        const bool ones = all && ch.strided && ch.nl > 1;
+        const uint32_t *const obs = observed + out.obs_word_offsets[it.obs];
+        const uint32_t nwords = (ch.len + 31u) >> 5;
+        uint32_t d = 0;
+        for (uint32_t w = tid; w < nwords; w += 256u) {
+            const uint32_t t = w << 5;
+            const uint32_t valid = ch.len - t >= 32u ? kFull : (1u << (ch.len - t)) - 1u;
+            uint32_t word = 0;
+            if (ones) word = kFull;
+            else if (!held || t < ch.per) word = ch.word(t, held, all);
+            d += (uint32_t)__popc((word ^ obs[w]) & valid);
+        }
+        d = __reduce_add_sync(kFull, d);
+        if ((tid & 31u) == 0) sums[tid >> 5] = d;
+        __syncthreads();
+        uint32_t total = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) total += sums[q];
+        if (total)
+            for (uint32_t c = tid; c < g.count; c += 256u)
+                atomicAdd(dist + cands[g.first + c], (unsigned long long)total);
+        __syncthreads();
     }
 }
 
@@ -693,15 +745,26 @@ cudaError_t launch_uniform_prep(const SimItem *items, const uint32_t *trace_unit
     return cudaGetLastError();
 }
 
-cudaError_t launch_uniform_out(const SimItem *items, uint64_t n_units, uint64_t max_len, int sms,
-                               const SimOut &out, uint32_t *live, cudaStream_t st) {
+cudaError_t launch_uniform_match(const SimItem *items, const UniformGroup *groups, uint32_t n_groups,
+                                 const uint32_t *cands, int sms, const SimOut &out, uint32_t *live,
+                                 cudaStream_t st) {
+    const uint32_t blocks = std::min(n_groups, (uint32_t)std::max(sms, 1) * 8u);
+    uniform_match_kernel<<<dim3(blocks, out.n_rep ? out.n_rep : 1u), 256, 0, st>>>(
+        items, groups, n_groups, cands, out, live);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_uniform_out(const SimItem *items, const uint32_t *units, uint64_t n_units,
+                               uint64_t max_len, int sms, const SimOut &out, uint32_t *live,
+                               cudaStream_t st) {
+    if (!n_units) return cudaSuccess;
     // (a part is 32 words at least)
     const uint64_t full = (uint64_t)std::max(sms, 1) * 64;
     uint32_t parts = 1;
     while (parts < 32 && n_units * parts < 2 * full && max_len > 1024ull * parts) parts *= 2;
     const uint64_t warps = n_units * parts;
     const uint64_t blocks = std::min<uint64_t>((warps + 7) / 8, (uint64_t)std::max(sms, 1) * 8);
-    uniform_out_kernel<<<(unsigned)blocks, 256, 0, st>>>(items, n_units, parts, out, live);
+    uniform_out_kernel<<<(unsigned)blocks, 256, 0, st>>>(items, units, n_units, parts, out, live);
     return cudaGetLastError();
 }
 

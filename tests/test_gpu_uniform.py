@@ -156,6 +156,36 @@ def test_matcher_over_uniform_chains():
         assert np.array_equal(x, y)
 
 
+@pytest.mark.parametrize("n_geom", [15, 16, 70])
+def test_matcher_groups_candidates(n_geom):
+    """Candidates whose words are the same are matched together: line sizes,
+    classes that overflow in part, mappings and unequal sets between them, one
+    line to a pass, index arrays of which one is not the chain it claims."""
+    runs = [W.Run(n // 4, s // 4, ln, n // s) for n, s, ln in
+            ((4096, 128, 31), (8192, 32, 1025), (12416, 128, 300), (64, 64, 77), (20480, 4, 12000),
+             (12288, 4096, 64), (16384, 128, 640))]
+    flat, offs = api.pchase_build_batch(runs)
+    flat[int(offs[6]) + 200] = 0
+    traces = [(flat[int(offs[i]):int(offs[i + 1])] if i % 2 == 0 else None, r.length, r.warmup, r.n_elems,
+               r.stride) for i, r in enumerate(runs)]
+    cands = [W.Geom(C, b, a, C // (a * b), p, 3 * a) for b in (32, 128) for a in (1, 2, 4, 8)
+             for C in (4096, 8192, 12288, 16384) for p in (0, 1, 2)]
+    cands = cands[::96 // n_geom][:n_geom - 2] + [W.Geom(8192, 32, 4, 64, 0, 1, mapping=2),
+                                                  W.Geom((3 * 4 + 5) * 128, 128, 4, 3, 0, 1, extra=5)]
+    assert len(cands) == n_geom
+    rng = np.random.Generator(np.random.PCG64(n_geom))
+    n = sum(r.length for r in runs)
+    lat = torch.from_numpy((100.0 + 300.0 * (rng.random((2, n)) < 0.4)).astype(np.float32)).cuda()
+    res = []
+    for tune in (None, UNITS):
+        plan = api.SimPlan(cands, traces, tune=tune)
+        d1, p1 = plan.infer(lat[0])
+        d2, p2 = api.infer_batch(plan, lat)
+        res.append([x.cpu().numpy() for x in (d1, p1, d2, p2)])
+    for x, y in zip(*res):
+        assert np.array_equal(x, y)
+
+
 def test_uniform_run_captured_in_a_graph():
     runs = [W.Run(n // 4, 32, 4 * (n // 128), n // 128) for n in (8192, 16512, 20480)]
     flat, offs = api.pchase_build_batch(runs)
