@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -595,6 +596,9 @@ struct pchase_sim_plan {
     cudaStream_t side = nullptr, side2 = nullptr, uside = nullptr, uside2 = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr, fork2 = nullptr, join2 = nullptr;
     cudaEvent_t ufork = nullptr, ujoin = nullptr, ujoin2 = nullptr;
+    // one run at a time records and waits for the events above: threads may
+    // run a plan on streams and workspaces of their own
+    std::mutex launching;
 
     ~pchase_sim_plan() {
         if (side) cudaStreamDestroy(side);
@@ -894,6 +898,7 @@ int plan_runtime(pchase_sim_plan *p) {
 }
 
 int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st) {
+    const std::lock_guard<std::mutex> lock(p->launching);
     int rc = plan_runtime(p);
     if (rc) return rc;
     uint8_t *w = static_cast<uint8_t *>(ws);

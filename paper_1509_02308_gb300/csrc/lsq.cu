@@ -88,8 +88,9 @@ struct LsqWork {
     Cand *cand;
     Flags *flags;
     size_t bytes;
+    // (the caller's buffer may start anywhere; the tensor maps' rows may not)
     LsqWork(void *base, size_t n) {
-        uint8_t *p = static_cast<uint8_t *>(base);
+        uint8_t *const p = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(base) + 255) & ~uintptr_t(255));
         size_t o = 0;
         auto take = [&](size_t b) {
             uint8_t *q = p + o;
@@ -106,7 +107,7 @@ struct LsqWork {
         every = reinterpret_cast<uint32_t *>(take(n * 4));
         ill = reinterpret_cast<uint32_t *>(take(kLsqIll * 4));
         flags = reinterpret_cast<Flags *>(take(sizeof(Flags)));
-        bytes = o;
+        bytes = o + 255;
     }
 };
 
