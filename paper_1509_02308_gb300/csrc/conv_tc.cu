@@ -40,7 +40,6 @@ constexpr int kTileRows = 128;
 constexpr int kGroups = 18;                           // 8-row groups per slab plane
 constexpr uint32_t kPlaneBytes = kGroups * 8 * 128;   // 18 KB
 constexpr uint32_t kSlabBytes = 2 * kPlaneBytes;      // 36 KB
-constexpr int kSlabs = 3;
 constexpr uint32_t kWBytes = kTaps * kCh * 128;       // 40 KB
 constexpr uint32_t kTmemCols = 128;                   // two 64-column accumulators
 
@@ -584,32 +583,58 @@ __global__ void __launch_bounds__(128, 1)
 // outputs go to global memory.  A layer-3 position q of trace b lands in row
 // 8 ((q >> 1) + 1) + 2b when q <= 33 and in row 8 ((q >> 1) - 15) + 2b + 1
 // when q >= 30 (plane q & 1); rows 2b of group 0 and 2b + 1 of group 17 are
-// the zero padding, written once.  Layer-3 input slabs stream in by cp.async
-// (three buffers).
-constexpr int kL34Threads = 512;  // the first 256 load slabs; all run the epilogues
-constexpr uint32_t kL34TmemCols = 256;  // accumulators: layer-3 tiles A, B and layer 4
-constexpr uint32_t kL34Smem = 1024 + 2 * kWBytes + kSlabs * kSlabBytes + kSlabBytes + 64;
+// the zero padding, written once.
+//
+// Roles: sixteen epilogue warps, one thread that loads, one that issues the
+// MMAs.  A layer-3 slab is two planes, each a stage of its own in a ring of
+// five (three TMA loads: groups 1-16, and the first and last group, whose rows
+// are the neighbouring blocks of 32 positions', zeros where the trace ends).
+// Layer 3's accumulators are double-buffered and its MMAs run up to two
+// iterations ahead of the epilogue, so a stage is free again as soon as its
+// tile's MMAs are done; layer 4's are double-buffered too, and its epilogue
+// runs under the next iteration's layer-4 MMAs.  The outputs go through shared
+// memory and leave as TMA stores, one per lane quarter (4 warps, 32 rows).
+// With cp.async loads by eight of the warps, one accumulator a tile, block
+// barriers between the phases and rows stored from registers the network took
+// 1325 us for 65,536 traces, 1210 us so.  An iteration moves 80 KB through
+// HBM and some 500 KB through an SM's shared memory (MMA operands 360 KB,
+// loads, slab and output writes and reads): those two bound it about equally.
+constexpr int kL34Epi = 16;                        // epilogue warps
+constexpr int kL34Threads = 32 * (kL34Epi + 2);
+constexpr int kL34Planes = 5;                      // ring stages
+constexpr uint32_t kL34TmemCols = 512;  // layer 3: 128 p + 64 X; layer 4: 256 + 64 p
+constexpr uint32_t kL34Bars = 2 * kL34Planes + 4 + 2 + 1;
+constexpr uint32_t kL34Smem =
+    1024 + 2 * kWBytes + kL34Planes * kPlaneBytes + kSlabBytes + kOutTile + 8 * kL34Bars + 16;
+static_assert(kL34Smem <= 232448, "shared memory");
+
+__device__ __forceinline__ void mma_commit_to(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+                 : "memory");
+}
 
 __global__ void __launch_bounds__(kL34Threads, 1)
-    conv34_tc_kernel(const __nv_bfloat16 *__restrict__ x, int nb,
-                     const __nv_bfloat16 *__restrict__ W3, const float *__restrict__ bias3,
+    conv34_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap emap,
+                     int nb, const __nv_bfloat16 *__restrict__ W3, const float *__restrict__ bias3,
                      const __nv_bfloat16 *__restrict__ W4, const float *__restrict__ bias4,
-                     __nv_bfloat16 *__restrict__ out, uint32_t *__restrict__ status) {
-    constexpr int kLin3 = 128, kL3 = 64, kL4 = 32;
+                     const __grid_constant__ CUtensorMap omap, uint32_t *__restrict__ status) {
     extern __shared__ uint8_t dsm[];
     const uint32_t raw = smem_u32(dsm);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *const gbase = dsm + (base - raw);
     const uint32_t sW3 = base, sW4 = base + kWBytes;
-    const uint32_t sSlab = base + 2 * kWBytes;         // layer-3 input slabs
-    const uint32_t sL4 = sSlab + kSlabs * kSlabBytes;  // layer-4 input slab
-    const uint32_t sBar = sL4 + kSlabBytes;            // mbarriers: tile A, tile B, layer 4
-    uint32_t *const tslot = reinterpret_cast<uint32_t *>(gbase + (sBar - base) + 32);
+    const uint32_t sRing = base + 2 * kWBytes;                // planes of layer-3 input slabs
+    const uint32_t sL4 = sRing + kL34Planes * kPlaneBytes;    // layer-4 input slab
+    const uint32_t sOut = sL4 + kSlabBytes;                   // output tile
+    // barriers: plane loaded [5], plane free [5], layer-3 tile done [2 p + X],
+    // layer-4 tile done [p], layer-4 slab written
+    const uint32_t full0 = sOut + kOutTile, free0 = full0 + 8u * kL34Planes,
+                   done3 = free0 + 8u * kL34Planes, done4 = done3 + 32u, ready4 = done4 + 16u;
+    uint32_t *const tslot = reinterpret_cast<uint32_t *>(gbase + (ready4 + 8u - base));
+    volatile uint32_t *const abort_flag = tslot + 1;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int M3 = nb * kL3, M4 = nb * kL4;
-    const int n4 = (M4 + kTileRows - 1) / kTileRows;  // iterations of 4 traces
-    const int n3 = 2 * n4;                            // layer-3 tiles: 2 it and 2 it + 1
+    const int iters = (nb - 1) / 4 + 1;  // of 4 traces
 
     for (int e = tid; e < kTaps * kCh * 8; e += kL34Threads) {
         const int k = e >> 9, co = (e >> 3) & 63, c = e & 7;
@@ -619,28 +644,6 @@ __global__ void __launch_bounds__(kL34Threads, 1)
         cp_async16(sW4 + off, W4 + src, true);
     }
     cp_async_commit();
-
-    const int ld_c = tid & 7, ld_i = (tid >> 3) & 7, ld_pl = (tid >> 6) & 1, ld_h = tid >> 7;
-    const int ld_g0 = ld_h * (kGroups / 2);
-    auto load_slab = [&](int buf, int u) {
-        if (u < n3 && tid < 256) {
-            const int mi = u * kTileRows + 16 * ld_i;
-            const int b = mi / kL3, p0 = mi - b * kL3;
-            const bool row_ok = mi < M3;
-            const int q0 = 2 * p0 + 2 * (ld_g0 - 1) + ld_pl;
-            const __nv_bfloat16 *src = x + ((size_t)(row_ok ? b : 0) * kLin3) * kCh + ld_c * 8;
-            const uint32_t dst = sSlab + buf * kSlabBytes + ld_pl * kPlaneBytes +
-                                 (8 * ld_g0 + ld_i) * 128 + ((ld_c ^ ld_i) << 4);
-#pragma unroll
-            for (int gg = 0; gg < kGroups / 2; ++gg) {
-                const int q = q0 + 2 * gg;
-                const bool ok = row_ok && q >= 0 && q < kLin3;
-                cp_async16(dst + gg * 1024, ok ? src + (size_t)q * kCh : x, ok);
-            }
-        }
-        cp_async_commit();  // one group per call, empty or not
-    };
-
     // the layer-4 slab's padding rows (never written again)
     if (tid < 2 * 4 * 2 * 8) {
         const int pl = tid >> 6, b = (tid >> 4) & 3, which = (tid >> 3) & 1, c = tid & 7;
@@ -649,9 +652,11 @@ __global__ void __launch_bounds__(kL34Threads, 1)
                                    ((c ^ (row & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
     }
     if (tid == 0) {
-        for (int q = 0; q < 3; ++q)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sBar + 8 * q) : "memory");
+        for (uint32_t q = 0; q + 1 < kL34Bars; ++q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8 * q) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(ready4), "r"(kL34Epi) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        *abort_flag = 0;
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -660,143 +665,239 @@ __global__ void __launch_bounds__(kL34Threads, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    load_slab(0, 2 * (int)blockIdx.x);
-    load_slab(1, 2 * (int)blockIdx.x + 1);
-    load_slab(2, 2 * ((int)blockIdx.x + (int)gridDim.x));
+    cp_async_wait_all();
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
 
-    // one thread: the 20 MMAs of a tile from slab a0 with weights sw into d
-    auto mma_tile = [&](uint32_t d, uint32_t slab, uint32_t sw, uint32_t bar) {
+    if (warp == kL34Epi) {
+        // ---------------- loads: planes are numbered through all of this CTA's
+        // tiles; plane b is in stage b mod 5
+        if (lane == 0) {
+            uint32_t b = 0, q = 0, par = 1;
+            for (int it = blockIdx.x; it < iters && !*abort_flag; it += (int)gridDim.x) {
+                for (int k = 0; k < 4; ++k, ++b) {
+                    if (!mbar_wait(free0 + 8u * q, par)) {
+                        *abort_flag = 1;
+                        break;
+                    }
+                    const int trace = 4 * it + 2 * (k >> 1), pl = k & 1;
+                    const uint32_t st = sRing + q * kPlaneBytes, bar = full0 + 8u * q;
+                    mbar_expect_tx(bar, kPlaneBytes);
+                    tma_load_5d(st + 1024u, &xmap, 0, 0, trace, 0, pl, bar);
+                    tma_load_5d(st, &emap, 0, -1, trace, 15, pl, bar);
+                    tma_load_5d(st + 17u * 1024u, &emap, 0, 1, trace, 0, pl, bar);
+                    if (++q == kL34Planes) {
+                        q = 0;
+                        par ^= 1u;
+                    }
+                }
+            }
+            // loads in flight land before the CTA leaves
+            for (uint32_t k = b > kL34Planes ? b - kL34Planes : 0u; k < b; ++k)
+                mbar_wait(full0 + 8u * (k % kL34Planes), (k / kL34Planes) & 1u);
+        }
+    } else if (warp == kL34Epi + 1) {
+        // ---------------- MMAs
+        if (lane == 0) {
+            uint32_t b = 0;
+            bool ok = true;
+            auto tap = [&](uint32_t d, int k, uint32_t plane, uint32_t sw) {
+                const uint32_t a0 = plane + (uint32_t)(k >> 1) * 1024u, b0 = sw + (uint32_t)k * 8192u;
 #pragma unroll
-        for (int k = 0; k < kTaps; ++k) {
-            const uint32_t a0 = slab + (uint32_t)(k & 1) * kPlaneBytes + (uint32_t)(k >> 1) * 1024u;
-            const uint32_t b0 = sw + (uint32_t)k * 8192u;
+                for (int s = 0; s < 4; ++s)
+                    mma_bf16(d, sw128_desc(a0 + 32u * s), sw128_desc(b0 + 32u * s), (k | s) != 0 ? 1u : 0u);
+            };
+            // both layer-3 tiles of this CTA's iteration j
+            auto layer3 = [&](int j) {
+                for (uint32_t X = 0; ok && X < 2; ++X) {
+                    const uint32_t q0 = b % kL34Planes, q1 = (b + 1u) % kL34Planes;
+                    ok = mbar_wait(full0 + 8u * q0, (b / kL34Planes) & 1u) &&
+                         mbar_wait(full0 + 8u * q1, ((b + 1u) / kL34Planes) & 1u);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t p0 = sRing + q0 * kPlaneBytes, p1 = sRing + q1 * kPlaneBytes;
+                    const uint32_t buf = 2u * ((uint32_t)j & 1u) + X;
 #pragma unroll
-            for (int s = 0; s < 4; ++s)
-                mma_bf16(d, sw128_desc(a0 + 32u * s), sw128_desc(b0 + 32u * s),
-                         (k | s) != 0 ? 1u : 0u);
-        }
-        asm volatile(
-            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-            : "memory");
-    };
-    // warp w reads TMEM lane quarter w mod 4 (its hardware quarter) and
-    // columns 16 (w / 4) .. + 15: a thread holds 16 values of one tile row
-    const int quarter = warp & 3, colq = warp >> 2;
-    const int r = quarter * 32 + lane;          // this thread's TMEM lane
-    const int mt = 16 * (r & 7) + (r >> 3);     // ... and the tile row it holds
-    const uint32_t lane_off = ((uint32_t)(quarter * 32) << 16) + (uint32_t)colq * 16u;
-    // bias + GELU of this thread's 16 columns of accumulator acc, as BF16 pairs
-    auto finish = [&](uint32_t acc, const float *bias, uint32_t (&pk)[8]) {
-        uint32_t v[16];
-        tmem_ld16(tmem + acc + lane_off, v);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    for (int k = 0; k < kTaps; ++k) tap(tmem + 64u * buf, k, (k & 1) ? p1 : p0, sW3);
+                    mma_commit_to(free0 + 8u * q0);
+                    mma_commit_to(free0 + 8u * q1);
+                    mma_commit_to(done3 + 8u * buf);
+                    b += 2;
+                }
+            };
+            const int mine = ((int)blockIdx.x < iters)
+                                 ? (iters - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+            for (int j = 0; j < 2 && j < mine; ++j) layer3(j);
+            int sent = 0;
+            for (int j = 0; ok && j < mine && !*abort_flag; ++j) {
+                // the slab of iteration j is written, and every epilogue warp has
+                // read iteration j's layer-3 sums and iteration j - 2's layer-4 sums
+                ok = mbar_wait(ready4, (uint32_t)j & 1u);
+                if (!ok) break;
+                tc_fence_after();
 #pragma unroll
-        for (int e = 0; e < 16; e += 2) {
-            const int n = colq * 16 + e;
-            pk[e >> 1] = gelu2_bf16(add2(f2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])),
-                                         f2(__ldg(bias + n), __ldg(bias + n + 1))));
+                for (int k = 0; k < kTaps; ++k)
+                    tap(tmem + 256u + 64u * ((uint32_t)j & 1u), k, sL4 + (uint32_t)(k & 1) * kPlaneBytes, sW4);
+                mma_commit_to(done4 + 8u * ((uint32_t)j & 1u));
+                sent = j + 1;
+                if (j + 2 < mine) layer3(j + 2);
+            }
+            if (!ok) *abort_flag = 1;
+            // the MMAs issued finish before TMEM is freed
+            if (b) mbar_wait(free0 + 8u * ((b - 1u) % kL34Planes), ((b - 1u) / kL34Planes) & 1u);
+            if (sent) mbar_wait(done4 + 8u * ((uint32_t)(sent - 1) & 1u), (uint32_t)((sent - 1) >> 1) & 1u);
         }
-    };
-    // the two 16-byte chunks of a row written in an order that alternates
-    // with the lane, so that a store instruction's lanes spread over more banks
-    auto put_row = [&](uint32_t pbase, uint32_t row, const uint32_t (&pk)[8]) {
+    } else {
+        // ---------------- epilogues: warp w reads TMEM lane quarter w mod 4 (its
+        // hardware quarter) and columns 16 (w / 4) .. + 15: a thread holds 16
+        // values of one tile row
+        const int quarter = warp & 3, colq = warp >> 2;
+        const int r = quarter * 32 + lane;       // this thread's TMEM lane
+        const int mt = 16 * (r & 7) + (r >> 3);  // ... and the tile row it holds
+        const uint32_t tlane = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)colq * 16u;
+        const bool storer = colq == 0 && lane == 0;
+        // 16 columns of accumulator acc, bias, GELU, as BF16 pairs
+        auto finish = [&](uint32_t acc, const float *bias, uint32_t (&pk)[8]) {
+            uint32_t v[16];
+            tmem_ld16(tlane + acc, v);
+            float4 f[4];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int cc = k ^ (lane & 1);
-            const uint32_t dst =
-                pbase + row * 128u + ((uint32_t)((colq * 2 + cc) ^ (int)(row & 7)) << 4);
-            const uint32_t w0 = cc ? pk[4] : pk[0], w1 = cc ? pk[5] : pk[1];
-            const uint32_t w2 = cc ? pk[6] : pk[2], w3 = cc ? pk[7] : pk[3];
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w0), "r"(w1),
-                         "r"(w2), "r"(w3)
-                         : "memory");
-        }
-    };
-
-    // Software pipeline over iterations n (tiles 2n, 2n + 1 of layer 3; one
-    // tile of layer 4): both layer-3 tiles' MMAs go out together, layer 4's
-    // epilogue of iteration n - 1 runs while they execute, then the layer-3
-    // epilogues fill the slab and layer 4's MMAs of iteration n go out, to
-    // complete while the next iteration's loads are awaited.  Tile s sits in
-    // buffer s mod 3, and tile s + 3 is loaded into it as soon as the
-    // epilogue of tile s has seen s's MMAs complete.
-    // layer 4's epilogue of the iteration at it (phase ph)
-    // (a wait that gives up marks `bad`; the block learns of it at its next
-    // barrier, so the waits themselves need none)
-    bool bad = false;
-    auto epilogue4 = [&](int it, uint32_t ph) {
-        if (!mbar_wait(sBar + 16u, ph)) bad = true;
-        tc_fence_after();
-        uint32_t pk[8];
-        finish(128u, bias4, pk);
-        const int m = it * kTileRows + mt;
-        if (m < M4) {
-            uint4 *o4 = reinterpret_cast<uint4 *>(out + (size_t)m * kCh + colq * 16);
-            o4[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-            o4[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-        }
-        tc_fence_before();
-    };
-    int n = 0;
-    bool ok = true;
-    for (int it = blockIdx.x; it < n4; it += gridDim.x, ++n) {
-        const uint32_t ph = (uint32_t)n & 1u;
-        const int itn = it + (int)gridDim.x;
-        // tiles 2n and 2n + 1 loaded (tile 2n + 2 may still be in flight)
-        cp_async_wait1();
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc_fence_before();
-        if (__syncthreads_or(bad)) {
-            ok = false;
-            break;
-        }
-        tc_fence_after();
-        if (tid == 0) {
-            mma_tile(tmem, sSlab + (uint32_t)((2 * n) % kSlabs) * kSlabBytes, sW3, sBar);
-            mma_tile(tmem + 64u, sSlab + (uint32_t)((2 * n + 1) % kSlabs) * kSlabBytes, sW3,
-                     sBar + 8u);
-        }
-        if (n > 0) epilogue4(it - (int)gridDim.x, ph ^ 1u);
-        // layer-3 epilogues into the layer-4 slab (layer 4's last MMAs
-        // completed: its epilogue just waited for them)
-        for (int X = 0; X < 2; ++X) {
-            if (!mbar_wait(sBar + 8u * (uint32_t)X, ph)) bad = true;
+            for (int e = 0; e < 4; ++e)
+                f[e] = __ldg(reinterpret_cast<const float4 *>(bias + colq * 16) + e);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                pk[2 * e] = gelu2_bf16(add2(f2(__uint_as_float(v[4 * e]), __uint_as_float(v[4 * e + 1])),
+                                            f2(f[e].x, f[e].y)));
+                pk[2 * e + 1] = gelu2_bf16(
+                    add2(f2(__uint_as_float(v[4 * e + 2]), __uint_as_float(v[4 * e + 3])), f2(f[e].z, f[e].w)));
+            }
+        };
+        // the two 16-byte chunks of a row written in an order that alternates
+        // with the lane, so that a store instruction's lanes spread over more banks
+        auto put_row = [&](uint32_t pbase, uint32_t row, const uint32_t (&pk)[8]) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int cc = k ^ (lane & 1);
+                const uint32_t dst =
+                    pbase + row * 128u + ((uint32_t)((colq * 2 + cc) ^ (int)(row & 7)) << 4);
+                const uint32_t w0 = cc ? pk[4] : pk[0], w1 = cc ? pk[5] : pk[1];
+                const uint32_t w2 = cc ? pk[6] : pk[2], w3 = cc ? pk[7] : pk[3];
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w0), "r"(w1),
+                             "r"(w2), "r"(w3)
+                             : "memory");
+            }
+        };
+        bool bad = false;  // a wait gave up (the quarter learns of it at its next barrier)
+        // layer 4's outputs of this CTA's iteration j, traces 4 it ..; false: leave
+        auto outputs = [&](int j, int it) {
             tc_fence_after();
-            // this tile's buffer is free: tile 2n + X + 3 of the sequence goes
-            // there (iteration n + 1's tile B, or iteration n + 2's tile A)
-            load_slab((2 * n + X) % kSlabs, X == 0 ? 2 * itn + 1 : 2 * (itn + (int)gridDim.x));
             uint32_t pk[8];
-            finish(64u * (uint32_t)X, bias3, pk);
-            const int b = 2 * X + (mt >> 6), q = mt & 63;
-            const uint32_t pbase = sL4 + (uint32_t)(q & 1) * kPlaneBytes;
-            if (q <= 33) put_row(pbase, 8u * (uint32_t)((q >> 1) + 1) + 2u * (uint32_t)b, pk);
-            if (q >= 30) put_row(pbase, 8u * (uint32_t)((q >> 1) - 15) + 2u * (uint32_t)b + 1u, pk);
+            finish(256u + 64u * ((uint32_t)j & 1u), bias4, pk);
+            // the quarter's rows of the last tile have left
+            if (storer) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            if (quarter_any(1 + quarter, bad || *abort_flag != 0)) return false;
+            // a quarter's row is its lane: the store's box has position / 16
+            // before position mod 16, as the accumulator's lanes do
+            put_row(sOut + (uint32_t)quarter * 4096u, (uint32_t)lane, pk);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("bar.sync %0, 128;" ::"r"(1 + quarter) : "memory");
+            if (storer) {
+                // (traces past the batch are out of the tensor)
+                asm volatile(
+                    "cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
+                        reinterpret_cast<uint64_t>(&omap)),
+                    "r"(0), "r"(8 * it), "r"(4 * quarter), "r"(sOut + (uint32_t)quarter * 4096u)
+                    : "memory");
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            }
+            return true;
+        };
+        int j = 0;
+        bool go = true;
+        for (int it = blockIdx.x; it < iters; it += (int)gridDim.x, ++j) {
+            // layer 3's outputs, worked out before the slab is free
+            uint32_t pk[2][8];
+#pragma unroll
+            for (uint32_t X = 0; X < 2; ++X) {
+                const uint32_t buf = 2u * ((uint32_t)j & 1u) + X;
+                if (!mbar_wait(done3 + 8u * buf, (uint32_t)(j >> 1) & 1u)) bad = true;
+                __syncwarp();
+                tc_fence_after();
+                finish(64u * buf, bias3, pk[X]);
+            }
+            // the slab's last MMAs are done
+            if (j > 0 && !mbar_wait(done4 + 8u * ((uint32_t)(j - 1) & 1u), (uint32_t)((j - 1) >> 1) & 1u))
+                bad = true;
+#pragma unroll
+            for (int X = 0; X < 2; ++X) {
+                const int b = 2 * X + (mt >> 6), q = mt & 63;
+                const uint32_t pbase = sL4 + (uint32_t)(q & 1) * kPlaneBytes;
+                if (q <= 33) put_row(pbase, 8u * (uint32_t)((q >> 1) + 1) + 2u * (uint32_t)b, pk[X]);
+                if (q >= 30) put_row(pbase, 8u * (uint32_t)((q >> 1) - 15) + 2u * (uint32_t)b + 1u, pk[X]);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             tc_fence_before();
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(ready4) : "memory");
+            if (j > 0 && !outputs(j - 1, it - (int)gridDim.x)) {
+                go = false;
+                break;
+            }
         }
-        // layer 4 from the slab just written
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (go && j > 0) {
+            if (!mbar_wait(done4 + 8u * ((uint32_t)(j - 1) & 1u), (uint32_t)((j - 1) >> 1) & 1u)) bad = true;
+            __syncwarp();
+            go = outputs(j - 1, (int)blockIdx.x + (j - 1) * (int)gridDim.x);
+        }
+        if (!go) *abort_flag = 1;
+        if (storer) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         tc_fence_before();
-        if (__syncthreads_or(bad)) {
-            ok = false;
-            break;
-        }
-        tc_fence_after();
-        if (tid == 0) mma_tile(tmem + 128u, sL4, sW4, sBar + 16u);
     }
-    if (ok && n > 0) epilogue4(blockIdx.x + (n - 1) * (int)gridDim.x, (uint32_t)(n - 1) & 1u);
-    if (__syncthreads_or(bad) && tid == 0) atomicOr(status, PCHASE_DEV_TIMEOUT);
-    cp_async_wait_all();
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (tid == 0 && *abort_flag) atomicOr(status, PCHASE_DEV_TIMEOUT);
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(kL34TmemCols)
                      : "memory");
+}
+
+// Layer 3's inputs [nb][128][64] BF16 as a 5-D tensor (channel, block of 32
+// positions, trace, pair in the block, parity).  A plane's groups 1-16 are a
+// box of 4 blocks x 2 traces x 16 pairs; its groups 0 and 17 are the last
+// (first) pair of the blocks before (after), a box of one pair that starts one
+// block early (late): zeros where that leaves the trace.
+static bool conv3_in_map(const __nv_bfloat16 *x, int nb, uint32_t pairs, CUtensorMap *map) {
+    const PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
+    if (!encode) return false;
+    const cuuint64_t dims[5] = {64, 4, (cuuint64_t)nb, 16, 2};
+    const cuuint64_t strides[4] = {32 * 128, 128 * 128, 2 * 128, 128};
+    const cuuint32_t box[5] = {64, 4, 2, pairs, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<__nv_bfloat16 *>(x), dims, strides,
+                  box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Layer 4's outputs [nb][32][64] BF16 as (channel, row / 16, row mod 16) of
+// the nb 32 rows: a lane quarter's rows are a box of 8 x 4
+static bool conv4_out_map(__nv_bfloat16 *out, int nb, CUtensorMap *map) {
+    const PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
+    if (!encode) return false;
+    const cuuint64_t dims[3] = {64, (cuuint64_t)nb * 2, 16};
+    const cuuint64_t strides[2] = {16 * 128, 128};
+    const cuuint32_t box[3] = {64, 8, 4};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, out, dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace
@@ -810,9 +911,11 @@ cudaError_t conv34_tc(const __nv_bfloat16 *x, int nb, const __nv_bfloat16 *W3, c
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kL34Smem);
     if (e != cudaSuccess) return e;
-    const long long iters = ((long long)nb * 32 + kTileRows - 1) / kTileRows;
-    const int grid = (int)std::min<long long>(iters, std::max(1, sms));
-    conv34_tc_kernel<<<grid, kL34Threads, kL34Smem, st>>>(x, nb, W3, bias3, W4, bias4, out, status);
+    const int grid = std::min((nb - 1) / 4 + 1, std::max(1, sms));
+    CUtensorMap xmap, emap, omap;
+    if (!conv3_in_map(x, nb, 16, &xmap) || !conv3_in_map(x, nb, 1, &emap) || !conv4_out_map(out, nb, &omap))
+        return cudaErrorInvalidValue;
+    conv34_tc_kernel<<<grid, kL34Threads, kL34Smem, st>>>(xmap, emap, nb, W3, bias3, W4, bias4, omap, status);
     return cudaGetLastError();
 }
 

@@ -34,9 +34,6 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool v
 __device__ __forceinline__ void cp_async_commit() {
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
-__device__ __forceinline__ void cp_async_wait1() {
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
@@ -90,6 +87,14 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
         : "memory");
 }
+__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map, int c0, int c1,
+                                            int c2, int c3, int c4, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
+        : "memory");
+}
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                  : "memory");
@@ -105,17 +110,20 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
-// OR of v over the 256 threads that meet at named barrier bar_id
-__device__ __forceinline__ bool group_any(int bar_id, bool v) {
+// OR of v over the N threads that meet at named barrier bar_id
+template <int N>
+__device__ __forceinline__ bool threads_any(int bar_id, bool v) {
     uint32_t r;
     asm volatile(
         "{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n"
-        " bar.red.or.pred p, %2, 256, q;\n selp.u32 %0, 1, 0, p;\n}"
+        " bar.red.or.pred p, %2, %3, q;\n selp.u32 %0, 1, 0, p;\n}"
         : "=r"(r)
-        : "r"((uint32_t)v), "r"(bar_id)
+        : "r"((uint32_t)v), "r"(bar_id), "n"(N)
         : "memory");
     return r != 0;
 }
+__device__ __forceinline__ bool group_any(int bar_id, bool v) { return threads_any<256>(bar_id, v); }
+__device__ __forceinline__ bool quarter_any(int bar_id, bool v) { return threads_any<128>(bar_id, v); }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
     asm volatile(
