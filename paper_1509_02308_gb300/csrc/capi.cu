@@ -158,6 +158,18 @@ constexpr uint32_t kUniformCaps[kUniformClasses] = {8192, 24576, 73728, 196608};
 // kUniformTaskNs of work.
 constexpr double kUniformMissNs = 30.0, kUniformHashMissNs = 50.0, kUniformWindowNs = 230.0;
 constexpr double kUniformTaskNs = 30.0e3;
+// Small sets of this many misses (1 ms and more miss by miss) are played in
+// segments, where their lines are enough more than their ways for a play to
+// forget its start (uniform.cu): two survey-length plays of 0.2 ms instead.
+constexpr double kUniformSegMisses = 8.0 * kUniformRun;
+inline bool uniform_forgets(uint32_t n, uint32_t ways) {
+    return (n >= ways + 2 || ways == 2) && 3ull * n >= 4ull * ways;
+}
+// Evictions to forget a guess by, ten times the mean (measured; the fewer lines
+// are out, the more it takes: 8 ways of 12 lines 102, of 11 200, of 10 1028).
+inline uint32_t uniform_warm(uint32_t n, uint32_t ways) {
+    return std::max(256u, (10ull * n >= 14ull * ways ? 128u : 256u) * ways);
+}
 
 // The tuning knobs as the planner reads them, and whether the plan's split
 // parts read head streams (plans of explicit pairs that are not a lower level
@@ -583,19 +595,24 @@ struct pchase_sim_plan {
     uint64_t n_uniform = 0, n_explicit = 0;
     std::vector<UniformTask> utasks;
     uint32_t uclass[kUniformClasses] = {};
+    // ... and of the long small sets, four segments each; segments in all
+    std::vector<UniformSeg> usegs;
+    uint32_t n_segstates = 0;
     std::vector<uint32_t> trace_unit;
     // a matcher's plan: groups of items with the same words, their candidates,
     // and the units of the other items
     std::vector<UniformGroup> ugroups;
     std::vector<uint32_t> ucands, urest;
-    size_t off_bad = 0, off_utasks = 0, off_tunit = 0, off_ugroups = 0, off_ucands = 0, off_urest = 0;
+    size_t off_bad = 0, off_utasks = 0, off_tunit = 0, off_ugroups = 0, off_ucands = 0, off_urest = 0,
+           off_usegs = 0, off_segstates = 0;
     double gwork_live[kUnitGroups] = {};  // (ulayout's)
     double gwork_main[kUnitGroups] = {};  // estimated work of each unit group in the
                                           // slot-mix launch
     bool affinity = false;
-    cudaStream_t side = nullptr, side2 = nullptr, uside = nullptr, uside2 = nullptr;
+    cudaStream_t side = nullptr, side2 = nullptr, uside = nullptr, uside2 = nullptr,
+                 uside3 = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr, fork2 = nullptr, join2 = nullptr;
-    cudaEvent_t ufork = nullptr, ujoin = nullptr, ujoin2 = nullptr;
+    cudaEvent_t ufork = nullptr, ujoin = nullptr, ujoin2 = nullptr, ujoin3 = nullptr;
     // one run at a time records and waits for the events above: threads may
     // run a plan on streams and workspaces of their own
     std::mutex launching;
@@ -605,9 +622,11 @@ struct pchase_sim_plan {
         if (side2) cudaStreamDestroy(side2);
         if (uside) cudaStreamDestroy(uside);
         if (uside2) cudaStreamDestroy(uside2);
+        if (uside3) cudaStreamDestroy(uside3);
         if (ufork) cudaEventDestroy(ufork);
         if (ujoin) cudaEventDestroy(ujoin);
         if (ujoin2) cudaEventDestroy(ujoin2);
+        if (ujoin3) cudaEventDestroy(ujoin3);
         if (fork) cudaEventDestroy(fork);
         if (join) cudaEventDestroy(join);
         if (fork2) cudaEventDestroy(fork2);
@@ -739,7 +758,7 @@ void plan_uniform(pchase_sim_plan *p) {
         // leaves missing is near 1 - (a / n)^2
         const double passes = (double)(it.len - c.per) / c.per + 1.0;
         const double n = c.n_max, r = it.ways / n, misses = passes * n * (1.0 - r * r);
-        uint32_t lanes = 0;
+        uint32_t lanes = 0, played = 0;  // (classes played in segments)
         double set_ns = passes * std::max(1.0, n / 32.0) * kUniformWindowNs;
         if (c.n_max <= 32) {
             lanes = 32;
@@ -750,12 +769,28 @@ void plan_uniform(pchase_sim_plan *p) {
             if (c.over <= 8 && ns > 1.5 * set_ns) lanes = 0;
             else set_ns = ns;
         }
+        if (c.n_max <= 32 && misses >= kUniformSegMisses && uniform_forgets(c.n_max, it.ways)) {
+            // (the estimate is 5 to 20 % low, most for few ways; what is left over is
+            // played on by the last segment)
+            const uint32_t segments = (uint32_t)((1.1 + 0.25 / it.ways) * misses / kUniformRun) + 1u;
+            uint32_t cls = 0;
+            for (; cls < c.over; ++cls) {
+                const uint32_t lines = (c.nl - cls - 1u) / c.Tp + 1u;
+                if (!uniform_forgets(lines, it.ways)) break;
+                for (uint32_t f = 0; f < segments; f += 4)
+                    p->usegs.push_back(
+                        {(uint32_t)k, cls, p->n_segstates, segments, f, uniform_warm(lines, it.ways)});
+                p->n_segstates += segments;
+            }
+            if (cls == c.over) continue;
+            played = cls;
+        }
         const uint32_t step = lanes ? 32u / lanes : 1u;
         const uint32_t steps = (uint32_t)std::max(1.0, std::min(1e6, kUniformTaskNs / set_ns));
         const uint32_t bytes = lanes ? kUniformSmallBytes : (uint32_t)uniform_window_bytes(c.n_max, it.ways);
         int cls = 0;
         while (kUniformCaps[cls] < bytes) ++cls;
-        for (uint64_t first = 0; first < c.over; first += (uint64_t)step * steps) {
+        for (uint64_t first = played; first < c.over; first += (uint64_t)step * steps) {
             const uint32_t count = (uint32_t)std::min<uint64_t>((uint64_t)step * steps, c.over - first);
             all.push_back({{(uint32_t)k, (uint32_t)first, count, lanes}, cls,
                            set_ns * ((count + step - 1) / step)});
@@ -883,7 +918,8 @@ int plan_runtime(pchase_sim_plan *p) {
     // other launches
     const bool large = p->utasks.size() > p->uclass[0];
     const bool beside = !p->uniform_every || !p->ugroups.empty();
-    if (!p->utasks.empty() && (large || beside))
+    const bool segments = !p->usegs.empty();
+    if ((!p->utasks.empty() && (large || beside)) || segments)
         PCHASE_CUDA(cudaEventCreateWithFlags(&p->ufork, cudaEventDisableTiming), "cudaEventCreate");
     if (p->uclass[0] && beside) {
         PCHASE_CUDA(cudaStreamCreateWithFlags(&p->uside, cudaStreamNonBlocking), "cudaStreamCreate");
@@ -892,6 +928,10 @@ int plan_runtime(pchase_sim_plan *p) {
     if (large) {
         PCHASE_CUDA(cudaStreamCreateWithFlags(&p->uside2, cudaStreamNonBlocking), "cudaStreamCreate");
         PCHASE_CUDA(cudaEventCreateWithFlags(&p->ujoin2, cudaEventDisableTiming), "cudaEventCreate");
+    }
+    if (segments) {
+        PCHASE_CUDA(cudaStreamCreateWithFlags(&p->uside3, cudaStreamNonBlocking), "cudaStreamCreate");
+        PCHASE_CUDA(cudaEventCreateWithFlags(&p->ujoin3, cudaEventDisableTiming), "cudaEventCreate");
     }
     p->device = dev;
     return PCHASE_OK;
@@ -939,6 +979,15 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
                     "uniform words");
         const UniformTask *const tasks = reinterpret_cast<const UniformTask *>(w + p->off_utasks);
         if (p->ufork && !o.dist) PCHASE_CUDA(cudaEventRecord(p->ufork, st), "cudaEventRecord");
+        if (p->uside3) {
+            PCHASE_CUDA(cudaStreamWaitEvent(p->uside3, p->ufork, 0), "cudaStreamWaitEvent");
+            PCHASE_CUDA(launch_uniform_segments(items, reinterpret_cast<const UniformSeg *>(w + p->off_usegs),
+                                                (uint32_t)p->usegs.size(),
+                                                reinterpret_cast<UniformSegState *>(w + p->off_segstates), o,
+                                                p->uside3),
+                        "uniform segments");
+            PCHASE_CUDA(cudaEventRecord(p->ujoin3, p->uside3), "cudaEventRecord");
+        }
         if (p->uside2) {
             PCHASE_CUDA(cudaStreamWaitEvent(p->uside2, p->ufork, 0), "cudaStreamWaitEvent");
             uint32_t first = (uint32_t)p->utasks.size();
@@ -1006,6 +1055,7 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
         PCHASE_CUDA(cudaStreamWaitEvent(st, p->join2, 0), "cudaStreamWaitEvent");
     if (uni && p->uside) PCHASE_CUDA(cudaStreamWaitEvent(st, p->ujoin, 0), "cudaStreamWaitEvent");
     if (uni && p->uside2) PCHASE_CUDA(cudaStreamWaitEvent(st, p->ujoin2, 0), "cudaStreamWaitEvent");
+    if (uni && p->uside3) PCHASE_CUDA(cudaStreamWaitEvent(st, p->ujoin3, 0), "cudaStreamWaitEvent");
     return PCHASE_OK;
 }
 
@@ -1808,6 +1858,10 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
     off = align256(off + p->ucands.size() * sizeof(uint32_t));
     p->off_urest = off;
     off = align256(off + p->urest.size() * sizeof(uint32_t));
+    p->off_usegs = off;
+    off = align256(off + p->usegs.size() * sizeof(UniformSeg));
+    p->off_segstates = off;
+    off = align256(off + (size_t)p->n_segstates * sizeof(UniformSegState));
     p->ws_bytes = off;
     *plan_out = p;
     return PCHASE_OK;
@@ -1823,6 +1877,7 @@ size_t pchase_sim_plan_upload_bytes(const pchase_sim_plan *plan) {
            plan->utasks.size() * sizeof(UniformTask) + plan->trace_unit.size() * sizeof(uint32_t) +
            plan->ugroups.size() * sizeof(UniformGroup) +
            (plan->ucands.size() + plan->urest.size()) * sizeof(uint32_t) +
+           plan->usegs.size() * sizeof(UniformSeg) +
            (plan->jobs.empty() ? 0
                                : plan->jobs.size() * sizeof(StreamJob) +
                                      plan->seg_job.size() * sizeof(uint32_t) +
@@ -1847,6 +1902,7 @@ uint32_t pchase_sim_plan_launches(const pchase_sim_plan *plan) {
     if (plan->uniform) {
         n += 1u;
         for (uint32_t c : plan->uclass) n += c ? 1u : 0u;
+        n += plan->usegs.empty() ? 0u : 2u;
         if (plan->uniform_all) return n;
     }
     return n + (plan->jobs.empty() ? 0u : 1u) +
@@ -1950,8 +2006,8 @@ size_t pchase_sim_plan_describe(const pchase_sim_plan *plan, char *buf, size_t b
         d += tmp;
         if (plan->uniform) {
             // items that may be done as uniform chains, tasks of played sets
-            snprintf(tmp, sizeof tmp, " uniform=%llu,%zu", (unsigned long long)plan->n_uniform,
-                     plan->utasks.size());
+            snprintf(tmp, sizeof tmp, " uniform=%llu,%zu,%zu", (unsigned long long)plan->n_uniform,
+                     plan->utasks.size(), plan->usegs.size());
             d += tmp;
             d += " live_slots=";
             for (uint32_t w = 0; w < plan->ulayout.nwarps; ++w) {
@@ -2031,6 +2087,10 @@ int pchase_sim_plan_upload(const pchase_sim_plan *plan, void *workspace, size_t 
                                     plan->ucands.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, st),
                     "upload uniform candidates");
     }
+    if (!plan->usegs.empty())
+        PCHASE_CUDA(cudaMemcpyAsync(w + plan->off_usegs, plan->usegs.data(),
+                                    plan->usegs.size() * sizeof(UniformSeg), cudaMemcpyHostToDevice, st),
+                    "upload uniform segments");
     if (!plan->urest.empty())
         PCHASE_CUDA(cudaMemcpyAsync(w + plan->off_urest, plan->urest.data(),
                                     plan->urest.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, st),

@@ -248,6 +248,20 @@ struct UniformTask {
     uint32_t count;
     uint32_t lanes;
 };
+// Four segments of a long small set (uniform.cu): `first` .. of `count`, each
+// kUniformRun evictions long, surveyed from `warm` evictions earlier; their
+// states start at `state`.
+constexpr uint32_t kUniformRun = 4096;
+struct UniformSeg {
+    uint32_t unit, cls;
+    uint32_t state, count, first;
+    uint32_t warm;
+};
+struct __align__(16) UniformSegState {
+    uint8_t start[32], end[32];  // per way, its line from the last miss's on
+    uint32_t lines;              // run heads gone by from start to end
+    uint32_t pad[3];
+};
 // Matcher items whose words are the same: one trace, one line size, and every
 // run head of the later passes missing or none.
 struct UniformGroup {
@@ -317,6 +331,9 @@ cudaError_t launch_uniform_match(const SimItem *items, const UniformGroup *group
                                  cudaStream_t st);
 cudaError_t launch_uniform_play(const SimItem *items, const UniformTask *tasks, uint32_t n_tasks,
                                 uint32_t smem_bytes, const SimOut &out, cudaStream_t st);
+// The survey of the long small sets' segments, then their play.
+cudaError_t launch_uniform_segments(const SimItem *items, const UniformSeg *segs, uint32_t n_segs,
+                                    UniformSegState *states, const SimOut &out, cudaStream_t st);
 // The head streams of a plan's split items (three launches on `st`).
 cudaError_t launch_streams(const SimItem *items, const StreamJob *jobs, uint32_t n_jobs,
                            const uint32_t *seg_job, uint32_t n_seg, uint32_t *cnt,

@@ -422,6 +422,26 @@ struct Sink {
     }
 };
 
+// A warp's sink; the matcher's observed words take the arena's first part.
+__device__ __forceinline__ uint8_t *open_sink(Sink &sink, const SimItem &it, const Chain &ch, const SimOut &out,
+                                              uint32_t rep, uint8_t *arena, uint32_t lane) {
+    sink.bm = nullptr;
+    sink.obs = nullptr;
+    sink.warmup = ch.warmup;
+    if (out.dist) {
+        uint32_t *const ob = reinterpret_cast<uint32_t *>(arena);
+        const uint32_t nwords = (ch.len + 31u) >> 5;  // at most kUniformMatchLen / 32
+        const uint32_t *const src = out.observed + rep * out.rep_obs_stride + out.obs_word_offsets[it.obs];
+        for (uint32_t w = lane; w < nwords; w += 32) ob[w] = src[w];
+        __syncwarp();
+        sink.obs = ob;
+        arena += kUniformMatchLen / 8;
+    } else if (out.bitmaps) {
+        sink.bm = out.bitmaps + (out.word_offsets ? out.word_offsets[it.out_item] : it.word_off);
+    }
+    return arena;
+}
+
 // Small sets (n <= 32 lines): one set per group of G lanes, miss by miss.
 // The set's state is a mask of the lines not held, line j at bit 31 - j; all
 // accesses up to the next line not held are hits, so the next miss is the
@@ -435,6 +455,86 @@ struct Sink {
 // bits, counts and distances are worked out for G misses at once.
 //
 // arena: uint8 occ[32 ways][32 lanes], uint32 toff[32 lines][32 lanes]
+// Where a small set is: lines not held (gone), those of them ahead in this pass
+// (below), the last miss's line p and its pass's first access.
+struct SmallSet {
+    uint32_t gone, below, base, p;
+};
+
+// G misses in a row.  wv: 32 times the way of this lane's (miss r of the
+// group's); mine_p, mine_base: that miss.
+template <int G>
+__device__ __forceinline__ void small_round(SmallSet &st, uint8_t *occ, uint32_t wv, uint32_t per,
+                                            uint32_t glane, uint32_t r, uint32_t &mine_p,
+                                            uint32_t &mine_base) {
+    uint32_t p = 0;
+    uint32_t w = G == 1 ? wv : __shfl_sync(kFull, wv, glane);
+    uint32_t ld = occ[w];  // line of way w, but for the miss ahead
+    bool again = false;    // the miss ahead took way w too
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+        // (the miss ahead took the same way: it is the line that leaves)
+        const uint32_t old = again ? p : ld;
+        const bool wrap = st.below == 0;
+        const uint32_t x = wrap ? st.gone : st.below;
+        st.base += wrap ? per : 0u;
+        p = 31u - (uint32_t)__clz(x);
+        uint32_t wn = 0;
+        if (q + 1 < G) {
+            wn = __shfl_sync(kFull, wv, glane + q + 1);
+            ld = occ[wn];
+            again = wn == w;
+        }
+        occ[w] = (uint8_t)p;
+        const uint32_t ob = 1u << old;
+        st.below = (st.gone | ob) & ~(kFull << p);
+        st.gone = (st.gone | ob) & ~(1u << p);
+        mine_p = r == (uint32_t)q ? p : mine_p;
+        mine_base = r == (uint32_t)q ? st.base : mine_base;
+        w = wn;
+    }
+    st.p = p;
+}
+
+// A miss at access t of each lane where `count`, a group's in order.
+template <int G>
+__device__ __forceinline__ void small_sink(Sink &sink, bool count, uint32_t t, uint32_t r) {
+    if (sink.obs) {
+        if (count) sink.dsum += (sink.obs[t >> 5] >> (t & 31u)) & 1u ? -1 : 1;
+        return;
+    }
+    sink.tot += count;
+    sink.aft += count && t >= sink.warmup;
+    if (sink.bm) {
+        // a group's misses come in order: the first of each word
+        // collects the others' bits
+        const uint32_t wd = count ? t >> 5 : 0xFFFFFFFFu;
+        uint32_t bits = 1u << (t & 31u);
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1) {
+            const uint32_t vb = __shfl_down_sync(kFull, bits, o);
+            const uint32_t vw = __shfl_down_sync(kFull, wd, o);
+            if (r + o < (uint32_t)G && vw == wd) bits |= vb;
+        }
+        const uint32_t wp = __shfl_up_sync(kFull, wd, 1);
+        if (count && (r == 0 || wp != wd)) atomicOr(sink.bm + wd, bits);
+    }
+}
+
+// The set after its first pass: lines 0 .. a - 1 have filled the ways, the
+// others have evicted n - a of them.
+__device__ __forceinline__ SmallSet small_first_pass(uint8_t *occ, uint32_t n, uint32_t a, uint64_t seed,
+                                                     uint32_t set, bool wtd) {
+    uint32_t gone = 0;
+    for (uint32_t w = 0; w < a; ++w) occ[32 * w] = (uint8_t)(31u - w);
+    for (uint32_t j = a; j < n; ++j) {
+        const uint32_t w = random_way(seed, set, j - a, a, wtd);
+        gone |= 1u << occ[32 * w];
+        occ[32 * w] = (uint8_t)(31u - j);
+    }
+    return SmallSet{gone, 0u, 0u, 31u - (n - 1u)};
+}
+
 template <int G>
 __device__ __forceinline__ void play_small(const SimItem &it, const Chain &ch, uint32_t first,
                                            uint32_t nsets, uint8_t *arena, Sink &sink, uint32_t lane) {
@@ -448,78 +548,177 @@ __device__ __forceinline__ void play_small(const SimItem &it, const Chain &ch, u
     const bool wtd = it.policy == PCHASE_WEIGHTED;
     const uint64_t seed = it.seed;
     for (uint32_t j = 0; j < n; ++j) toff[32 * (31u - j)] = ch.first(c + j * ch.Tp);
-    // the first pass: lines 0 .. a - 1 fill the ways, the others evict
-    uint32_t gone = 0;  // lines not held
-    for (uint32_t w = 0; w < a; ++w) occ[32 * w] = (uint8_t)(31u - w);
-    uint32_t k = 0;  // evictions
-    for (uint32_t j = a; j < n; ++j, ++k) {
-        const uint32_t w = random_way(seed, set, k, a, wtd);
-        gone |= 1u << occ[32 * w];
-        occ[32 * w] = (uint8_t)(31u - j);
-    }
+    SmallSet st = small_first_pass(occ, n, a, seed, set, wtd);
+    uint32_t k = n - a;  // evictions
     const uint32_t glane = lane & ~(uint32_t)(G - 1);
     const uint32_t len = ch.len, per = ch.per;
-    uint32_t base = per;
-    uint32_t below = gone;  // lines not held that are still ahead in this pass
     bool done = !on;
     while (!__all_sync(kFull, done)) {
         constexpr int kRounds = G >= 8 ? 1 : 8 / G;  // 8 misses at least to a vote
         for (int round = 0; round < kRounds; ++round) {
             const uint32_t wv = 32u * random_way(seed, set, k + r, a, wtd);
             k += G;
-            uint32_t p = 0, mine_p = 0, mine_base = 0;
-            uint32_t w = G == 1 ? wv : __shfl_sync(kFull, wv, glane);
-            uint32_t ld = occ[w];       // line of way w, but for the miss ahead
-            bool again = false;         // the miss ahead took way w too
-#pragma unroll
-            for (int q = 0; q < G; ++q) {
-                // (the miss ahead took the same way: it is the line that leaves)
-                const uint32_t old = again ? p : ld;
-                const bool wrap = below == 0;
-                const uint32_t x = wrap ? gone : below;
-                base += wrap ? per : 0u;
-                p = 31u - (uint32_t)__clz(x);
-                uint32_t wn = 0;
-                if (q + 1 < G) {
-                    wn = __shfl_sync(kFull, wv, glane + q + 1);
-                    ld = occ[wn];
-                    again = wn == w;
-                }
-                occ[w] = (uint8_t)p;
-                const uint32_t ob = 1u << old;
-                below = (gone | ob) & ~(kFull << p);
-                gone = (gone | ob) & ~(1u << p);
-                mine_p = r == (uint32_t)q ? p : mine_p;
-                mine_base = r == (uint32_t)q ? base : mine_base;
-                w = wn;
-            }
+            uint32_t mine_p = 0, mine_base = 0;
+            small_round<G>(st, occ, wv, per, glane, r, mine_p, mine_base);
             const uint32_t t = mine_base + toff[32 * mine_p];
             const bool count = !done && t < len;
             const uint32_t latest = __shfl_sync(kFull, t, glane + G - 1);
             done = done || latest >= len;
-            if (sink.obs) {
-                if (count) sink.dsum += (sink.obs[t >> 5] >> (t & 31u)) & 1u ? -1 : 1;
-            } else {
-                sink.tot += count;
-                sink.aft += count && t >= sink.warmup;
-                if (sink.bm) {
-                    // a group's misses come in order: the first of each word
-                    // collects the others' bits
-                    const uint32_t wd = count ? t >> 5 : 0xFFFFFFFFu;
-                    uint32_t bits = 1u << (t & 31u);
-#pragma unroll
-                    for (int o = 1; o < G; o <<= 1) {
-                        const uint32_t vb = __shfl_down_sync(kFull, bits, o);
-                        const uint32_t vw = __shfl_down_sync(kFull, wd, o);
-                        if (r + o < (uint32_t)G && vw == wd) bits |= vb;
-                    }
-                    const uint32_t wp = __shfl_up_sync(kFull, wd, 1);
-                    if (count && (r == 0 || wp != wd)) atomicOr(sink.bm + wd, bits);
-                }
-            }
+            small_sink<G>(sink, count, t, r);
         }
     }
     __syncwarp();
+}
+
+// ---- one long small set by many groups of lanes
+// The chain of a set's misses is serial, and one of 300K misses (11.7 ms) set
+// the time of a batch.  But what a miss depends on, the lines held counted from
+// the last miss's line on, forgets where it came from: two plays of the same
+// victims from different states become the same play, up to a rotation of the
+// lines, within some tens to hundreds of misses where two lines or more are
+// always out (4 ways, 6 lines: 34 on average, 250 at most of 300; 16 ways of 23
+// lines: 374, 1837; 4 ways of 5 lines: never; 3 lines in 2 ways: at once).  So the evictions are cut into
+// segments.  A survey plays each from a guess kUniformRun evictions long,
+// after `warm` evictions to forget it, and notes the state at its start and
+// end and the lines it went by.  Then every segment is played from the state
+// noted at its start, rotated by the lines all segments before it went by: it
+// is the true one if each of those ended in the state the next one's start
+// noted.  Where one did not, the segment before plays on to the end alone.
+// Segment i is evictions n - a + warm + i kUniformRun and on, the first one
+// from n - a (the first pass's) on.
+constexpr int kSegG = 8;  // lanes of a segment: four segments a warp
+
+__device__ __forceinline__ bool same_state(const uint8_t *x, const uint8_t *y) {
+    const uint4 *const u = reinterpret_cast<const uint4 *>(x), *const v = reinterpret_cast<const uint4 *>(y);
+    const uint4 a = u[0], b = v[0], c = u[1], d = v[1];
+    return a.x == b.x && a.y == b.y && a.z == b.z && a.w == b.w && c.x == d.x && c.y == d.y && c.z == d.z &&
+           c.w == d.w;
+}
+
+__global__ void __launch_bounds__(32) uniform_survey_kernel(const SimItem *__restrict__ items,
+                                                            const UniformSeg *__restrict__ segs,
+                                                            UniformSegState *__restrict__ states,
+                                                            SimOut out) {
+    __shared__ uint8_t arena[1024];
+    const uint32_t lane = threadIdx.x, r = lane % kSegG, glane = lane & ~(uint32_t)(kSegG - 1);
+    const UniformSeg sg = segs[blockIdx.x];
+    const SimItem it = items[sg.unit];
+    if (!taken(it, out.uniform_bad) || (out.dist && !((it.lsh >> kUniformMatchBit) & 1u))) return;
+    const Chain ch(it);
+    const uint32_t i = sg.first + lane / kSegG;
+    const uint32_t n = ch.lines_of(sg.cls), a = ch.a;
+    const uint32_t set = (uint32_t)(((uint64_t)sg.cls * ch.st) % ch.T);
+    const bool wtd = it.policy == PCHASE_WEIGHTED;
+    uint8_t *const occ = arena + lane;
+    SmallSet st;
+    if (i == 0) {
+        st = small_first_pass(occ, n, a, it.seed, set, wtd);
+    } else {
+        // (3 lines in 2 ways: every eviction swaps two of way 0's, way 1's and the
+        // one out, so an odd number of them, 1 + i kUniformRun, leaves an odd
+        // order; two plays of the same parity are one play but for a rotation)
+        const uint32_t flip = n == 3u ? 1u : 0u;
+        for (uint32_t w = 0; w < a; ++w) occ[32 * w] = (uint8_t)(31u - (w ^ flip));
+        st = SmallSet{(kFull >> a) & ~(n < 32u ? kFull >> n : 0u), 0u, 0u, 31u - (a - 1u)};
+        st.below = st.gone & ~(kFull << st.p);
+    }
+    __syncwarp();
+    uint32_t k = n - a + i * kUniformRun;
+    // (pass numbers times n: the lines gone by are base + 31 - p)
+    uint32_t from = st.base + 31u - st.p;
+    UniformSegState *const o = states + sg.state + i;
+    auto note = [&](uint8_t *to) {
+        if (i < sg.count)
+            for (uint32_t w = r; w < 32u; w += kSegG) {
+                // line of way w from the last miss's on
+                const uint32_t d = w < a ? st.p + n - occ[32 * w] : 0u;
+                to[w] = (uint8_t)(d >= n ? d - n : d);
+            }
+    };
+    auto play = [&](uint32_t evictions) {
+        for (uint32_t e = 0; e < evictions; e += kSegG) {
+            const uint32_t wv = 32u * random_way(it.seed, set, k + r, a, wtd);
+            k += kSegG;
+            uint32_t mp = 0, mb = 0;
+            small_round<kSegG>(st, occ, wv, n, glane, r, mp, mb);
+        }
+    };
+    play(sg.warm);
+    note(o->start);
+    if (i) from = st.base + 31u - st.p;
+    play(kUniformRun);
+    note(o->end);
+    if (i < sg.count && r == 0) o->lines = st.base + 31u - st.p - from;
+}
+
+__global__ void __launch_bounds__(32) uniform_segment_kernel(const SimItem *__restrict__ items,
+                                                             const UniformSeg *__restrict__ segs,
+                                                             const UniformSegState *__restrict__ states,
+                                                             SimOut out) {
+    uint8_t *arena = u_smem;
+    const uint32_t lane = threadIdx.x, r = lane % kSegG, glane = lane & ~(uint32_t)(kSegG - 1);
+    const UniformSeg sg = segs[blockIdx.x];
+    const SimItem it = items[sg.unit];
+    if (!taken(it, out.uniform_bad) || (out.dist && !((it.lsh >> kUniformMatchBit) & 1u))) return;
+    Chain ch(it);
+    ch.prepare_first();
+    Sink sink;
+    arena = open_sink(sink, it, ch, out, blockIdx.y, arena, lane);
+    const uint32_t i = sg.first + lane / kSegG;
+    const uint32_t n = ch.lines_of(sg.cls), a = ch.a;
+    const uint32_t set = (uint32_t)(((uint64_t)sg.cls * ch.st) % ch.T);
+    const bool wtd = it.policy == PCHASE_WEIGHTED;
+    uint8_t *const occ = arena + lane;
+    uint32_t *const toff = reinterpret_cast<uint32_t *>(arena + 1024) + lane;
+    for (uint32_t j = 0; j < n; ++j) toff[32 * (31u - j)] = ch.first(sg.cls + j * ch.Tp);
+    // the segments before this one: the lines they went by, and whether each
+    // ended where the next one started
+    const UniformSegState *const s0 = states + sg.state;
+    uint32_t lines = 0;
+    bool known = i < sg.count;
+    for (uint32_t q = r; known && q < i; q += kSegG) {
+        lines += s0[q].lines;
+        known = same_state(s0[q].end, s0[q + 1].start);
+    }
+#pragma unroll
+    for (int o = kSegG / 2; o; o >>= 1) {
+        lines += __shfl_xor_sync(kFull, lines, o);
+        known = __shfl_xor_sync(kFull, known ? 1 : 0, o) && known;
+    }
+    SmallSet st = small_first_pass(occ, n, a, it.seed, set, wtd);
+    uint32_t k = n - a;
+    if (i) {
+        k += sg.warm + i * kUniformRun;
+        lines += n - 1u;  // (the first pass)
+        const uint32_t line = lines % n;
+        st.base = lines / n * ch.per;
+        st.p = 31u - line;
+        st.gone = n < 32u ? ~(kFull >> n) : kFull;
+        for (uint32_t w = 0; known && w < a; ++w) {
+            uint32_t j = line + s0[i].start[w];
+            j -= j >= n ? n : 0u;
+            occ[32 * w] = (uint8_t)(31u - j);
+            st.gone &= ~(0x80000000u >> j);
+        }
+        st.below = st.gone & ~(kFull << st.p);
+    }
+    const bool ends = known && i + 1u < sg.count && same_state(s0[i].end, s0[i + 1u].start);
+    const uint32_t last = ends ? n - a + sg.warm + (i + 1u) * kUniformRun : 0xFFFFFFFFu;
+    __syncwarp();
+    const uint32_t len = ch.len, per = ch.per;
+    bool done = !known || st.base >= len;
+    while (!__all_sync(kFull, done)) {
+        const uint32_t wv = 32u * random_way(it.seed, set, k + r, a, wtd);
+        k += kSegG;
+        uint32_t mine_p = 0, mine_base = 0;
+        small_round<kSegG>(st, occ, wv, per, glane, r, mine_p, mine_base);
+        const uint32_t t = mine_base + toff[32 * mine_p];
+        const bool count = !done && t < len;
+        const uint32_t latest = __shfl_sync(kFull, t, glane + kSegG - 1);
+        done = done || latest >= len || k >= last;
+        small_sink<kSegG>(sink, count, t, r);
+    }
+    sink.finish(it, out, blockIdx.y, lane);
 }
 
 // Larger sets: one warp per set, a window of up to 32 H run heads at a time, H
@@ -678,23 +877,8 @@ __global__ void __launch_bounds__(32) uniform_play_kernel(const SimItem *__restr
     if (ham && !((it.lsh >> kUniformMatchBit) & 1u)) return;
     Chain ch(it);
     ch.prepare_first();
-    uint8_t *arena = u_smem;
     Sink sink;
-    sink.bm = nullptr;
-    sink.obs = nullptr;
-    sink.warmup = ch.warmup;
-    if (ham) {
-        uint32_t *const ob = reinterpret_cast<uint32_t *>(arena);
-        const uint32_t nwords = (ch.len + 31u) >> 5;  // at most kUniformMatchLen / 32
-        const uint32_t *const src =
-            out.observed + blockIdx.y * out.rep_obs_stride + out.obs_word_offsets[it.obs];
-        for (uint32_t w = lane; w < nwords; w += 32) ob[w] = src[w];
-        __syncwarp();
-        sink.obs = ob;
-        arena += kUniformMatchLen / 8;
-    } else if (out.bitmaps) {
-        sink.bm = out.bitmaps + (out.word_offsets ? out.word_offsets[it.out_item] : it.word_off);
-    }
+    uint8_t *const arena = open_sink(sink, it, ch, out, blockIdx.y, u_smem, lane);
     if (task.lanes) {
         const uint32_t per_warp = 32u / task.lanes;
         for (uint32_t c = 0; c < task.count; c += per_warp) {
@@ -780,6 +964,17 @@ cudaError_t launch_uniform_play(const SimItem *items, const UniformTask *tasks, 
     const uint32_t bytes = smem_bytes + (ham ? kUniformMatchLen / 8 : 0u);
     uniform_play_kernel<<<dim3(n_tasks, ham && out.n_rep ? out.n_rep : 1u), 32, bytes, st>>>(items, tasks,
                                                                                              out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_uniform_segments(const SimItem *items, const UniformSeg *segs, uint32_t n_segs,
+                                    UniformSegState *states, const SimOut &out, cudaStream_t st) {
+    if (!n_segs) return cudaSuccess;
+    const bool ham = out.dist != nullptr;
+    const uint32_t bytes = kUniformSmallBytes + (ham ? kUniformMatchLen / 8 : 0u);
+    uniform_survey_kernel<<<n_segs, 32, 0, st>>>(items, segs, states, out);
+    uniform_segment_kernel<<<dim3(n_segs, ham && out.n_rep ? out.n_rep : 1u), 32, bytes, st>>>(items, segs,
+                                                                                               states, out);
     return cudaGetLastError();
 }
 

@@ -186,6 +186,43 @@ def test_matcher_groups_candidates(n_geom):
         assert np.array_equal(x, y)
 
 
+@pytest.mark.parametrize("explicit", [False, True])
+def test_long_small_sets_by_segments(explicit):
+    """Overflowing sets of at most 32 lines with enough misses to be cut into
+    segments: few and many ways, classes of which only the larger ones are cut,
+    a line and several accesses to a line, weighted victims, plays that forget
+    their start late or (28 lines in 20 ways) perhaps not in time, and traces
+    that end anywhere in a segment."""
+    forms = []
+    for a, nl, T, stride, ln, pol in ((4, 6, 1, 8, 100003, W.RANDOM), (2, 9, 2, 8, 180000, W.RANDOM),
+                                      (4, 11, 2, 8, 190001, W.RANDOM), (2, 4, 1, 8, 90000, W.RANDOM),
+                                      (16, 23, 1, 8, 120000, W.RANDOM), (20, 28, 1, 16, 130007, W.RANDOM),
+                                      (22, 32, 1, 8, 131000, W.RANDOM), (4, 6, 1, 1, 500000, W.RANDOM),
+                                      (4, 7, 1, 8, 99999, W.WEIGHTED), (8, 36, 3, 8, 260000, W.RANDOM),
+                                      (2, 3, 1, 8, 77777, W.RANDOM), (8, 11, 1, 8, 90000, W.RANDOM),
+                                      (12, 16, 1, 8, 110000, W.RANDOM)):
+        n = 8 * nl if stride <= 8 else stride * nl
+        forms.append((W.Geom(a * T * 32, 32, a, T, pol, 1000 + 7 * len(forms)),
+                      W.Run(n, stride, ln, n // stride)))
+    runs = [r for _, r in forms]
+    flat, offs = api.pchase_build_batch(runs)
+    traces = [(flat[int(offs[i]):int(offs[i + 1])] if explicit else None, r.length, r.warmup, r.n_elems,
+               r.stride) for i, r in enumerate(runs)]
+    pairs = [(i, i) for i in range(len(runs))]
+    geoms = [g for g, _ in forms]
+    plan = api.SimPlan(geoms, traces, pairs=pairs)
+    cut = int(plan.description.split("uniform=")[1].split()[0].split(",")[2])
+    assert cut >= 3 * len(forms)  # every item is, into eight segments and more
+    for _ in range(2):  # (the second run over the first one's states)
+        bits, counts = plan.run()
+    words, counts = bits.cpu().numpy().view(np.uint32), counts.cpu().numpy().reshape(-1, 2)
+    for i, (g, r) in enumerate(forms):
+        want = _want(g, r)
+        have = api.unpack_bits(words[int(plan.word_offsets[i]):], r.length)
+        assert np.array_equal(have, want), (i, g, r, int(np.argmax(have != want)))
+        assert counts[i].tolist() == [int(want.sum()), int(want[r.warmup:].sum())], (i, g, r)
+
+
 def test_uniform_run_captured_in_a_graph():
     runs = [W.Run(n // 4, 32, 4 * (n // 128), n // 128) for n in (8192, 16512, 20480)]
     flat, offs = api.pchase_build_batch(runs)
