@@ -78,9 +78,20 @@ cudaError_t tc_gemm(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int
                     cudaStream_t st);
 
 // out [Cpad][ldo] = transpose of in [R][C] (row stride ldi), zero beyond R
-// columns and C rows.
-cudaError_t transpose_bf16(const __nv_bfloat16 *in, int R, int C, int ldi, __nv_bfloat16 *out,
-                           int ldo, int Cpad, cudaStream_t st);
+// columns and C rows.  C, ldi and ldo are even and the bases 4-byte aligned.
+struct TransposeJob {
+    const __nv_bfloat16 *in;
+    __nv_bfloat16 *out;
+    int R, C, ldi, ldo, Cpad;
+    uint32_t tiles;
+};
+constexpr int kTransposeJobs = 5;
+struct TransposeJobs {
+    TransposeJob job[kTransposeJobs];
+};
+TransposeJob transpose_job(const __nv_bfloat16 *in, int R, int C, int ldi, __nv_bfloat16 *out, int ldo,
+                           int Cpad);
+cudaError_t transpose_bf16(const TransposeJob *jobs, int n, cudaStream_t st);
 
 // The exhaustive least-squares matcher (lsq.cu) of the first min(n, *n_dev)
 // traces y [n][512] (n_dev NULL: all) against rates [n_geoms][512]: best

@@ -367,7 +367,7 @@ struct pchase_inverse {
     InverseLayout L;
     uint32_t max_batch;
     size_t p_w, p_wb, p_g, p_m, p_v, p_bytes;
-    size_t status, pre[4], act[4], pre4, h4, logits, dlog, dlogb, tA, tB, w4t, w5t, dh, dzf, dzb, dbig,
+    size_t status, pre[4], act[4], pre4, h4, logits, dlog, dlogb, tA, tB, tD, w4t, w5t, dh, dzf, dzb, dbig,
         dsmall, work_bytes, infer_bytes;
 };
 
@@ -506,6 +506,7 @@ int pchase_inverse_create(uint32_t max_batch, pchase_inverse **out) {
         const size_t ldk = (B + 7) / 8 * 8;
         h->tA = o; o = a256(o + 2 * kHidden * ldk);
         h->tB = o; o = a256(o + 2 * kFlat * ldk);
+        h->tD = o; o = a256(o + 2 * kLogitsPad * ldk);
         h->w4t = o; o = a256(o + 2 * (size_t)kFlat * kHidden);
         h->w5t = o; o = a256(o + 2 * (size_t)kHidden * kLogitsPad);
     }
@@ -607,13 +608,21 @@ int pchase_inverse_train_step(const pchase_inverse *h, void *params, void *work,
     __nv_bfloat16 *h4 = at<__nv_bfloat16>(work, h->h4);
     __nv_bfloat16 *tA = at<__nv_bfloat16>(work, h->tA), *tB = at<__nv_bfloat16>(work, h->tB);
     __nv_bfloat16 *w4t = at<__nv_bfloat16>(work, h->w4t), *w5t = at<__nv_bfloat16>(work, h->w5t);
-    INV_CUDA(transpose_bf16(wb + L.w[4], kHidden, kFlat, kFlat, w4t, kHidden, kFlat, st));
-    INV_CUDA(transpose_bf16(wb + L.w[5], kLogits, kHidden, kHidden, w5t, kLogitsPad, kHidden, st));
+    __nv_bfloat16 *tD = at<__nv_bfloat16>(work, h->tD);
+    {
+        // what can be transposed by now, in one launch (five of them: 40 us of
+        // a step of 4096 traces)
+        const TransposeJob jobs[kTransposeJobs] = {
+            transpose_job(at<__nv_bfloat16>(work, h->act[3]), (int)B, kFlat, kFlat, tB, ldk, kFlat),
+            transpose_job(wb + L.w[4], kHidden, kFlat, kFlat, w4t, kHidden, kFlat),
+            transpose_job(wb + L.w[5], kLogits, kHidden, kHidden, w5t, kLogitsPad, kHidden),
+            transpose_job(h4, (int)B, kHidden, kHidden, tA, ldk, kHidden),
+            transpose_job(dlogb, (int)B, kLogitsPad, kLogitsPad, tD, ldk, kLogitsPad)};
+        INV_CUDA(transpose_bf16(jobs, kTransposeJobs, st));
+    }
     {
         // grad W5 [31][256] = dlogb^T h4, as (h4^T) (dlogb^T)^T stored transposed
-        INV_CUDA(transpose_bf16(h4, (int)B, kHidden, kHidden, tA, ldk, kHidden, st));
-        INV_CUDA(transpose_bf16(dlogb, (int)B, kLogitsPad, kLogitsPad, tB, ldk, kLogitsPad, st));
-        INV_CUDA(tc_gemm(tA, ldk, tB, ldk, kHidden, kLogits, ldk, 32, 32, nullptr, grad + L.w[5],
+        INV_CUDA(tc_gemm(tA, ldk, tD, ldk, kHidden, kLogits, ldk, 32, 32, nullptr, grad + L.w[5],
                          kHidden, true, true, nullptr, nullptr, status, st));
         colsum_atomic_kernel<<<dim3(1, (B + 31) / 32), 32, 0, st>>>(dlog, (int)B, kLogits, 32,
                                                                      grad + L.b[5]);
@@ -631,9 +640,8 @@ int pchase_inverse_train_step(const pchase_inverse *h, void *params, void *work,
         gelu_back_kernel<<<grid_for(m), 256, 0, st>>>(at<float>(work, h->dh),
                                                       at<float>(work, h->pre4), m, dzf, dzb);
         // grad W4 [256][2048] = dzb^T act3
-        INV_CUDA(transpose_bf16(dzb, (int)B, kHidden, kHidden, tA, ldk, kHidden, st));
-        INV_CUDA(transpose_bf16(at<__nv_bfloat16>(work, h->act[3]), (int)B, kFlat, kFlat, tB, ldk,
-                                kFlat, st));
+        const TransposeJob job = transpose_job(dzb, (int)B, kHidden, kHidden, tA, ldk, kHidden);
+        INV_CUDA(transpose_bf16(&job, 1, st));
         INV_CUDA(tc_gemm(tA, ldk, tB, ldk, kHidden, kFlat, ldk, 128, 4, nullptr, grad + L.w[4],
                          kFlat, true, false, nullptr, nullptr, status, st));
         colsum_atomic_kernel<<<dim3((kHidden + 127) / 128, (B + 31) / 32), 128, 0, st>>>(

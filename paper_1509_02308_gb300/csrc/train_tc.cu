@@ -737,7 +737,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
 // frees it once its MMAs are done.  Epilogues: kStore (C[m][n], or C[n][m] when transposed,
 // + bias[n] if given; FP32 atomics when K is sliced) and kGelu (v = sum +
 // bias[n]: pre[m][n] = v, Cb[m][n] = BF16(GELU(v)) with the exact tanh).
-constexpr int kGemmStages = 4;
+// Three stages leave room for two CTAs of 128 columns on an SM, so that one's
+// loads and MMAs run under the other's epilogue.
+constexpr int kGemmStages = 3;
 enum GemmEpi { kStore = 0, kGelu = 1 };
 
 struct TcGemm {
@@ -925,21 +927,30 @@ __global__ void __launch_bounds__(128)
 }
 
 // out[c][r] = in[r][c] for r < R, c < C (out row stride ldo); columns R ..
-// ldo - 1 of each out row and rows C .. Cpad - 1 are zero.  32 x 32 tiles
-// through shared memory.
-__global__ void transpose_bf16_kernel(const __nv_bfloat16 *__restrict__ in, int R, int C, int ldi,
-                                      __nv_bfloat16 *__restrict__ out, int ldo, int Cpad) {
-    __shared__ __nv_bfloat16 t[32][33];
-    const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8 threads
-    for (int i = ty; i < 32; i += 8) {
-        const int r = r0 + i, c = c0 + tx;
-        t[i][tx] = (r < R && c < C) ? in[(size_t)r * ldi + c] : __float2bfloat16(0.0f);
+// ldo - 1 of each out row and rows C .. Cpad - 1 are zero.  64 x 64 tiles
+// through shared memory, two elements a lane in and out (C, ldi and ldo are
+// even); a launch takes several matrices, a job each.
+__global__ void __launch_bounds__(256) transpose_bf16_kernel(const TransposeJobs jobs) {
+    __shared__ uint32_t t[64][33];  // row r, columns 2 x and 2 x + 1
+    int j = 0;
+    uint32_t tile = blockIdx.x;
+    while (tile >= jobs.job[j].tiles) tile -= jobs.job[j++].tiles;
+    const TransposeJob &J = jobs.job[j];
+    const uint32_t across = (uint32_t)(J.Cpad + 63) / 64u;
+    const int r0 = (int)(tile / across) * 64, c0 = (int)(tile % across) * 64;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = ty; i < 64; i += 8) {
+        const int r = r0 + i, c = c0 + 2 * tx;
+        t[i][tx] = (r < J.R && c < J.C) ? *reinterpret_cast<const uint32_t *>(J.in + (size_t)r * J.ldi + c) : 0u;
     }
     __syncthreads();
-    for (int i = ty; i < 32; i += 8) {
-        const int c = c0 + i, r = r0 + tx;
-        if (c < Cpad && r < ldo) out[(size_t)c * ldo + r] = t[tx][i];
+#pragma unroll
+    for (int i = ty; i < 64; i += 8) {
+        const int c = c0 + i, r = r0 + 2 * tx;
+        if (c < J.Cpad && r < J.ldo)
+            *reinterpret_cast<uint32_t *>(J.out + (size_t)c * J.ldo + r) =
+                __byte_perm(t[2 * tx][i >> 1], t[2 * tx + 1][i >> 1], i & 1 ? 0x7632 : 0x5410);
     }
 }
 
@@ -1067,11 +1078,23 @@ cudaError_t tc_gemm(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int
     return cudaErrorInvalidValue;
 }
 
-cudaError_t transpose_bf16(const __nv_bfloat16 *in, int R, int C, int ldi, __nv_bfloat16 *out,
-                           int ldo, int Cpad, cudaStream_t st) {
-    if (R <= 0 || Cpad <= 0) return cudaSuccess;
-    dim3 grid((std::max(R, ldo) + 31) / 32, (Cpad + 31) / 32);
-    transpose_bf16_kernel<<<grid, 256, 0, st>>>(in, R, C, ldi, out, ldo, Cpad);
+TransposeJob transpose_job(const __nv_bfloat16 *in, int R, int C, int ldi, __nv_bfloat16 *out, int ldo,
+                           int Cpad) {
+    return TransposeJob{in, out, R, C, ldi, ldo, Cpad,
+                        (uint32_t)((std::max(R, ldo) + 63) / 64) * (uint32_t)((Cpad + 63) / 64)};
+}
+
+cudaError_t transpose_bf16(const TransposeJob *jobs, int n, cudaStream_t st) {
+    TransposeJobs all{};
+    uint32_t tiles = 0;
+    if (n > kTransposeJobs) return cudaErrorInvalidValue;
+    for (int j = 0; j < n; ++j) {
+        if ((jobs[j].C | jobs[j].ldi | jobs[j].ldo) & 1) return cudaErrorInvalidValue;
+        all.job[j] = jobs[j];
+        tiles += jobs[j].tiles;
+    }
+    if (!tiles) return cudaSuccess;
+    transpose_bf16_kernel<<<tiles, 256, 0, st>>>(all);
     return cudaGetLastError();
 }
 
