@@ -158,6 +158,9 @@ constexpr uint32_t kUniformCaps[kUniformClasses] = {8192, 24576, 73728, 196608};
 // kUniformTaskNs of work.
 constexpr double kUniformMissNs = 30.0, kUniformHashMissNs = 50.0, kUniformWindowNs = 230.0;
 constexpr double kUniformTaskNs = 30.0e3;
+// What the launches of uniform chains cost a plan that needs the units as well,
+// and the warps that the units' work is taken to be shared by.
+constexpr double kUniformGainNs = 15.0e3, kUniformGainSlots = 152.0 * 8.0;
 // Small sets of this many misses (1 ms and more miss by miss) are played in
 // segments, where their lines are enough more than their ways for a play to
 // forget its start (uniform.cu): two survey-length plays of 0.2 ms instead.
@@ -1525,6 +1528,21 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
     for (uint64_t k = 0; k < n_units; ++k) p->items.push_back(items[order[k]]);
     // the pool's units after every size class, costliest first
     for (const SimItem &it : gitems) p->items.push_back(it);
+    if (tn.uniform && gitems.empty() && !(p->cross && p->n_geom >= kUniformGroupGeoms)) {
+        // Beside items that stay with the units, uniform chains pay by the time
+        // the units are spared: their launches cost kUniformGainNs (sweeps of 385
+        // array sizes of which a quarter are uniform: 67 us with them, 60 without).
+        double most[2] = {}, sum[2] = {};
+        for (uint64_t i = 0; i < n_units; ++i) {
+            const int u = (items[i].lsh >> kUniformBit) & 1u;
+            most[u] = std::max(most[u], cost[i]);
+            sum[u] += cost[i];
+        }
+        const double left = std::max(most[0], sum[0] / kUniformGainSlots);
+        const double whole = std::max(std::max(most[0], most[1]), (sum[0] + sum[1]) / kUniformGainSlots);
+        if (sum[0] > 0.0 && whole - left < kUniformGainNs)
+            for (SimItem &it : p->items) it.lsh &= ~((1u << kUniformBit) | (1u << kUniformMatchBit));
+    }
     try {
         if (tn.uniform) plan_uniform(p);
     } catch (...) {

@@ -23,10 +23,10 @@
 //
 // What bounds it: uniform_prep_kernel reads 4 B per access (HBM), the output
 // kernel writes a bit per access; the played sets are chains of dependent
-// events, so they are cut into one warp per set (or 32 small sets) and the
-// costliest start first.  Against stepping the same items in the units, the
-// 4096-item batch (0.64 G accesses, index arrays) went from 43.3 to 13.9 ms
-// (12.7 of them the longest played sets), a 384-item batch of short traces
+// events, so they are cut into one warp per set (or 32 small sets), long small
+// sets into segments, and the costliest start first.  Against stepping the same
+// items in the units, the 4096-item batch (0.64 G accesses, index arrays) went
+// from 43.3 to 9.4 ms (8 of them the longest played sets), a 384-item batch of short traces
 // from 519 to 155 us, matching 1308 candidates against 108 traces from 3.54 to
 // 0.18 ms.
 #include <algorithm>
@@ -738,7 +738,9 @@ __global__ void __launch_bounds__(32) uniform_segment_kernel(const SimItem *__re
 //
 // A window costs two shared-memory round trips and three to five votes; its
 // length, not its instructions, is what counts (one warp to a set), hence as
-// many heads a lane as the set's lines allow.
+// many heads a lane as the set's lines allow.  (Tables of each eviction's next
+// one of the same way, worked out in parallel beforehand, in place of the
+// hashing: the batch 10.0 -> 10.9 ms, their loads being on the window's chain.)
 //
 // arena: int32 leave[n], uint32 last[a] (1 + the last hashed eviction of a
 // way), int32 next[kAhead], uint16 occ[a], uint16 way[kAhead]
