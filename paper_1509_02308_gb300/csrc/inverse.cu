@@ -59,9 +59,15 @@ __global__ void gelu_back_kernel(const float *dy, const float *pre, size_t n, fl
 // softmax cross-entropy over the four heads; loss (mean over the batch and
 // heads) accumulated into *loss; dlogits = (softmax - onehot) / (4 batch).  A
 // thread per trace and head (a thread per trace left 4096 traces to 32 CTAs:
-// 16 us); a warp adds its losses before the one atomic.
+// 16 us); warps add their losses in FP64 to *sum, and the last block to arrive
+// adds that to *loss, so the loss is rounded once.
+constexpr size_t kLossOffset = 16;  // behind the status word
+struct LossSum {
+    double sum;
+    uint32_t blocks;
+};
 __global__ void xent_kernel(const float *logits, const uint32_t *labels, int nb, float *dlog,
-                            __nv_bfloat16 *dlogb, float *loss) {
+                            __nv_bfloat16 *dlogb, LossSum *sum, float *loss) {
     const int u = blockIdx.x * blockDim.x + threadIdx.x;
     const int b = u >> 2, h = u & 3;
     float l = 0.0f;
@@ -85,7 +91,13 @@ __global__ void xent_kernel(const float *logits, const uint32_t *labels, int nb,
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(kFull, l, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, l);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&sum->sum, (double)l);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&sum->blocks, 1u) + 1u == gridDim.x) {
+        __threadfence();
+        atomicAdd(loss, (float)atomicAdd(&sum->sum, 0.0));
+    }
 }
 
 // Adam (Kingma & Ba 2015) on FP32 master weights; refreshes BF16 copies
@@ -480,7 +492,7 @@ int pchase_inverse_create(uint32_t max_batch, pchase_inverse **out) {
     // inference's buffers first (a caller that only infers allocates that
     // prefix, pchase_inverse_infer_work_bytes), then the training step's
     o = 0;
-    h->status = o; o = a256(o + 4);
+    h->status = o; o = a256(o + kLossOffset + sizeof(LossSum));
     for (int l = 0; l < 4; ++l) {
         const size_t lout = h->L.lin[l] / 2;
         h->act[l] = o; o = a256(o + 2 * B * lout * kCh);
@@ -588,7 +600,7 @@ int pchase_inverse_train_step(const pchase_inverse *h, void *params, void *work,
     if (B == 0 || B > h->max_batch) return inv_fail(PCHASE_ERANGE, "batch above max_batch");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const InverseLayout &L = h->L;
-    INV_CUDA(cudaMemsetAsync(at<uint32_t>(work, h->status), 0, 4, st));
+    INV_CUDA(cudaMemsetAsync(at<uint32_t>(work, h->status), 0, kLossOffset + sizeof(LossSum), st));
     int rc = forward(h, params, work, B, st, true, x);
     if (rc) return rc;
     const size_t n = L.n_params;
@@ -598,7 +610,7 @@ int pchase_inverse_train_step(const pchase_inverse *h, void *params, void *work,
     float *dlog = at<float>(work, h->dlog);
     __nv_bfloat16 *dlogb = at<__nv_bfloat16>(work, h->dlogb);
     xent_kernel<<<(B + 31) / 32, 128, 0, st>>>(at<float>(work, h->logits), labels, (int)B, dlog,
-                                                 dlogb, loss_accum);
+                                                 dlogb, at<LossSum>(work, h->status + kLossOffset), loss_accum);
     // heads and FC on the tcgen05 tensor cores.  Products over the batch
     // (weight gradients) take both operands batch-contiguous: transposed
     // copies, rows padded with zeros to a multiple of 8 traces, K split over
