@@ -10,6 +10,7 @@ from __future__ import annotations
 import ctypes
 import os
 import threading
+from operator import index
 
 import numpy as np
 
@@ -184,8 +185,9 @@ def stream_handle(stream=None) -> int | None:
 
 # The descriptor arrays are filled through numpy views of the same layout, a
 # row per descriptor, not one ctypes structure after the other: 256 geometries,
-# traces and pairs take 0.3 ms instead of 1.1.  Values wrap to the field's
-# width, as a ctypes assignment does.
+# traces and pairs take 0.3 ms instead of 1.1.  Values are taken as a ctypes
+# assignment takes them: anything with __index__ (NumPy integers too), wrapped
+# to the field's width, and nothing else.
 _M32, _M64 = 0xFFFFFFFF, 0xFFFFFFFFFFFFFFFF
 _GEOM_ROW = np.dtype([("C_bytes", "<u4"), ("line_bytes", "<u4"), ("ways", "<u4"), ("sets", "<u4"),
                       ("policy", "<u4"), ("mapping", "<u4"), ("seed", "<u8")])
@@ -197,8 +199,9 @@ assert _GEOM_ROW.itemsize == ctypes.sizeof(Geom) and _TRACE_ROW.itemsize == ctyp
 def geom_array(geoms) -> ctypes.Array:
     arr = (Geom * max(1, len(geoms)))()
     if len(geoms):
-        rows = [(g.C & _M32, g.b & _M32, g.ways & _M32, g.sets & _M32, g.policy & _M32,
-                 (getattr(g, "mapping", 0) | (getattr(g, "extra", 0) << 8)) & _M32, g.seed & _M64)
+        rows = [(index(g.C) & _M32, index(g.b) & _M32, index(g.ways) & _M32, index(g.sets) & _M32,
+                 index(g.policy) & _M32,
+                 index(getattr(g, "mapping", 0) | (getattr(g, "extra", 0) << 8)) & _M32, index(g.seed & _M64))
                 for g in geoms]
         np.frombuffer(arr, dtype=_GEOM_ROW)[:] = rows
     return arr
@@ -215,8 +218,8 @@ def plan_units(h) -> list:
 
 def trace_array(descs) -> ctypes.Array:
     """descs: iterable of (idx_tensor_or_None, len, warmup, n_elems, stride)."""
-    rows = [(0 if t is None else t.data_ptr(), L & _M64, w & _M64, n & _M32, s & _M32)
-            for t, L, w, n, s in descs]
+    rows = [(0 if t is None else t.data_ptr(), index(L) & _M64, index(w) & _M64, index(n) & _M32,
+             index(s) & _M32) for t, L, w, n, s in descs]
     arr = (Trace * max(1, len(rows)))()
     if rows:
         np.frombuffer(arr, dtype=_TRACE_ROW)[:] = rows
@@ -224,11 +227,10 @@ def trace_array(descs) -> ctypes.Array:
 
 
 def pair_array(pairs) -> ctypes.Array:
-    pairs = list(pairs)
-    arr = (Pair * max(1, len(pairs)))()
-    if pairs:
-        np.frombuffer(arr, dtype="<u4").reshape(-1, 2)[:] = \
-            np.asarray(pairs, dtype=np.int64).reshape(-1, 2).astype(np.uint32)
+    rows = [(index(g) & _M32, index(t) & _M32) for g, t in pairs]
+    arr = (Pair * max(1, len(rows)))()
+    if rows:
+        np.frombuffer(arr, dtype="<u4").reshape(-1, 2)[:] = rows
     return arr
 
 
