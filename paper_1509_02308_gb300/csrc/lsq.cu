@@ -25,9 +25,13 @@
 //      sum, which takes over when Var_y is small against it (then FP32 sums
 //      cancel, the list overflows and every candidate is evaluated);
 //   3. the residuals of the candidates within the margin of the best estimate
-//      by the FP32 sums themselves, and the smallest of them.  Rows that are
-//      nearly constant (their variance below 1/64 of their mean square), whose
-//      FP32 variance cancels, are evaluated for every trace.
+//      by the FP32 sums themselves, and the smallest of them.
+// A row whose Var_r could lie below 1/64 of its square sum for some trace
+// (nearly constant rows, and rows that five points can take nearly all of) has
+// no estimate to rely on: differences cancel in it, and the FP32 sums may say
+// anything.  Such a row sets no trace's bound and is evaluated for every trace.
+// For the others the estimates stay within a fifth of half the margin of the
+// FP32 sums' residuals (emulated, Var_r from 1/2 to 1/60 of the square sum).
 // Evaluating every pair on the CUDA cores (three FP32 accumulators, 64 x 64
 // tiles) took 1388 us for 8192 traces x 1308 candidates, 80 % of it FP32 issue
 // and shared-memory loads; with the dropped points' sums as three more tensor
@@ -52,7 +56,7 @@ constexpr int kPoints = 512;
 constexpr int kKeep = kPoints - 5;
 constexpr uint32_t kLsqChunk = 2048;   // candidates converted at a time
 constexpr uint32_t kLsqList = 128;     // listed candidates of a trace
-constexpr uint32_t kLsqIll = 4096;     // nearly constant rows
+constexpr uint32_t kLsqIll = 4096;     // rows without estimates
 constexpr int kDrop = kPoints - kKeep; // points a trace drops, at most
 constexpr int kCols = 2 * kPoints;     // an operand row: high parts, low parts
 
@@ -73,8 +77,8 @@ struct __align__(16) Cand {
     float mean, s2;
 };
 struct Flags {
-    uint32_t all;    // 1: evaluate every candidate (a wait gave up, too many flat rows)
-    uint32_t n_ill;  // nearly constant rows
+    uint32_t all;    // 1: evaluate every candidate (a wait gave up, too many rows without estimates)
+    uint32_t n_ill;  // rows without estimates
     uint32_t n_every;  // traces that evaluate every candidate
 };
 
@@ -272,13 +276,16 @@ __global__ void __launch_bounds__(256) lsq_rates_kernel(const float *__restrict_
         // (their sum)^2 / 507, below a hundredth of their squares
         const float low = s2 * (1.0f - 1e-5f) - 1.02f * top;
         Cand c;
-        c.inv_low = low > 1e-3f * s2 && low > 1e-9f ? 1.0f / low : __int_as_float(0x7F800000);
-        c.inv_s2 = low > 1e-9f ? 1.0f / s2 : 0.0f;
+        // (also rows whose sums are not finite, and rows so small that Var_r
+        // may be on either side of the 1e-12 that makes it 0; a row of zeros
+        // has the trace's variance as its residual exactly)
+        const bool ill = !(64.0f * low >= raw) || (raw > 0.0f && !(low > 1e-9f));
+        c.inv_low = ill || raw == 0.0f ? 0.0f : 1.0f / low;
+        c.inv_s2 = ill || raw == 0.0f ? 0.0f : 1.0f / s2;
         c.mean = mean;
-        c.s2 = s2;
+        c.s2 = ill ? 0.0f : s2;  // (0: estimated at the trace's variance, above every residual)
         w.cand[k] = c;
-        // (also rows whose sums are not finite)
-        if (!(64.0f * s2 >= raw)) {
+        if (ill) {
             const uint32_t at = atomicAdd(&w.flags->n_ill, 1u);
             if (at < kLsqIll) w.ill[at] = g0 + k;
             else w.flags->all = 1u;
