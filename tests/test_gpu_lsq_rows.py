@@ -1,5 +1,5 @@
 """The least-squares judge (lsq.cu) against float64 where its estimates are at
-their weakest.  Bounds as in
+their weakest and where its CTAs take several tiles.  Bounds as in
 test_gpu_lsq.py: the error of FP32 sums of 512 terms, to first order, doubled."""
 import numpy as np
 import pytest
@@ -51,3 +51,14 @@ def test_judge_by_five_high_points_over_a_small_ramp(amp, base):
     best = _check(rates, y)
     if base == 0.0:  # (sums over rows far above their ramp decide nothing)
         assert (best == 2 * np.arange(60)).all()
+
+# candidates per tile (on 152 SMs): 96, 128, 160, 224 and 256 in one wave, then
+# two and three tiles to a CTA, with a second chunk of one candidate
+@pytest.mark.parametrize("n,G", [(1000, 1308), (1500, 1308), (2047, 1307), (3000, 1308), (5000, 700),
+                                 (2600, 1999), (4097, 1308), (4097, 2049), (8191, 1308)])
+def test_judge_over_many_tiles(n, G):
+    rng = np.random.Generator(np.random.PCG64(1000 * n + G))
+    rates = _rows(G, rng)
+    y = rates[rng.integers(0, G, n)] + 0.02 * rng.standard_normal((n, R.POINTS))
+    y[rng.random(y.shape) < 0.005] *= 4.0
+    _check(rates, y.astype(np.float32))
