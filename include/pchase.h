@@ -306,7 +306,9 @@ int pchase_sim_plan_upload(const pchase_sim_plan *plan, void *workspace, size_t 
  *   dev_status: uint32 status word (PCHASE_DEV_* bits); may be NULL.
  * Only kernel launches and a memset are queued (no host copies), so the call
  * can be captured into a CUDA graph; the work fans out over internal streams
- * that join back into `stream`.
+ * that join back into `stream`, or, while `stream` is being captured, over
+ * branches of the graph: a capture takes nothing from the plan, which may run
+ * on other streams and workspaces, or be captured again, before it ends.
  */
 int pchase_sim_run(const pchase_sim_plan *plan, void *workspace, uint32_t *bitmaps,
                    const uint64_t *word_offsets, uint64_t *miss_counts, uint32_t *dev_status,

@@ -612,6 +612,9 @@ struct pchase_sim_plan {
     double gwork_main[kUnitGroups] = {};  // estimated work of each unit group in the
                                           // slot-mix launch
     bool affinity = false;
+    // Streams beside the caller's, and the events that fork to and join from
+    // them.  Runs that are being captured use none of them (Beside below), so a
+    // capture never takes them from the plan's other runs.
     cudaStream_t side = nullptr, side2 = nullptr, uside = nullptr, uside2 = nullptr,
                  uside3 = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr, fork2 = nullptr, join2 = nullptr;
@@ -904,46 +907,144 @@ int plan_runtime(pchase_sim_plan *p) {
         if (per <= 0) return fail(PCHASE_ECUDA, "simulator kernel cannot be resident");
         p->jgrid = (int)std::max<uint64_t>(
             1, std::min<uint64_t>((uint64_t)per * (jsms ? jsms : p->sms), p->n_jumbo));
-        PCHASE_CUDA(cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking), "cudaStreamCreate");
-        PCHASE_CUDA(cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming), "cudaEventCreate");
-        PCHASE_CUDA(cudaEventCreateWithFlags(&p->join, cudaEventDisableTiming), "cudaEventCreate");
     }
-    if (p->gpool.nwarps) {
-        // the pool launch has exactly pool_warps warps: one state region each
-        p->ggrid = (int)(p->pool_warps / p->gpool.nwarps);
-        PCHASE_CUDA(cudaStreamCreateWithFlags(&p->side2, cudaStreamNonBlocking), "cudaStreamCreate");
-        PCHASE_CUDA(cudaEventCreateWithFlags(&p->fork2, cudaEventDisableTiming), "cudaEventCreate");
-        PCHASE_CUDA(cudaEventCreateWithFlags(&p->join2, cudaEventDisableTiming), "cudaEventCreate");
-    }
-    // played sets run beside the simulator's units, the large ones beside the
-    // small ones (where every item may be a uniform chain the units mostly have
-    // nothing to do, and one stream less is needed), and beside the matcher's
-    // other launches
-    const bool large = p->utasks.size() > p->uclass[0];
-    const bool beside = !p->uniform_every || !p->ugroups.empty();
-    const bool segments = !p->usegs.empty();
-    if ((!p->utasks.empty() && (large || beside)) || segments)
-        PCHASE_CUDA(cudaEventCreateWithFlags(&p->ufork, cudaEventDisableTiming), "cudaEventCreate");
-    if (p->uclass[0] && beside) {
-        PCHASE_CUDA(cudaStreamCreateWithFlags(&p->uside, cudaStreamNonBlocking), "cudaStreamCreate");
-        PCHASE_CUDA(cudaEventCreateWithFlags(&p->ujoin, cudaEventDisableTiming), "cudaEventCreate");
-    }
-    if (large) {
-        PCHASE_CUDA(cudaStreamCreateWithFlags(&p->uside2, cudaStreamNonBlocking), "cudaStreamCreate");
-        PCHASE_CUDA(cudaEventCreateWithFlags(&p->ujoin2, cudaEventDisableTiming), "cudaEventCreate");
-    }
-    if (segments) {
-        PCHASE_CUDA(cudaStreamCreateWithFlags(&p->uside3, cudaStreamNonBlocking), "cudaStreamCreate");
-        PCHASE_CUDA(cudaEventCreateWithFlags(&p->ujoin3, cudaEventDisableTiming), "cudaEventCreate");
-    }
+    // the pool launch has exactly pool_warps warps: one state region each
+    if (p->gpool.nwarps) p->ggrid = (int)(p->pool_warps / p->gpool.nwarps);
     p->device = dev;
     return PCHASE_OK;
 }
+
+// Where a plan's launches fan out beside the caller's stream.  Played sets run
+// beside the simulator's units, the large ones beside the small ones (where
+// every item may be a uniform chain the units mostly have nothing to do, and
+// one stream less is needed), and beside the matcher's other launches.
+struct Lanes {
+    bool jumbo, pool, small, large, segments;
+    explicit Lanes(const pchase_sim_plan &p)
+        : jumbo(p.jumbo.nwarps != 0),
+          pool(p.gpool.nwarps != 0),
+          small(p.uclass[0] && (!p.uniform_every || !p.ugroups.empty())),
+          large(p.utasks.size() > p.uclass[0]),
+          segments(!p.usegs.empty()) {}
+    bool any() const { return jumbo || pool || small || large || segments; }
+};
+
+// The plan's own streams and events, with its first run that is not captured.
+int plan_streams(pchase_sim_plan *p, const Lanes &lanes) {
+    const struct {
+        bool want;
+        cudaStream_t *stream;
+        cudaEvent_t *fork, *join;
+    } all[] = {{lanes.jumbo, &p->side, &p->fork, &p->join},
+               {lanes.pool, &p->side2, &p->fork2, &p->join2},
+               {lanes.small, &p->uside, &p->ufork, &p->ujoin},
+               {lanes.large, &p->uside2, &p->ufork, &p->ujoin2},
+               {lanes.segments, &p->uside3, &p->ufork, &p->ujoin3}};
+    for (const auto &l : all) {
+        if (!l.want) continue;
+        if (!*l.stream)
+            PCHASE_CUDA(cudaStreamCreateWithFlags(l.stream, cudaStreamNonBlocking), "cudaStreamCreate");
+        for (cudaEvent_t *e : {l.fork, l.join})
+            if (!*e) PCHASE_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming), "cudaEventCreate");
+    }
+    return PCHASE_OK;
+}
+
+// Launches beside those on `st`: on a stream of the plan's, forked from and
+// joined to `st` by events; or, while `st` is being captured, on `st` itself,
+// its capture dependencies set back to the fork's for them and again to the
+// launches' in between afterwards (the graph is the same).  Streams of the
+// plan's that had joined a capture would stay in it until it ends, and any other
+// run of the plan meanwhile, by another thread or into another graph, would
+// fail and spoil the capture.
+class Beside {
+public:
+    explicit Beside(cudaStream_t st) : st_(st) {}
+    cudaError_t init() {
+        cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+        if (st_) {
+            const cudaError_t e = cudaStreamIsCapturing(st_, &s);
+            if (e != cudaSuccess) return e;
+        }
+        capturing_ = s == cudaStreamCaptureStatusActive;
+        return cudaSuccess;
+    }
+    bool capturing() const { return capturing_; }
+
+    // what `st` depends on where lanes fork
+    struct Point {
+        std::vector<cudaGraphNode_t> nodes;
+        std::vector<cudaGraphEdgeData> edges;
+    };
+    cudaError_t fork(cudaEvent_t event, Point &at) {
+        return capturing_ ? get(at) : cudaEventRecord(event, st_);
+    }
+    // the stream to launch on until end()
+    cudaError_t begin(cudaStream_t side, cudaEvent_t event, Point &at, cudaStream_t *on) {
+        *on = capturing_ ? st_ : side;
+        if (!capturing_) return cudaStreamWaitEvent(side, event, 0);
+        const cudaError_t e = get(main_);
+        return e == cudaSuccess ? set(at, cudaStreamSetCaptureDependencies) : e;
+    }
+    cudaError_t end(cudaStream_t side, cudaEvent_t event) {
+        if (n_ == kLanes) return cudaErrorInvalidValue;
+        joins_[n_] = event;
+        Point &last = ends_[n_++];
+        if (!capturing_) return cudaEventRecord(event, side);
+        const cudaError_t e = get(last);
+        return e == cudaSuccess ? set(main_, cudaStreamSetCaptureDependencies) : e;
+    }
+    // what follows on `st` waits for every lane
+    cudaError_t join() {
+        cudaError_t e = cudaSuccess;
+        for (int k = 0; k < n_ && e == cudaSuccess; ++k)
+            e = capturing_ ? set(ends_[k], cudaStreamAddCaptureDependencies)
+                           : cudaStreamWaitEvent(st_, joins_[k], 0);
+        return e;
+    }
+
+private:
+    cudaError_t get(Point &at) {
+        cudaStreamCaptureStatus s;
+        const cudaGraphNode_t *nodes = nullptr;
+        const cudaGraphEdgeData *edges = nullptr;
+        size_t n = 0;
+        const cudaError_t e = cudaStreamGetCaptureInfo(st_, &s, nullptr, nullptr, &nodes, &edges, &n);
+        if (e != cudaSuccess) return e;
+        if (s != cudaStreamCaptureStatusActive) return cudaErrorStreamCaptureInvalidated;
+        try {
+            at.nodes.assign(nodes, nodes + n);
+            at.edges.assign(n, cudaGraphEdgeData{});
+        } catch (...) {
+            return cudaErrorMemoryAllocation;
+        }
+        if (edges) std::copy(edges, edges + n, at.edges.begin());
+        return cudaSuccess;
+    }
+    cudaError_t set(Point &at, unsigned flags) {
+        return cudaStreamUpdateCaptureDependencies(st_, at.nodes.data(), at.edges.data(), at.nodes.size(), flags);
+    }
+    cudaStream_t st_;
+    bool capturing_ = false;
+    Point main_;
+    static constexpr int kLanes = 5;
+    Point ends_[kLanes];
+    cudaEvent_t joins_[kLanes] = {};
+    int n_ = 0;
+};
 
 int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st) {
     const std::lock_guard<std::mutex> lock(p->launching);
     int rc = plan_runtime(p);
     if (rc) return rc;
+    const Lanes lanes(*p);
+    Beside beside(st);
+    if (lanes.any()) {
+        PCHASE_CUDA(beside.init(), "cudaStreamIsCapturing");
+        if (!beside.capturing() && (rc = plan_streams(p, lanes))) return rc;
+    }
+    Beside::Point at;
+    cudaStream_t on = st;
     uint8_t *w = static_cast<uint8_t *>(ws);
     SimOut o = out;
     // uniform chains, unless the run filters accesses, records a timeline of
@@ -967,7 +1068,8 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
         // the played sets add bits to the words, or (the matcher) only to the
         // distances, beside the launches that work these out: 188 -> 177 us a
         // match of 1308 candidates x 108 traces
-        if (p->ufork && o.dist) PCHASE_CUDA(cudaEventRecord(p->ufork, st), "cudaEventRecord");
+        const bool played = lanes.small || lanes.large || lanes.segments;
+        if (played && o.dist) PCHASE_CUDA(beside.fork(p->ufork, at), "fork");
         const bool grouped = o.dist && !p->ugroups.empty();
         if (grouped)
             PCHASE_CUDA(launch_uniform_match(items, reinterpret_cast<const UniformGroup *>(w + p->off_ugroups),
@@ -981,33 +1083,32 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
                                        live, st),
                     "uniform words");
         const UniformTask *const tasks = reinterpret_cast<const UniformTask *>(w + p->off_utasks);
-        if (p->ufork && !o.dist) PCHASE_CUDA(cudaEventRecord(p->ufork, st), "cudaEventRecord");
-        if (p->uside3) {
-            PCHASE_CUDA(cudaStreamWaitEvent(p->uside3, p->ufork, 0), "cudaStreamWaitEvent");
+        if (played && !o.dist) PCHASE_CUDA(beside.fork(p->ufork, at), "fork");
+        if (lanes.segments) {
+            PCHASE_CUDA(beside.begin(p->uside3, p->ufork, at, &on), "fork");
             PCHASE_CUDA(launch_uniform_segments(items, reinterpret_cast<const UniformSeg *>(w + p->off_usegs),
                                                 (uint32_t)p->usegs.size(),
                                                 reinterpret_cast<UniformSegState *>(w + p->off_segstates), o,
-                                                p->uside3),
+                                                on),
                         "uniform segments");
-            PCHASE_CUDA(cudaEventRecord(p->ujoin3, p->uside3), "cudaEventRecord");
+            PCHASE_CUDA(beside.end(p->uside3, p->ujoin3), "fork");
         }
-        if (p->uside2) {
-            PCHASE_CUDA(cudaStreamWaitEvent(p->uside2, p->ufork, 0), "cudaStreamWaitEvent");
+        if (lanes.large) {
+            PCHASE_CUDA(beside.begin(p->uside2, p->ufork, at, &on), "fork");
             uint32_t first = (uint32_t)p->utasks.size();
             for (int c = kUniformClasses - 1; c > 0; --c) {
                 first -= p->uclass[c];
-                PCHASE_CUDA(launch_uniform_play(items, tasks + first, p->uclass[c], kUniformCaps[c], o,
-                                                p->uside2),
+                PCHASE_CUDA(launch_uniform_play(items, tasks + first, p->uclass[c], kUniformCaps[c], o, on),
                             "uniform sets");
             }
-            PCHASE_CUDA(cudaEventRecord(p->ujoin2, p->uside2), "cudaEventRecord");
+            PCHASE_CUDA(beside.end(p->uside2, p->ujoin2), "fork");
         }
         if (p->uclass[0]) {
-            cudaStream_t us = p->uside ? p->uside : st;
-            if (p->uside) PCHASE_CUDA(cudaStreamWaitEvent(us, p->ufork, 0), "cudaStreamWaitEvent");
-            PCHASE_CUDA(launch_uniform_play(items, tasks, p->uclass[0], kUniformCaps[0], o, us),
+            on = st;
+            if (lanes.small) PCHASE_CUDA(beside.begin(p->uside, p->ufork, at, &on), "fork");
+            PCHASE_CUDA(launch_uniform_play(items, tasks, p->uclass[0], kUniformCaps[0], o, on),
                         "uniform sets");
-            if (p->uside) PCHASE_CUDA(cudaEventRecord(p->ujoin, us), "cudaEventRecord");
+            if (lanes.small) PCHASE_CUDA(beside.end(p->uside, p->ujoin), "fork");
         }
     } else {
         PCHASE_CUDA(launch_sim_zero(items, p->n_units, p->sms, o, st), "output clear");
@@ -1033,32 +1134,26 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
                                    o.uniform_bad, st),
                     "head streams");
     }
-    if (units && p->gpool.nwarps) {
+    if (units && lanes.pool) {
         // units with global set state first (the longest of a hierarchy's
-        // large levels), on a side stream of their own joined back below
-        PCHASE_CUDA(cudaEventRecord(p->fork2, st), "cudaEventRecord");
-        PCHASE_CUDA(cudaStreamWaitEvent(p->side2, p->fork2, 0), "cudaStreamWaitEvent");
-        PCHASE_CUDA(launch_sim(items, p->gpool, queues, p->ggrid, o, p->side2), "pool launch");
-        PCHASE_CUDA(cudaEventRecord(p->join2, p->side2), "cudaEventRecord");
+        // large levels), beside the others
+        PCHASE_CUDA(beside.fork(p->fork2, at), "fork");
+        PCHASE_CUDA(beside.begin(p->side2, p->fork2, at, &on), "fork");
+        PCHASE_CUDA(launch_sim(items, p->gpool, queues, p->ggrid, o, on), "pool launch");
+        PCHASE_CUDA(beside.end(p->side2, p->join2), "fork");
     }
-    // jumbo items first, on a side stream joined back before returning
-    const bool jside = units && p->jumbo.nwarps;
-    if (jside) {
-        PCHASE_CUDA(cudaEventRecord(p->fork, st), "cudaEventRecord");
-        PCHASE_CUDA(cudaStreamWaitEvent(p->side, p->fork, 0), "cudaStreamWaitEvent");
-        PCHASE_CUDA(launch_sim(items, p->jumbo, queues, p->jgrid, o, p->side), "jumbo launch");
-        PCHASE_CUDA(cudaEventRecord(p->join, p->side), "cudaEventRecord");
+    if (units && lanes.jumbo) {
+        // jumbo items first, beside the main launch
+        PCHASE_CUDA(beside.fork(p->fork, at), "fork");
+        PCHASE_CUDA(beside.begin(p->side, p->fork, at, &on), "fork");
+        PCHASE_CUDA(launch_sim(items, p->jumbo, queues, p->jgrid, o, on), "jumbo launch");
+        PCHASE_CUDA(beside.end(p->side, p->join), "fork");
     }
     if (units && p->layout.nwarps)
         PCHASE_CUDA(launch_sim(items, uni ? p->ulayout : p->layout, queues, uni ? p->ugrid : p->grid, o,
                                st),
                     "simulator launch");
-    if (jside) PCHASE_CUDA(cudaStreamWaitEvent(st, p->join, 0), "cudaStreamWaitEvent");
-    if (units && p->gpool.nwarps)
-        PCHASE_CUDA(cudaStreamWaitEvent(st, p->join2, 0), "cudaStreamWaitEvent");
-    if (uni && p->uside) PCHASE_CUDA(cudaStreamWaitEvent(st, p->ujoin, 0), "cudaStreamWaitEvent");
-    if (uni && p->uside2) PCHASE_CUDA(cudaStreamWaitEvent(st, p->ujoin2, 0), "cudaStreamWaitEvent");
-    if (uni && p->uside3) PCHASE_CUDA(cudaStreamWaitEvent(st, p->ujoin3, 0), "cudaStreamWaitEvent");
+    PCHASE_CUDA(beside.join(), "join");
     return PCHASE_OK;
 }
 
