@@ -161,10 +161,9 @@ constexpr double kUniformTaskNs = 30.0e3;
 // What the launches of uniform chains cost a plan that needs the units as well,
 // and the warps that the units' work is taken to be shared by.
 constexpr double kUniformGainNs = 15.0e3, kUniformGainSlots = 152.0 * 8.0;
-// Small sets of this many misses (1 ms and more miss by miss) are played in
+// Small sets of kUniformSegMisses (1 ms and more miss by miss) are played in
 // segments, where their lines are enough more than their ways for a play to
 // forget its start (uniform.cu): two survey-length plays of 0.2 ms instead.
-constexpr double kUniformSegMisses = 8.0 * kUniformRun;
 inline bool uniform_forgets(uint32_t n, uint32_t ways) {
     return (n >= ways + 2 || ways == 2) && 3ull * n >= 4ull * ways;
 }
@@ -1068,7 +1067,8 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
         // the played sets add bits to the words, or (the matcher) only to the
         // distances, beside the launches that work these out: 188 -> 177 us a
         // match of 1308 candidates x 108 traces
-        const bool played = lanes.small || lanes.large || lanes.segments;
+        // (segmented items are longer than those the matcher plays)
+        const bool segments = lanes.segments && !o.dist, played = lanes.small || lanes.large || segments;
         if (played && o.dist) PCHASE_CUDA(beside.fork(p->ufork, at), "fork");
         const bool grouped = o.dist && !p->ugroups.empty();
         if (grouped)
@@ -1084,7 +1084,7 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
                     "uniform words");
         const UniformTask *const tasks = reinterpret_cast<const UniformTask *>(w + p->off_utasks);
         if (played && !o.dist) PCHASE_CUDA(beside.fork(p->ufork, at), "fork");
-        if (lanes.segments) {
+        if (segments) {
             PCHASE_CUDA(beside.begin(p->uside3, p->ufork, at, &on), "fork");
             PCHASE_CUDA(launch_uniform_segments(items, reinterpret_cast<const UniformSeg *>(w + p->off_usegs),
                                                 (uint32_t)p->usegs.size(),

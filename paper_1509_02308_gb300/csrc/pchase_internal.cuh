@@ -252,6 +252,8 @@ struct UniformTask {
 // kUniformRun evictions long, surveyed from `warm` evictions earlier; their
 // states start at `state`.
 constexpr uint32_t kUniformRun = 4096;
+constexpr uint32_t kUniformSegMisses = 8 * kUniformRun;  // of a set that is cut
+static_assert(kUniformSegMisses >= kUniformMatchLen, "the matcher would have to play segments");
 struct UniformSeg {
     uint32_t unit, cls;
     uint32_t state, count, first;

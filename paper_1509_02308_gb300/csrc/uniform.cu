@@ -586,6 +586,8 @@ __device__ __forceinline__ void play_small(const SimItem &it, const Chain &ch, u
 // noted.  Where one did not, the segment before plays on to the end alone.
 // Segment i is evictions n - a + warm + i kUniformRun and on, the first one
 // from n - a (the first pass's) on.
+// (Not in the matcher: a set with enough misses for it is in an item of more
+// than kUniformMatchLen accesses, which the matcher's runs leave to the units.)
 constexpr int kSegG = 8;  // lanes of a segment: four segments a warp
 
 __device__ __forceinline__ bool same_state(const uint8_t *x, const uint8_t *y) {
@@ -603,7 +605,7 @@ __global__ void __launch_bounds__(32) uniform_survey_kernel(const SimItem *__res
     const uint32_t lane = threadIdx.x, r = lane % kSegG, glane = lane & ~(uint32_t)(kSegG - 1);
     const UniformSeg sg = segs[blockIdx.x];
     const SimItem it = items[sg.unit];
-    if (!taken(it, out.uniform_bad) || (out.dist && !((it.lsh >> kUniformMatchBit) & 1u))) return;
+    if (!taken(it, out.uniform_bad)) return;
     const Chain ch(it);
     const uint32_t i = sg.first + lane / kSegG;
     const uint32_t n = ch.lines_of(sg.cls), a = ch.a;
@@ -655,15 +657,15 @@ __global__ void __launch_bounds__(32) uniform_segment_kernel(const SimItem *__re
                                                              const UniformSeg *__restrict__ segs,
                                                              const UniformSegState *__restrict__ states,
                                                              SimOut out) {
-    uint8_t *arena = u_smem;
+    uint8_t *const arena = u_smem;
     const uint32_t lane = threadIdx.x, r = lane % kSegG, glane = lane & ~(uint32_t)(kSegG - 1);
     const UniformSeg sg = segs[blockIdx.x];
     const SimItem it = items[sg.unit];
-    if (!taken(it, out.uniform_bad) || (out.dist && !((it.lsh >> kUniformMatchBit) & 1u))) return;
+    if (!taken(it, out.uniform_bad)) return;
     Chain ch(it);
     ch.prepare_first();
     Sink sink;
-    arena = open_sink(sink, it, ch, out, blockIdx.y, arena, lane);
+    open_sink(sink, it, ch, out, 0, arena, lane);
     const uint32_t i = sg.first + lane / kSegG;
     const uint32_t n = ch.lines_of(sg.cls), a = ch.a;
     const uint32_t set = (uint32_t)(((uint64_t)sg.cls * ch.st) % ch.T);
@@ -718,7 +720,7 @@ __global__ void __launch_bounds__(32) uniform_segment_kernel(const SimItem *__re
         done = done || latest >= len || k >= last;
         small_sink<kSegG>(sink, count, t, r);
     }
-    sink.finish(it, out, blockIdx.y, lane);
+    sink.finish(it, out, 0, lane);
 }
 
 // Larger sets: one warp per set, a window of up to 32 H run heads at a time, H
@@ -972,11 +974,8 @@ cudaError_t launch_uniform_play(const SimItem *items, const UniformTask *tasks, 
 cudaError_t launch_uniform_segments(const SimItem *items, const UniformSeg *segs, uint32_t n_segs,
                                     UniformSegState *states, const SimOut &out, cudaStream_t st) {
     if (!n_segs) return cudaSuccess;
-    const bool ham = out.dist != nullptr;
-    const uint32_t bytes = kUniformSmallBytes + (ham ? kUniformMatchLen / 8 : 0u);
     uniform_survey_kernel<<<n_segs, 32, 0, st>>>(items, segs, states, out);
-    uniform_segment_kernel<<<dim3(n_segs, ham && out.n_rep ? out.n_rep : 1u), 32, bytes, st>>>(items, segs,
-                                                                                               states, out);
+    uniform_segment_kernel<<<n_segs, 32, kUniformSmallBytes, st>>>(items, segs, states, out);
     return cudaGetLastError();
 }
 

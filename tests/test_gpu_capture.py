@@ -154,3 +154,33 @@ def test_a_plan_runs_while_it_is_captured_twice(explicit, first_captured):
     finally:
         for g in graphs:
             g.close()
+
+
+@pytest.mark.parametrize("n_geom", [3, 16])
+def test_a_match_launches_no_segments(n_geom):
+    """Sets long enough for segments are in items that the matcher leaves to the
+    units: a match queues the check, the words (of groups too, from 16
+    candidates on), the played sets and the units, and nothing for segments."""
+    runs = [W.Run(48, 8, 100003, 6), W.Run(800, 8, 9001, 100)]
+    traces = [(None, r.length, r.warmup, r.n_elems, r.stride) for r in runs]
+    cands = [W.Geom(4 * 32 * (1 + k % 4), 32, 4 * (1 + k % 4), 1, (W.RANDOM, W.LRU, W.FIFO)[k % 3], 5 + k)
+             for k in range(n_geom)]
+    rng = np.random.Generator(np.random.PCG64(n_geom))
+    words = [(r.length + 31) // 32 for r in runs]
+    obs = torch.from_numpy(rng.integers(-2**31, 2**31, sum(words)).astype(np.int32)).cuda()
+    owo = torch.tensor([0, words[0]], dtype=torch.int64, device="cuda")
+    plan = api.SimPlan(cands, traces)
+    assert int(plan.description.split("uniform=")[1].split()[0].split(",")[2]) >= 1, plan.description
+    dist = torch.zeros(n_geom, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    g = _Graph(_runtime())
+    try:
+        C.check(plan.L.pchase_match_run(plan.h, plan._ws, C.ptr(obs), C.ptr(owo), 2**64 - 1, C.ptr(dist),
+                                        None, C.stream_handle(g.stream)))
+        g.end()
+        assert g.kernels() == 4 + (n_geom >= 16)
+        g.launch()
+    finally:
+        g.close()
+    want = api.SimPlan(cands, traces, tune={"head_streams": 2}).match(obs, owo)
+    assert torch.equal(dist, want) and torch.equal(plan.match(obs, owo), want)
