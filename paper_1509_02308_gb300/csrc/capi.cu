@@ -550,8 +550,14 @@ int pchase::set_last_error(int code, const char *msg) { return fail(code, msg); 
 struct pchase_sim_plan {
     std::vector<SimItem> items;
     SlotLayout layout{};
-    SlotLayout ulayout{};  // layout with the slot mix and homes of a run whose analytic
-                           // uniform chains are not the units' work
+    // the slot mix, homes and grid of runs whose uniform chains are not the
+    // units' work: of those that step no analytic one, and of the matcher's,
+    // which leaves the played ones above kUniformMatchLen to the units
+    struct LiveMix {
+        SlotLayout layout{};
+        double gwork[kUnitGroups] = {};
+        int grid = 0;
+    } live, matched;
     SlotLayout jumbo{};   // items too large for the main slot mix (nwarps 0: none)
     SlotLayout gpool{};   // units with global set state, one pool region per warp
     uint32_t pool_warps = 0;    // warps (and state regions) of the pool launch
@@ -574,7 +580,7 @@ struct pchase_sim_plan {
     double est_sum = 0.0, est_critical = 0.0, est_target = 0.0, est_max_unit = 0.0;
     bool filtered = false;  // every unit queued (pchase_sim_run_filtered)
     // runtime state, set on the first run
-    int device = -1, sms = 0, grid = 0, ugrid = 0, jgrid = 0, ggrid = 0;
+    int device = -1, sms = 0, grid = 0, jgrid = 0, ggrid = 0;
     uint64_t n_isolated = 0;  // units given an SM of their own (in the jumbo launch)
     uint64_t n_gmem = 0;        // units with their set state in global memory
     uint64_t gstate_bytes = 0;  // their state area (workspace, after the pooled offsets)
@@ -607,7 +613,6 @@ struct pchase_sim_plan {
     std::vector<uint32_t> ucands, urest;
     size_t off_bad = 0, off_utasks = 0, off_tunit = 0, off_ugroups = 0, off_ucands = 0, off_urest = 0,
            off_usegs = 0, off_segstates = 0;
-    double gwork_live[kUnitGroups] = {};  // (ulayout's)
     double gwork_main[kUnitGroups] = {};  // estimated work of each unit group in the
                                           // slot-mix launch
     bool affinity = false;
@@ -894,12 +899,14 @@ int plan_runtime(pchase_sim_plan *p) {
             1, std::min<uint64_t>((uint64_t)per * (p->sms - jsms), p->n_units - p->n_jumbo));
         const uint32_t sites = (uint32_t)std::max(1, std::min(p->grid, p->sms - jsms));
         set_homes(p->layout, p->gwork_main, p->affinity, sites);
-        const int uper = sim_max_ctas_per_sm(p->ulayout);
-        if (uper <= 0) return fail(PCHASE_ECUDA, "simulator kernel cannot be resident");
-        p->ugrid = (int)std::max<uint64_t>(
-            1, std::min<uint64_t>((uint64_t)uper * (p->sms - jsms), p->n_units - p->n_jumbo));
-        set_homes(p->ulayout, p->gwork_live, p->affinity,
-                  (uint32_t)std::max(1, std::min(p->ugrid, p->sms - jsms)));
+        for (pchase_sim_plan::LiveMix *m : {&p->live, &p->matched}) {
+            const int mper = sim_max_ctas_per_sm(m->layout);
+            if (mper <= 0) return fail(PCHASE_ECUDA, "simulator kernel cannot be resident");
+            m->grid = (int)std::max<uint64_t>(
+                1, std::min<uint64_t>((uint64_t)mper * (p->sms - jsms), p->n_units - p->n_jumbo));
+            set_homes(m->layout, m->gwork, p->affinity,
+                      (uint32_t)std::max(1, std::min(m->grid, p->sms - jsms)));
+        }
     }
     if (p->jumbo.nwarps) {
         const int per = sim_max_ctas_per_sm(p->jumbo);
@@ -1149,10 +1156,11 @@ int plan_launch(pchase_sim_plan *p, void *ws, const SimOut &out, cudaStream_t st
         PCHASE_CUDA(launch_sim(items, p->jumbo, queues, p->jgrid, o, on), "jumbo launch");
         PCHASE_CUDA(beside.end(p->side, p->join), "fork");
     }
-    if (units && p->layout.nwarps)
-        PCHASE_CUDA(launch_sim(items, uni ? p->ulayout : p->layout, queues, uni ? p->ugrid : p->grid, o,
-                               st),
+    if (units && p->layout.nwarps) {
+        const pchase_sim_plan::LiveMix &m = o.dist ? p->matched : p->live;
+        PCHASE_CUDA(launch_sim(items, uni ? m.layout : p->layout, queues, uni ? m.grid : p->grid, o, st),
                     "simulator launch");
+    }
     PCHASE_CUDA(beside.join(), "join");
     return PCHASE_OK;
 }
@@ -1274,8 +1282,9 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
     }
     uint64_t word = 0;
     double total = 0.0;
-    // done outside the units in most runs (an analytic uniform chain)
-    auto certain = [](const SimItem &it) { return !it.idx && ((it.lsh >> kUniformBit) & 1u); };
+    // done outside the units in most runs (an analytic uniform chain), or in
+    // the matcher's (bit kUniformMatchBit)
+    auto certain = [](const SimItem &it, uint32_t bit) { return !it.idx && ((it.lsh >> bit) & 1u); };
     const uint32_t max_split = std::max<uint32_t>(1, tn.max_split);
     for (uint64_t i = 0; i < n_items; ++i) {
         uint32_t g, t;
@@ -1713,9 +1722,11 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
     memset(&L, 0, sizeof L);
     std::vector<double> work(ncap, 0.0);
     // (live: what analytic uniform chains leave to the units)
-    std::vector<double> gwork[kUnitGroups], glive[kUnitGroups], wlive(ncap, 0.0);
+    std::vector<double> gwork[kUnitGroups], wlive(ncap, 0.0), wmatched(ncap, 0.0);
     for (auto &v : gwork) v.assign(ncap, 0.0);
+    std::vector<double> glive[kUnitGroups], gmatched[kUnitGroups];
     for (auto &v : glive) v.assign(ncap, 0.0);
+    for (auto &v : gmatched) v.assign(ncap, 0.0);
     uint32_t nclass = 0;
     {
         // classes present, in increasing cap order, renumbered 0..nclass-1
@@ -1742,9 +1753,13 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
                         ++count;
                         work[q] += cost[order[k]];
                         gwork[g][q] += cost[order[k]];
-                        if (!certain(items[order[k]])) {
+                        if (!certain(items[order[k]], kUniformBit)) {
                             glive[g][q] += cost[order[k]];
                             wlive[q] += cost[order[k]];
+                        }
+                        if (!certain(items[order[k]], kUniformMatchBit)) {
+                            gmatched[g][q] += cost[order[k]];
+                            wmatched[q] += cost[order[k]];
                         }
                     }
                 L.cls_first[g][q] = (uint32_t)(count ? first : 0);
@@ -1875,7 +1890,8 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
         for (int g = 0; g < kUnitGroups; ++g)
             for (int q = 0; q <= main_top; ++q) {
                 p->gwork_main[g] += gwork[g][q];
-                p->gwork_live[g] += glive[g][q];
+                p->live.gwork[g] += glive[g][q];
+                p->matched.gwork[g] += gmatched[g][q];
             }
         p->affinity = tn.kind_affinity != 0;
         // The same for runs whose analytic uniform chains are done elsewhere:
@@ -1883,12 +1899,14 @@ int pchase_sim_plan_create(const pchase_geom *geoms, uint32_t n_geom, const pcha
         // 448 chains beside 64 index arrays whose line tables need 70-110 KB
         // each; 3.6 warps active per SM, 14.1 ms a table of 64 candidates; 10.5 ms
         // with this and the slots above).
-        p->ulayout = L;
-        {
-            double live = 0.0;
-            for (int q = 0; q <= main_top; ++q) live += wlive[q];
-            if (live > 0.0) slot_mix(p->ulayout, wlive, main_top);
-        }
+        auto mix_for = [&](pchase_sim_plan::LiveMix &m, const std::vector<double> &w) {
+            m.layout = L;
+            double sum = 0.0;
+            for (int q = 0; q <= main_top; ++q) sum += w[q];
+            if (sum > 0.0) slot_mix(m.layout, w, main_top);
+        };
+        mix_for(p->live, wlive);
+        mix_for(p->matched, wmatched);
         // jumbo layout: one warp, the largest jumbo arena; serves jumbo classes
         SlotLayout &J = p->jumbo;
         memset(&J, 0, sizeof J);
@@ -2122,13 +2140,16 @@ size_t pchase_sim_plan_describe(const pchase_sim_plan *plan, char *buf, size_t b
             snprintf(tmp, sizeof tmp, " uniform=%llu,%zu,%zu", (unsigned long long)plan->n_uniform,
                      plan->utasks.size(), plan->usegs.size());
             d += tmp;
-            d += " live_slots=";
-            for (uint32_t w = 0; w < plan->ulayout.nwarps; ++w) {
-                const uint32_t next = w + 1 < plan->ulayout.nwarps ? plan->ulayout.warp_off[w + 1]
-                                                                   : plan->ulayout.smem_bytes;
-                snprintf(tmp, sizeof tmp, "%s%u", w ? "," : "", next - plan->ulayout.warp_off[w]);
-                d += tmp;
-            }
+            auto slots = [&](const char *name, const SlotLayout &L) {
+                d += name;
+                for (uint32_t w = 0; w < L.nwarps; ++w) {
+                    const uint32_t next = w + 1 < L.nwarps ? L.warp_off[w + 1] : L.smem_bytes;
+                    snprintf(tmp, sizeof tmp, "%s%u", w ? "," : "", next - L.warp_off[w]);
+                    d += tmp;
+                }
+            };
+            slots(" live_slots=", plan->live.layout);
+            if (plan->cross) slots(" match_slots=", plan->matched.layout);
         }
         if (!plan->jobs.empty()) {
             // head streams: split items, their parts, entries (8 bytes each);
