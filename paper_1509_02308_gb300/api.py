@@ -22,6 +22,17 @@ def _on_current(stream) -> bool:
     return stream is None or stream.cuda_stream == torch.cuda.current_stream().cuda_stream
 
 
+def _lend(stream, *temporaries):
+    """Temporaries of a call that goes to another stream than the current one,
+    whose memory they are of: dropped when the call returns, they are given out
+    again only after that stream has done with them."""
+    if not _on_current(stream):
+        if not isinstance(stream, torch.cuda.Stream):  # (anything with a handle)
+            stream = torch.cuda.ExternalStream(stream.cuda_stream)
+        for t in temporaries:
+            t.record_stream(stream)
+
+
 def status_word(device=DEV) -> torch.Tensor:
     return torch.zeros(1, dtype=torch.int32, device=device)
 
@@ -36,6 +47,7 @@ def pchase_build(n_elems: int, stride: int, length: int, next_chain: torch.Tenso
     arr = _u32(n_elems) if with_array else None
     if next_chain is not None and status is None:
         status = status_word()
+        _lend(stream, status)
     C.check(L.pchase_build(n_elems, stride, C.ptr(next_chain), length, C.ptr(trace), C.ptr(arr),
                            C.ptr(status), C.stream_handle(stream)))
     return (trace, arr) if with_array else trace
@@ -161,6 +173,7 @@ class SimPlan:
         scratch_b = int(self.L.pchase_infer_scratch_bytes(self.h))
         if getattr(self, "_scratch", None) is None or self._scratch.numel() < scratch_b + 256:
             self._scratch = torch.empty(scratch_b + 256, dtype=torch.uint8, device=DEV)
+        _lend(stream, self._scratch)
         sp = (C.ptr(self._scratch) + 255) & ~255
         dist = torch.empty(max(1, len(self.geoms)), dtype=torch.int64, device=DEV)
         pick = torch.empty(2, dtype=torch.int32, device=DEV)
@@ -180,6 +193,7 @@ def infer_batch(plan: "SimPlan", lats: torch.Tensor, stop_above: int = 2**64 - 1
     sp = (C.ptr(scratch) + 255) & ~255
     dist = torch.empty(n_obs, max(1, len(plan.geoms)), dtype=torch.int64, device=DEV)
     pick = torch.empty(n_obs, 2, dtype=torch.int32, device=DEV)
+    _lend(stream, scratch)
     C.check(L.infer_geometry_batch(plan.h, plan._ws, C.ptr(lats), n_obs, sp, stop_above,
                                    C.ptr(dist), C.ptr(pick), C.ptr(status),
                                    C.stream_handle(stream)))
@@ -261,7 +275,8 @@ def pchase_classify(lats: list[torch.Tensor], stream=None):
                        for x in lats]) if lats else torch.zeros(1, device=DEV))
     max_len = max(n) if n else 0
     # both offset arrays in one copy, which waits for the device only when the
-    # call goes to another stream than the one that makes its inputs
+    # call goes to another stream than the one that makes its inputs (a copy out
+    # of pageable memory has read it when it returns: the arrays may go)
     d_both = torch.from_numpy(np.concatenate([offs, w])).to(DEV, non_blocking=_on_current(stream))
     d_offs, d_w = d_both[:len(offs)], d_both[len(offs):]
     nwords = int(sum((x + 31) // 32 for x in n))
@@ -270,6 +285,7 @@ def pchase_classify(lats: list[torch.Tensor], stream=None):
     ws = torch.empty(int(L.pchase_classify_workspace_bytes(len(lats), max_len)) + 256,
                      dtype=torch.uint8, device=DEV)
     wp = (C.ptr(ws) + 255) & ~255
+    _lend(stream, flat, d_both, ws)
     C.check(L.pchase_classify(C.ptr(flat), C.ptr(d_offs), len(lats), max_len, C.ptr(bits),
                               C.ptr(d_w), C.ptr(thr), wp, C.stream_handle(stream)))
     return bits, w, thr
@@ -280,6 +296,7 @@ def pchase_canonical_pick(geoms: list[Geom], dist: torch.Tensor, stream=None):
     ga = C.geom_array(geoms)
     dg = torch.frombuffer(bytearray(ga), dtype=torch.uint8).to(DEV)
     pick = torch.empty(2, dtype=torch.int32, device=DEV)
+    _lend(stream, dg)
     C.check(L.pchase_canonical_pick(C.ptr(dg), C.ptr(dist), len(geoms), C.ptr(pick),
                                     C.stream_handle(stream)))
     return pick
