@@ -238,11 +238,14 @@ size_t pchase_sim_plan_upload_bytes(const pchase_sim_plan *plan);
 /* Number of items, and of bitmap words when the plan lays bitmaps out itself. */
 uint64_t pchase_sim_plan_items(const pchase_sim_plan *plan);
 uint64_t pchase_sim_plan_bitmap_words(const pchase_sim_plan *plan);
-/* Kernel launches one pchase_sim_run queues (the output clear; when the plan
- * splits items by sets, the three launches of their head streams; the
- * slot-mix launch; and the side launches of jumbo and pool units, when it has
- * them); pchase_match_run queues neither the output clear nor the head
- * streams. */
+/* Kernel launches one pchase_sim_run queues: the output clear, or, in a plan
+ * with uniform chains, their check, their words, a launch per shared-memory
+ * class of played sets and two for segments; when the plan splits items by
+ * sets, the three launches of their head streams; the slot-mix launch; and the
+ * side launches of jumbo and pool units, when it has them (a plan of analytic
+ * uniform chains alone launches nothing for units).  pchase_match_run queues
+ * neither the output clear nor segments nor head streams, and one launch more
+ * where it matches candidates in groups (16 candidates and more). */
 uint32_t pchase_sim_plan_launches(const pchase_sim_plan *plan);
 /*
  * Writes a one-line text description of the plan (items split by sets and

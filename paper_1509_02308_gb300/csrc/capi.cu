@@ -127,12 +127,12 @@ constexpr double kAffinityMinNsPerSm = 20.0e6;
 // launch): the costliest kIsolateMax within kIsolateFrac of the costliest.
 constexpr double kIsolateFrac = 0.6;
 constexpr size_t kIsolateMax = 12;
-// A matcher's groups are one launch more (2 us): worth it from a few candidates
-// to a group on (1308 candidates x 108 traces: 312 -> 188 us a match).
-constexpr uint32_t kUniformGroupGeoms = 16;
 // ... in plans whose longest unit takes this long: a second launch beside the
 // main one, forked and joined, costs the host and the GPU some 6 us.
 constexpr double kIsolateMinNs = 1.0e5;
+// A matcher's groups are one launch more (2 us): worth it from a few candidates
+// to a group on (1308 candidates x 108 traces: 312 -> 188 us a match).
+constexpr uint32_t kUniformGroupGeoms = 16;
 // Way scans over set state in global memory (L2-resident) against shared memory.
 constexpr double kGlobalScanFactor = 2.0;
 // A time part's backward read of 32 accesses while it rebuilds the recency

@@ -100,8 +100,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
     float *const xs = reinterpret_cast<float *>(gbase + (sOut - base) + 2 * kOutTile);
     float *const sBias2 = xs + 2 * kFusedXs;
     const uint32_t sBar = sOut + 2 * kOutTile + 2 * 4 * kFusedXs + 4 * kCh;
-    // barriers: slab_full[4] at sBar + 8b, slab_empty[4] at sEmpty + 8b,
-    // acc_full[2] at sAcc + 8a, acc_empty[2] at sFree + 8a; then the TMEM
+    // barriers: slab_full[kFusedSlabs] at sBar + 8b, slab_empty[kFusedSlabs] at
+    // sEmpty + 8b, acc_full[2] at sAcc + 8a, acc_empty[2] at sFree + 8a; then the TMEM
     // address and the abort flag
     const uint32_t sEmpty = sBar + 8u * kFusedSlabs, sAcc = sEmpty + 8u * kFusedSlabs, sFree = sAcc + 16u;
     uint32_t *const tslot = reinterpret_cast<uint32_t *>(gbase + (sFree - base) + 16);

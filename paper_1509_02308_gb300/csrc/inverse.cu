@@ -59,8 +59,8 @@ __global__ void gelu_back_kernel(const float *dy, const float *pre, size_t n, fl
 // softmax cross-entropy over the four heads; loss (mean over the batch and
 // heads) accumulated into *loss; dlogits = (softmax - onehot) / (4 batch).  A
 // thread per trace and head (a thread per trace left 4096 traces to 32 CTAs:
-// 16 us); warps add their losses in FP64 to *sum, and the last block to arrive
-// adds that to *loss, so the loss is rounded once.
+// 16 us).  A term and a warp's sum of 32 are FP32; the warps' sums are added in
+// FP64 to *sum, and the last block to arrive adds that to *loss.
 constexpr size_t kLossOffset = 16;  // behind the status word
 struct LossSum {
     double sum;

@@ -732,7 +732,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
 // of the K blocks (gridDim.z slices of 64-element blocks).  One thread runs
 // the main loop: both operands' 64-column blocks are TMA tile loads (2-D
 // tensor maps, 128-byte swizzle; rows past M or N and columns past K are out
-// of the tensor and read as zeros) into a 4-stage ring, three blocks ahead;
+// of the tensor and read as zeros) into a ring of kGemmStages, two blocks ahead;
 // a stage's mbarrier counts its bytes in, and a second one (tcgen05.commit)
 // frees it once its MMAs are done.  Epilogues: kStore (C[m][n], or C[n][m] when transposed,
 // + bias[n] if given; FP32 atomics when K is sliced) and kGelu (v = sum +
