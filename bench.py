@@ -110,7 +110,8 @@ def max_over_ranks(value: float, world: int, device=None) -> float:
 
 # ----------------------------------------------------------------- clocks
 class ClockSampler:
-    """nvidia-smi clocks and throttle reasons, sampled every 200 ms."""
+    """nvidia-smi clocks and throttle reasons, sampled every 20 ms (the timed
+    steps of a default run take some 60 ms)."""
 
     FIELDS = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.active,"
               "clocks_event_reasons.hw_slowdown,clocks_event_reasons.hw_thermal_slowdown,"
@@ -128,10 +129,14 @@ class ClockSampler:
             self.f = open(self.path, "w")
             self.proc = subprocess.Popen(
                 ["nvidia-smi", f"--id={self.gpu}", f"--query-gpu={self.FIELDS}",
-                 "--format=csv,noheader,nounits", "-lms", "200"],
+                 "--format=csv,noheader,nounits", "-lms", "20"],
                 stdout=self.f, stderr=subprocess.DEVNULL)
         except Exception:
             self.proc = None
+
+    def sampling(self) -> bool:
+        """Whether samples have begun to come (nvidia-smi takes a while to start)."""
+        return self.proc is None or os.path.getsize(self.path) > 0
 
     def stop(self) -> dict:
         if self.proc is None:
@@ -380,15 +385,17 @@ def ours(args):
             import torch.distributed as dist
             dist.barrier()
 
+    vis = [x for x in os.environ.get("CUDA_VISIBLE_DEVICES", "").split(",") if x.strip().isdigit()]
+    clocks = ClockSampler(int(vis[local]) if local < len(vis) else local)
+    clocks.start()
+    t0 = time.perf_counter()
+    while not clocks.sampling() and time.perf_counter() - t0 < 5.0:
+        time.sleep(0.01)
     for _ in range(args.warmup):
         graph.replay()
     torch.cuda.synchronize()
-
-    vis = [x for x in os.environ.get("CUDA_VISIBLE_DEVICES", "").split(",") if x.strip().isdigit()]
-    clocks = ClockSampler(int(vis[local]) if local < len(vis) else local)
     barrier()
     torch.cuda.synchronize()
-    clocks.start()
     cur = torch.cuda.current_stream()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     e0.record(cur)

@@ -3,6 +3,7 @@ enough to be found whole at the end of a cut-off output."""
 import importlib.util
 import json
 import os
+import time
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 spec = importlib.util.spec_from_file_location("bench", os.path.join(ROOT, "bench.py"))
@@ -62,3 +63,25 @@ def test_sections_that_failed_or_were_skipped():
     d = json.loads(bench.contract_line(full))
     assert d["hierarchy"]["error"].startswith("RuntimeError(") and len(d["hierarchy"]["error"]) == 80
     assert "e2e" not in d and "mixed" not in d and d["learned_inverse"] == {"error": "q"}
+
+
+def test_clock_samples_have_begun_before_the_steps(tmp_path, monkeypatch):
+    """nvidia-smi takes longer to start than the timed steps take: the sampler
+    says when its samples have begun to come."""
+    fake = tmp_path / "nvidia-smi"
+    fake.write_text("#!/bin/sh\nsleep 0.3\nwhile true; do\n"
+                    "echo '0, 2000, 2070, 900.0, 0x4, Not Active, Not Active, Not Active, Active'\n"
+                    "sleep 0.01\ndone\n")
+    fake.chmod(0o755)
+    monkeypatch.setenv("PATH", f"{tmp_path}:{os.environ['PATH']}")
+    clocks = bench.ClockSampler(0)
+    clocks.start()
+    assert not clocks.sampling()
+    t0 = time.perf_counter()
+    while not clocks.sampling():
+        assert time.perf_counter() - t0 < 10.0
+        time.sleep(0.01)
+    time.sleep(0.1)
+    got = clocks.stop()
+    assert got["sm_mhz"] == 2000.0 and got["sm_max_mhz"] == 2070.0 and got["reasons"] == ["sw_power_cap"]
+    assert got["samples"] >= 2
