@@ -25,9 +25,9 @@
 // kernel writes a bit per access; the played sets are chains of dependent
 // events, so they are cut into one warp per set (or 32 small sets), long small
 // sets into segments, and the costliest start first.  Against stepping the same
-// items in the units, the 4096-item batch (0.64 G accesses, index arrays) went
-// from 43.3 to 9.4 ms (8 of them the longest played sets), a 384-item batch of short traces
-// from 519 to 155 us, matching 1308 candidates against 108 traces from 3.54 to
+// items in the units, batches of 4096 items (0.63 G accesses, index arrays) went
+// from 44 to 9-15 ms and the benchmark's from 21.8 to 4.4 (their longest played
+// sets all but 1.1 ms of it), a 384-item batch of short traces from 519 to 155 us, matching 1308 candidates against 108 traces from 3.54 to
 // 0.18 ms.
 #include <algorithm>
 
